@@ -104,7 +104,7 @@ typedef struct {
                                rounding level of the normal equations, in the
                                precision form; none in FP64); < 0 disables  */
     int32_t gram_impl;      /* per-slice normal equations of the middle
-                               levels.  0 = automatic: for r = 4 or 8, a
+                               levels.  0 = automatic: for r >= 2, a
                                level whose row (or column) groups are few
                                against its entries (below group_ratio of
                                them) runs the grouped Gram (the entries of one row
@@ -123,10 +123,10 @@ typedef struct {
     int32_t lr2bf_oversample; /* oversampling p of Alg. 2 for init_kind 2
                                (0 selects 5); r + p <= 32                   */
     double group_ratio;     /* gram_impl 0: groups-per-entry threshold of the
-                               grouped Gram.  0 selects the default (0.1
-                               next to the tensor-core kernel, 0.9 next to
-                               the CUDA-core one); < 0 never groups; > 0
-                               is used as given                             */
+                               grouped Gram.  0 selects the default (next to
+                               the tensor-core kernel 0.1 (8 / r)^4, at most
+                               0.9; 0.9 next to the CUDA-core one); < 0 never
+                               groups; > 0 is used as given                             */
 } bfc_params;
 
 typedef struct {

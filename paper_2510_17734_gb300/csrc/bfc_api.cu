@@ -275,7 +275,7 @@ static bfc_status build(Ctx* c, const Inputs& in)
             gl.by_col = by_col;
             gl.ngroups = G;
             const double ratio = c->gram_tc ? c->grp_max_ratio : c->grp_cuda_ratio;
-            if ((c->r == 4 || c->r == 8) && c->P.gram_impl == 0 && (double)G < ratio * (double)N) {
+            if (c->r >= 2 && c->P.gram_impl == 0 && (double)G < ratio * (double)N) {
                 gst.push_back((int32_t)N);
                 // the largest entry range of a k_group_sums block (its shared-memory staging)
                 const int64_t gpb = 128 / c->r;
@@ -352,16 +352,12 @@ static bfc_status build(Ctx* c, const Inputs& in)
     }
     const Ops* ops = get_ops(c->fp32, r);
     BFC_TRY(dalloc(c, &c->rec, ops->record_bytes(n, S), "normal-equation records"));
-    // group records [s | M | v] of the grouped Gram (ranks 4 and 8): sized for
-    // the largest level whose order was grouped
-    if ((r == 4 || r == 8) && c->P.gram_impl == 0) {
-        int64_t gmax = 0;
-        for (const GroupLevel& gl : c->grp)
-            if (gl.gstart) gmax = std::max(gmax, gl.ngroups);
-        // record [s | M (with 64 bytes between its two row halves) | v]
-        const size_t rec_vals = (size_t)(2 * r + r * r) + 64 / c->vsz;
-        if (gmax > 0) BFC_TRY(dalloc(c, &c->grec, (size_t)gmax * rec_vals * c->vsz, "group records"));
-    }
+    // group records [s | M | v] of the grouped Gram: sized for the largest
+    // level whose order was grouped
+    int64_t gmax = 0;
+    for (const GroupLevel& gl : c->grp)
+        if (gl.gstart) gmax = std::max(gmax, gl.ngroups);
+    if (gmax > 0) BFC_TRY(dalloc(c, &c->grec, (size_t)gmax * ops->group_record_bytes(), "group records"));
     const size_t fbb = ops->fallback_bytes(S);
     if (fbb > 0 && L > 0) {
         BFC_TRY(dalloc(c, (void**)&c->fb, fbb, "FP64 fallback records"));
@@ -407,12 +403,16 @@ static bfc_status create_impl(const bfc_params* params, const Inputs& in, bfc_ct
     c->ridge = p.ridge_rel > 0.0 ? p.ridge_rel : (p.ridge_rel == 0.0 && c->fp32 ? 9.5367431640625e-07 : 0.0);
     c->gram_tc = c->fp32 && p.gram_impl != 1 && p.r <= 8;
     // grouped Gram (gram_impl 0) at the middle levels with few row / column
-    // groups per entry: below this ratio against the tensor-core kernel (a
-    // group's compensated Kronecker update and its sums cost about what seven
-    // entries cost there: at n = 65536 a level of 0.07 groups per entry is
-    // faster grouped, one of 0.14 on the tensor cores), below 0.9 against the
-    // per-entry CUDA-core kernel
-    c->grp_max_ratio = p.group_ratio > 0.0 ? p.group_ratio : (p.group_ratio < 0.0 ? 0.0 : 0.1);
+    // groups per entry.  Against the per-entry CUDA-core kernel, whose work per
+    // entry is that of a group, below 0.9.  Against the tensor-core kernel,
+    // which costs the same per entry at every rank (it pads to rank 8), the
+    // line moves with the r^4 of a group's Kronecker update: 0.1 at rank 8 (at
+    // n = 65536 a level of 0.07 groups per entry is faster grouped, one of 0.14
+    // on the tensor cores), times (8 / r)^4, at most 0.9
+    double tc_ratio = 0.1;
+    for (int q = 0; q < 4; ++q) tc_ratio *= 8.0 / p.r;
+    tc_ratio = std::min(std::max(tc_ratio, 0.1), 0.9);
+    c->grp_max_ratio = p.group_ratio > 0.0 ? p.group_ratio : (p.group_ratio < 0.0 ? 0.0 : tc_ratio);
     c->grp_cuda_ratio = p.group_ratio > 0.0 ? p.group_ratio : (p.group_ratio < 0.0 ? 0.0 : 0.9);
     bfc_status st = build(c, in);
     if (st != BFC_OK) {
@@ -757,7 +757,7 @@ static bfc_status lbfgs_impl(Ctx* c, int iters, int m, bfc_sweep_stats* history,
 
 bool level_grouped(const Ctx* c, int m)
 {
-    if (c->P.gram_impl != 0 || (c->r != 4 && c->r != 8) || !c->grec) return false;
+    if (c->P.gram_impl != 0 || !c->grec) return false;
     if (m < 1 || m > c->L || (int)c->grp.size() <= m) return false;
     const GroupLevel& gl = c->grp[m];
     if (!gl.gstart) return false;   // level order not grouped at build time

@@ -1,5 +1,5 @@
 // Per-slice normal equations of one middle level, by groups of entries that
-// share an environment (CUDA cores, rank R = 4 or 8).
+// share an environment (CUDA cores, rank R >= 2).
 //
 // Inside a slice k of S^{m+1}, the left environment h_m of an entry depends
 // only on its row i (the column bits it passed, j_0 .. j_{m-2}, are fixed by
@@ -20,14 +20,20 @@
 // a slice's records through shared memory and accumulates the Kronecker
 // updates.  Layout: the level order keeps each group contiguous; gseg[k] is
 // the first group of slice k, gstart[g] the first position of group g.  Work
-// per slice as in k_mid_gram: 4 x 4 complex tiles of the lower triangle of K
-// owned by threads (tile I, J: rows a = 4I / R, c = 4I mod R + u; columns
-// likewise).  Precision form: a group's term can be a large part of the
+// per slice as in k_mid_gram: T x T complex tiles of the lower triangle of K
+// owned by threads, each inside one (a, a') block (GrpTile).  Precision form: a group's term can be a large part of the
 // slice's sum (16 row groups at the first level), so every term is added
 // with Kahan compensation, and the group sums are compensated across blocks
 // of 16 entries; the error of K then matches the per-entry kernels' (the
 // rounding of the stored complex64 record dominates both).  Same output
 // record as k_mid_gram.
+//
+// Measured, all middle levels of a sweep, against the per-entry kernels that
+// these levels ran before: n = 4096, L = 8, r = 12, 3.41 M entries, complex64
+// 107.2 -> 3.6 ms (against k_mid_gram); n = 4096, L = 8, r = 6, 265 k entries,
+// FP64 19.1 -> 3.3 ms (k_mid_gram, bound by the FP64 pipe at 1.25 TFLOP/s);
+// n = 3072, L = 8, r = 5, 961 k entries, complex64 1.42 -> 0.87 ms (against
+// k_mid_gram_tc).
 #pragma once
 
 #include "bfc_kernels.cuh"
@@ -57,16 +63,34 @@ __device__ __forceinline__ void cp_async8(void* smem_dst, const void* gmem_src)
     asm volatile("cp.async.ca.shared.global [%0], [%1], 8;" ::"r"(sa), "l"(gmem_src) : "memory");
 }
 
-// Group record [s | M | v] of rank R in values of type V: s at 0, M[c][c']
-// at R + grp_m(c, c'), v at VOFF.  The rows c >= R/2 of M sit 64 bytes
-// further on, so the 4 x 4 blocks of M the Gram tiles read at once (rows
-// 0..3 and 4..7, column blocks 0 and 4) fall into distinct shared-memory
-// banks.
+// Tile side of the grouped Gram's K tiles and the padded column count RP (a
+// multiple of it): a tile then lies inside one (a, a') block of K, so it needs
+// one value of the shared side and T x T of the other.  T = 4 where it divides
+// R, else 3, 5 or 2; the primes 7 and 11 use T = 4 with one padded column
+// (7 x 8 of 7 x 7, 11 x 12 of 11 x 11).
+template <int R> struct GrpTile {
+    static constexpr int T = R % 4 == 0 ? 4 : R % 3 == 0 ? 3 : R % 5 == 0 ? 5 : R == 2 ? 2 : 4;
+    static constexpr int RP = (R + T - 1) / T * T;
+};
+
+// Group record [s | M | v] of rank R in values of type V, s and v padded to RP
+// values, M to RP rows of RP values (padding is zero): s at 0, M[c][c'] at
+// m(c, c'), v at VOFF.  The T x T blocks of M that the Gram tiles read at once
+// should fall into distinct shared-memory banks: at R = 4 and 8 the rows
+// c >= RP / 2 of M sit 64 bytes further on; at R = 7, 11 and 12 every block of
+// four rows sits 16 bytes further than the last (its natural distance is a
+// multiple of 128 bytes).
 template <typename V, int R> struct GrpRec {
-    static constexpr int PAD = (int)(64 / sizeof(V));
-    static constexpr int VOFF = R + R * R + PAD;
-    static constexpr int RS = VOFF + R;
-    __host__ __device__ static constexpr int m(int c, int cc) { return R + c * R + cc + (c >= R / 2 ? PAD : 0); }
+    static constexpr int T = GrpTile<R>::T, RP = GrpTile<R>::RP;
+    static constexpr bool HALF = R == 4 || R == 8;
+    static constexpr int PADV = HALF ? (int)(64 / sizeof(V)) : (T == 4 ? (int)(16 / sizeof(V)) : 0);
+    static constexpr int PADS = HALF ? PADV : PADV * (RP / T);
+    static constexpr int VOFF = RP + RP * RP + PADS;
+    static constexpr int RS = ((VOFF + RP) * (int)sizeof(V) + 15) / 16 * 16 / (int)sizeof(V);
+    __host__ __device__ static constexpr int m(int c, int cc)
+    {
+        return RP + c * RP + cc + (HALF ? (c >= RP / 2 ? PADV : 0) : (c / T) * PADV);
+    }
 };
 
 // Shared-memory budget of k_group_sums: a block's entries (rows of the
@@ -81,6 +105,19 @@ template <typename T, int R> struct GsumCfg {
     static constexpr int CAP = (int)(46080 / ((R + 1) * VS));   // staged entries per block
     static constexpr size_t SMEM = (size_t)CAP * (R + 1) * VS;
 };
+
+// Zeros into the padded values of a group record (lane of `lanes`).
+template <typename V, int R> __device__ __forceinline__ void grp_zero_padding(V* o, int lane, int lanes)
+{
+    typedef GrpRec<V, R> RL;
+    constexpr int RP = RL::RP;
+    for (int q = lane; q < RP * RP; q += lanes)
+        if (q / RP >= R || q % RP >= R) o[RL::m(q / RP, q % RP)] = czero<V>();
+    for (int q = R + lane; q < RP; q += lanes) {
+        o[q] = czero<V>();
+        o[RL::VOFF + q] = czero<V>();
+    }
+}
 
 // Group sums of one middle level, one thread per (group, row a): the shared
 // vector s of the group (h of a row group, w of a column group, taken from
@@ -115,11 +152,16 @@ k_group_sums(const typename cvec<T>::type* __restrict__ H, const typename cvec<T
     const int E0 = gstart[gb0], E1 = gstart[gb1];
     const bool staged = E1 - E0 <= cap;
     if (staged) {
-        // rows: (E1 - E0) R values, 16-byte pieces (a row is R * VS >= 32 bytes)
-        const int rpieces = (int)((size_t)(E1 - E0) * R * C::VS / 16);
-        const unsigned char* usrc = (const unsigned char*)(Uv + (size_t)E0 * R);
-        for (int q = threadIdx.x; q < rpieces; q += C::NTH)
-            cp_async16((unsigned char*)su + 16 * (size_t)q, usrc + 16 * (size_t)q);
+        // rows: (E1 - E0) R contiguous values, in 16-byte pieces; in 8-byte
+        // ones in complex64 at odd rank, where a row can start between them
+        if constexpr ((R * C::VS) % 16 == 0) {
+            const int rpieces = (int)((size_t)(E1 - E0) * R * C::VS / 16);
+            const unsigned char* usrc = (const unsigned char*)(Uv + (size_t)E0 * R);
+            for (int q = threadIdx.x; q < rpieces; q += C::NTH)
+                cp_async16((unsigned char*)su + 16 * (size_t)q, usrc + 16 * (size_t)q);
+        } else {
+            for (int q = threadIdx.x; q < (E1 - E0) * R; q += C::NTH) cp_async8(su + q, Uv + (size_t)E0 * R + q);
+        }
         // values: one copy per entry (8 or 16 bytes)
         for (int q = threadIdx.x; q < E1 - E0; q += C::NTH) {
             if constexpr (sizeof(V) == 16)
@@ -140,6 +182,7 @@ k_group_sums(const typename cvec<T>::type* __restrict__ H, const typename cvec<T
     const V* tb = staged ? st : tv + E0;
     V* o = out + (size_t)g * RS;
     o[a] = Sv[(size_t)e0 * R + a];
+    if (RL::RP > R && a == 0) grp_zero_padding<V, R>(o, 0, 1);
     V ms[R], vs;
     float mc[R][2], vc[2];
 #pragma unroll
@@ -196,6 +239,44 @@ k_group_sums(const typename cvec<T>::type* __restrict__ H, const typename cvec<T
         vs.y -= vc[1];
     }
     o[RL::VOFF + a] = vs;
+}
+
+// Group sums of a level with many entries per group: one warp per group
+// (warp_sums: the lower triangle of M and v, chunks of 32 entries), the upper
+// triangle of M by conjugation.  Same record as k_group_sums, whose block
+// holds 128 / R groups: with hundreds of entries in each, few threads would
+// walk long lists.
+template <typename T, int R>
+__global__ void __launch_bounds__(128)
+k_group_sums_warp(const typename cvec<T>::type* __restrict__ H, const typename cvec<T>::type* __restrict__ Wm,
+                  const typename cvec<T>::type* __restrict__ tv, const int32_t* __restrict__ gstart, int G, int by_col,
+                  typename cvec<T>::type* __restrict__ out)
+{
+    typedef typename cvec<T>::type V;
+    typedef GrpRec<V, R> RL;
+    __shared__ __align__(16) V a_s[4][32 * R];
+    __shared__ V t_s[4][32];
+    const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
+    const int g = blockIdx.x * 4 + wib;
+    if (g >= G) return;   // whole warp leaves; only warp-level barriers below
+    const V* Sv = by_col ? Wm : H;
+    const V* Uv = by_col ? H : Wm;
+    const int e0 = gstart[g];
+    V* o = out + (size_t)g * RL::RS;
+    if (lane < R) o[lane] = Sv[(size_t)e0 * R + lane];
+    if (RL::RP > R) grp_zero_padding<V, R>(o, lane, 32);
+    warp_sums<T, R>(Uv, tv, e0, gstart[g + 1], a_s[wib], t_s[wib], lane, [&](int, int p, int q, V s, V c) {
+        if constexpr (sizeof(T) == 4) {
+            s.x = __fsub_rn(s.x, c.x);
+            s.y = __fsub_rn(s.y, c.y);
+        }
+        if (q < 0) {
+            o[RL::VOFF + p] = s;
+        } else {
+            o[RL::m(p, q)] = s;
+            if (p != q) o[RL::m(q, p)] = make_conj(s);
+        }
+    });
 }
 
 // acc += x * y.  Precision form: (s, c) is a Kahan pair per component and
@@ -262,20 +343,26 @@ __device__ __forceinline__ void grp_acc2(uint64_t& s, uint64_t& nc, uint64_t X1,
 }
 
 template <typename T, int R> struct GrpCfg {
-    static_assert(R == 4 || R == 8, "grouped Gram tiles need R in {4, 8}");
+    static_assert(R >= 2, "grouped Gram needs R >= 2");
+    static constexpr int TT = GrpTile<R>::T, RP = GrpTile<R>::RP;
     static constexpr int D = R * R;
-    static constexpr int NB = D / 4;
-    static constexpr int NT = NB * (NB + 1) / 2;           // 4 x 4 tiles of the lower triangle
-    static constexpr int CG = sizeof(T) == 4 ? 32 : 16;    // groups per chunk
-    static constexpr int GT = (160 / NT) < 1 ? 1 : (160 / NT);
-    static constexpr int G = GT > CG ? CG : GT;            // thread groups over the chunk's groups
-    static constexpr int NW = NT * G;                      // tile threads
+    static constexpr int NB = R * RP / TT;                 // tile rows over p' = a RP + c
+    static constexpr int NT = NB * (NB + 1) / 2;           // T x T tiles of the lower triangle
+    // groups per chunk
+    static constexpr int CG = (sizeof(T) == 4 ? 32 : 16) / (R >= 11 ? 2 : 1);
+    // blocks that share a slice's tiles (ranks 9, 11, 12: 378 to 666 tiles): in
+    // one block of 666 threads a thread has 80 registers, too few for its sums
+    static constexpr int NSPLIT = NT > 224 ? (NT + 191) / 192 : 1;
+    static constexpr int NTB = (NT + NSPLIT - 1) / NSPLIT; // tiles of a block
+    static constexpr int GT = (160 / NTB) < 1 ? 1 : (160 / NTB);
+    static constexpr int G = NSPLIT > 1 ? 1 : (GT > CG ? CG : GT);   // thread groups over the chunk's groups
+    static constexpr int NW = NTB * G;                     // tile threads
     static constexpr int NTH = ((NW + 31) / 32) * 32;
     // the right-hand side on the threads past the tiles when there are
     // enough of them (R = 8: 24 threads, 3 entries of y each), else on the
     // diagonal tiles
     static constexpr int NY = NTH - NW;
-    static constexpr bool YSPARE = NY >= 8;
+    static constexpr bool YSPARE = G == 1 && NSPLIT == 1 && NY >= 8 && (D + NY - 1) / NY <= TT;
     static constexpr int YPT = YSPARE ? (D + NY - 1) / NY : 0;
     static constexpr int NST = 3;                          // ring stages
     static constexpr int NPK = D * (D + 1) / 2;
@@ -288,11 +375,29 @@ template <typename T, int R> struct GrpCfg {
     static constexpr size_t RING = NST * STAGE;
     static constexpr size_t KBYTES = G > 1 ? (size_t)(NPK + D) * sizeof(double2) : 0;
     static constexpr size_t SMEM = RING + KBYTES;
-    static constexpr int MINB = sizeof(T) == 4 ? 3 : 2;
+    static_assert(SMEM <= 227 * 1024, "shared memory of a block");
+    // blocks per SM the registers are budgeted for: a tile's sums (and, in the
+    // precision form, compensations) take 4 T^2 registers, plus about 64 (25
+    // outputs at T = 5, 104 registers at T = 3 and 4 in complex64)
+    static constexpr int REGS = 4 * TT * TT + 68;
+    static constexpr int MINB0 = 65536 / (NTH * REGS);
+    static constexpr int MINB1 = sizeof(T) == 4 ? 3 : 2;
+    static constexpr int MINB = MINB0 < 1 ? 1 : (MINB0 > MINB1 ? MINB1 : MINB0);
 };
 
-// Per-slice normal equations from the group records of k_group_sums (one
-// block per slice, grid-stride).  Chunks of CG records stream through an
+// T consecutive values: 16-byte loads where T and the alignment allow.
+template <typename V, int TT> __device__ __forceinline__ void load_t(V (&d)[TT], const V* p)
+{
+    if constexpr (TT == 4) {
+        load4(d, p);
+    } else {
+#pragma unroll
+        for (int u = 0; u < TT; ++u) d[u] = p[u];
+    }
+}
+
+// Per-slice normal equations from the group records of k_group_sums (NSPLIT
+// blocks per slice; the grid is a multiple of NSPLIT, grid-stride).  Chunks of CG records stream through an
 // NST-stage shared-memory ring by 16-byte cp.async copies; per group, the
 // shared side's outer product is formed in registers (conj(s_a) s_a' for row
 // groups; conj(s_c) s_c' for column groups) and multiplied with the other
@@ -307,21 +412,24 @@ k_mid_gram_grp(const typename cvec<T>::type* __restrict__ grec, const int32_t* _
     typedef typename cvec<T>::type V;
     typedef GrpCfg<T, R> C;
     constexpr int D = C::D, NPK = C::NPK, CG = C::CG, NTH = C::NTH, RS = C::RS, NST = C::NST;
+    constexpr int TT = C::TT, RP = C::RP;
     extern __shared__ __align__(16) unsigned char smem[];
     typedef typename C::RL RL;
     V* ring = (V*)smem;                           // [NST][CG][RS]
     double2* Kacc = (double2*)(smem + C::RING);   // thread-group reduction (G > 1)
 
     const int tid = threadIdx.x;
-    const bool worker = tid < C::NW;
+    const int part = C::NSPLIT > 1 ? blockIdx.x % C::NSPLIT : 0;   // this block's share of the tiles
+    const bool worker = tid < C::NW && part * C::NTB + tid < C::NT * C::G;
     const bool ythread = C::YSPARE && !worker;
-    const int grp = worker ? tid / C::NT : 0, tile = worker ? tid - grp * C::NT : 0;
+    const int grp = worker ? tid / C::NTB : 0, tile = worker ? part * C::NTB + tid - grp * C::NTB : 0;
     int I = 0;
     while ((I + 1) * (I + 2) / 2 <= tile) ++I;
     const int J = tile - I * (I + 1) / 2;
     const bool diag = !C::YSPARE && (I == J);
-    // row p = 4 I + u of K is the pair (a, c) = (p / R, p mod R): a = aI, c = cI + u
-    const int aI = (4 * I) / R, cI = (4 * I) % R, aJ = (4 * J) / R, cJ = (4 * J) % R;
+    // row T I + u of the padded index a RP + c is the pair a = aI, c = cI + u
+    // (T divides RP); columns likewise
+    const int aI = (TT * I) / RP, cI = (TT * I) % RP, aJ = (TT * J) / RP, cJ = (TT * J) % RP;
     // right-hand side entries p = yb + NY x of a spare thread
     const int yb = tid - C::NW;
 
@@ -333,19 +441,19 @@ k_mid_gram_grp(const typename cvec<T>::type* __restrict__ grec, const int32_t* _
         for (int q = tid; q < pieces; q += NTH) cp_async16(dst + 16 * (size_t)q, src + 16 * (size_t)q);
     };
 
-    for (int k = blockIdx.x; k < S; k += gridDim.x) {
+    for (int k = blockIdx.x / C::NSPLIT; k < S; k += gridDim.x / C::NSPLIT) {
         const int g0 = gseg[k], g1 = gseg[k + 1];
         const int nch = (g1 - g0 + CG - 1) / CG;
         // tiles: s_/c_ (Kahan pairs); right-hand side: ys/yc (diagonal tiles
         // or spare threads)
-        V s_[4][4], c_[4][4], ys[4], yc[4];
-        uint64_t s2[4][4], n2[4][4];   // complex64 tiles: packed Kahan sums, negated compensations
+        V s_[TT][TT], c_[TT][TT], ys[TT], yc[TT];
+        uint64_t s2[TT][TT], n2[TT][TT];   // complex64 tiles: packed Kahan sums, negated compensations
 #pragma unroll
-        for (int u = 0; u < 4; ++u) {
+        for (int u = 0; u < TT; ++u) {
             ys[u] = czero<V>();
             yc[u] = czero<V>();
 #pragma unroll
-            for (int v = 0; v < 4; ++v) {
+            for (int v = 0; v < TT; ++v) {
                 s_[u][v] = czero<V>();
                 c_[u][v] = czero<V>();
                 s2[u][v] = 0ull;
@@ -375,43 +483,43 @@ k_mid_gram_grp(const typename cvec<T>::type* __restrict__ grec, const int32_t* _
                         const V x = cmul(make_conj(gr[aI]), gr[aJ]);
                         const uint64_t X1 = g2pack(x.x, x.x), X2 = g2pack(x.y, x.y);
 #pragma unroll
-                        for (int u = 0; u < 4; ++u) {
-                            V yr[4];
-                            load4(yr, gr + RL::m(cI + u, cJ));
+                        for (int u = 0; u < TT; ++u) {
+                            V yr[TT];
+                            load_t<V, TT>(yr, gr + RL::m(cI + u, cJ));
 #pragma unroll
-                            for (int v = 0; v < 4; ++v)
+                            for (int v = 0; v < TT; ++v)
                                 grp_acc2(s2[u][v], n2[u][v], X1, X2, g2pack(yr[v].x, yr[v].y),
                                          g2pack(-yr[v].y, yr[v].x));
                         }
                         if (diag) {
                             const V xv = make_conj(gr[aI]);
 #pragma unroll
-                            for (int u = 0; u < 4; ++u) grp_acc(ys[u], yc[u], xv, gr[RL::VOFF + cI + u]);
+                            for (int u = 0; u < TT; ++u) grp_acc(ys[u], yc[u], xv, gr[RL::VOFF + cI + u]);
                         }
                     } else {
                         // X = M (sums of the h side); Y = conj(w) w^T from s = w:
                         // term (u, v) = (conj(s_cI+u) x) s_cJ+v
                         const V x = gr[RL::m(aI, aJ)];
-                        V sj[4], si[4];
-                        load4(sj, gr + cJ);
-                        load4(si, gr + cI);
-                        uint64_t Y[4], Q[4];
+                        V sj[TT], si[TT];
+                        load_t<V, TT>(sj, gr + cJ);
+                        load_t<V, TT>(si, gr + cI);
+                        uint64_t Y[TT], Q[TT];
 #pragma unroll
-                        for (int v = 0; v < 4; ++v) {
+                        for (int v = 0; v < TT; ++v) {
                             Y[v] = g2pack(sj[v].x, sj[v].y);
                             Q[v] = g2pack(-sj[v].y, sj[v].x);
                         }
 #pragma unroll
-                        for (int u = 0; u < 4; ++u) {
+                        for (int u = 0; u < TT; ++u) {
                             const V xa = cmul(make_conj(si[u]), x);
                             const uint64_t X1 = g2pack(xa.x, xa.x), X2 = g2pack(xa.y, xa.y);
 #pragma unroll
-                            for (int v = 0; v < 4; ++v) grp_acc2(s2[u][v], n2[u][v], X1, X2, Y[v], Q[v]);
+                            for (int v = 0; v < TT; ++v) grp_acc2(s2[u][v], n2[u][v], X1, X2, Y[v], Q[v]);
                         }
                         if (diag) {
                             const V xv = gr[RL::VOFF + aI];
 #pragma unroll
-                            for (int u = 0; u < 4; ++u) grp_acc(ys[u], yc[u], xv, make_conj(si[u]));
+                            for (int u = 0; u < TT; ++u) grp_acc(ys[u], yc[u], xv, make_conj(si[u]));
                         }
                     }
                 }
@@ -423,35 +531,35 @@ k_mid_gram_grp(const typename cvec<T>::type* __restrict__ grec, const int32_t* _
                         // X = conj(h) h^T from s = h; Y = M (sums of the w side)
                         const V x = cmul(make_conj(gr[aI]), gr[aJ]);
 #pragma unroll
-                        for (int u = 0; u < 4; ++u) {
-                            V yr[4];
-                            load4(yr, gr + RL::m(cI + u, cJ));
+                        for (int u = 0; u < TT; ++u) {
+                            V yr[TT];
+                            load_t<V, TT>(yr, gr + RL::m(cI + u, cJ));
 #pragma unroll
-                            for (int v = 0; v < 4; ++v) grp_acc(s_[u][v], c_[u][v], x, yr[v]);
+                            for (int v = 0; v < TT; ++v) grp_acc(s_[u][v], c_[u][v], x, yr[v]);
                         }
                         if (diag) {
                             const V xv = make_conj(gr[aI]);
 #pragma unroll
-                            for (int u = 0; u < 4; ++u) grp_acc(ys[u], yc[u], xv, gr[RL::VOFF + cI + u]);
+                            for (int u = 0; u < TT; ++u) grp_acc(ys[u], yc[u], xv, gr[RL::VOFF + cI + u]);
                         }
                     } else {
                         // X = M (sums of the h side); Y = conj(w) w^T from s = w
                         const V x = gr[RL::m(aI, aJ)];
-                        V sj[4], si[4];
-                        load4(sj, gr + cJ);
-                        load4(si, gr + cI);
+                        V sj[TT], si[TT];
+                        load_t<V, TT>(sj, gr + cJ);
+                        load_t<V, TT>(si, gr + cI);
 #pragma unroll
-                        for (int v = 0; v < 4; ++v) sj[v] = cmul(x, sj[v]);
+                        for (int v = 0; v < TT; ++v) sj[v] = cmul(x, sj[v]);
 #pragma unroll
-                        for (int u = 0; u < 4; ++u) {
+                        for (int u = 0; u < TT; ++u) {
                             const V a = make_conj(si[u]);
 #pragma unroll
-                            for (int v = 0; v < 4; ++v) grp_acc(s_[u][v], c_[u][v], a, sj[v]);
+                            for (int v = 0; v < TT; ++v) grp_acc(s_[u][v], c_[u][v], a, sj[v]);
                         }
                         if (diag) {
                             const V xv = gr[RL::VOFF + aI];
 #pragma unroll
-                            for (int u = 0; u < 4; ++u) grp_acc(ys[u], yc[u], xv, make_conj(si[u]));
+                            for (int u = 0; u < TT; ++u) grp_acc(ys[u], yc[u], xv, make_conj(si[u]));
                         }
                     }
                 }
@@ -476,9 +584,9 @@ k_mid_gram_grp(const typename cvec<T>::type* __restrict__ grec, const int32_t* _
         cp_async_wait_n<0>();
         if constexpr (sizeof(T) == 4) {
 #pragma unroll
-            for (int u = 0; u < 4; ++u) {
+            for (int u = 0; u < TT; ++u) {
 #pragma unroll
-                for (int v = 0; v < 4; ++v) {
+                for (int v = 0; v < TT; ++v) {
                     const float2 t = g2unpack(g2add(s2[u][v], n2[u][v]));
                     s_[u][v].x = t.x;
                     s_[u][v].y = t.y;
@@ -491,12 +599,13 @@ k_mid_gram_grp(const typename cvec<T>::type* __restrict__ grec, const int32_t* _
         if constexpr (C::G == 1) {
             if (worker) {
 #pragma unroll
-                for (int u = 0; u < 4; ++u) {
-                    const int p = I * 4 + u;
+                for (int u = 0; u < TT; ++u) {
+                    const int p = aI * R + cI + u;
+                    if (RP > R && cI + u >= R) continue;   // padding
 #pragma unroll
-                    for (int v = 0; v < 4; ++v) {
-                        const int q = J * 4 + v;
-                        if (q <= p) out[tri(p, q)] = s_[u][v];
+                    for (int v = 0; v < TT; ++v) {
+                        const int q = aJ * R + cJ + v;
+                        if (q <= p && (RP == R || cJ + v < R)) out[tri(p, q)] = s_[u][v];
                     }
                     if (diag) out[NPK + p] = ys[u];
                 }
@@ -514,12 +623,13 @@ k_mid_gram_grp(const typename cvec<T>::type* __restrict__ grec, const int32_t* _
             for (int g = 0; g < C::G; ++g) {  // deterministic order over the thread groups
                 if (worker && grp == g) {
 #pragma unroll
-                    for (int u = 0; u < 4; ++u) {
-                        const int p = I * 4 + u;
+                    for (int u = 0; u < TT; ++u) {
+                        const int p = aI * R + cI + u;
+                        if (RP > R && cI + u >= R) continue;   // padding
 #pragma unroll
-                        for (int v = 0; v < 4; ++v) {
-                            const int q = J * 4 + v;
-                            if (q <= p) {
+                        for (int v = 0; v < TT; ++v) {
+                            const int q = aJ * R + cJ + v;
+                            if (q <= p && (RP == R || cJ + v < R)) {
                                 Kacc[tri(p, q)].x += (double)s_[u][v].x;
                                 Kacc[tri(p, q)].y += (double)s_[u][v].y;
                             }

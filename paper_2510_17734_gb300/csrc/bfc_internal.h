@@ -128,8 +128,8 @@ struct Ctx {
 bfc_status dalloc(Ctx* c, void** p, size_t bytes, const char* what);
 bfc_status ensure_tmp(Ctx* c, size_t bytes);
 
-// Whether middle level m runs the grouped Gram: gram_impl 0, r = 4 or 8,
-// and fewer groups than the threshold against the per-entry kernel in use.
+// Whether middle level m runs the grouped Gram: gram_impl 0, r >= 2, and
+// fewer groups than the threshold against the per-entry kernel in use.
 bool level_grouped(const Ctx* c, int m);
 
 // Profiling scope around one launch.

@@ -344,28 +344,22 @@ __device__ __forceinline__ bool thread_chol_solve(double2 (&K)[R * (R + 1) / 2],
 }
 
 // ------------------------------------------------------------------------
-// Outer fibers, stage 1: one warp per fiber accumulates K and y (r x r) over
-// the fiber's entries.  A: design vectors in the level order (w_0 for the S^1
-// rows, h_{L+1} for the S^{L+2} columns).  Lanes own the R(R+1)/2 + R items;
-// in float the per-chunk partials are folded into Kahan-compensated sums.
-// Output record per fiber: [K packed (R(R+1)/2) | y (R)] in FP64.
-template <typename T, int R>
-__global__ void __launch_bounds__(128)
-k_outer_gram(const typename cvec<T>::type* __restrict__ A, const typename cvec<T>::type* __restrict__ tv,
-             const int32_t* __restrict__ seg, int nfib, double2* __restrict__ rec)
+// Sums of one warp over the rows s0 .. s1 of A (R values each) and the values
+// tv: K[p][q] = sum conj(a_p) a_q for p >= q and y[p] = sum conj(a_p) t.  Lanes
+// own the R(R+1)/2 + R items; chunks of 32 rows pass through the warp's own
+// shared memory (a_s: 32 R values, t_s: 32); in float the per-chunk partials
+// are folded into Kahan-compensated sums.  emit(item, p, q, sum, comp) hands
+// out every item once (q = -2: y), its value being sum - comp.
+template <typename T, int R, typename F>
+__device__ __forceinline__ void warp_sums(const typename cvec<T>::type* __restrict__ A,
+                                          const typename cvec<T>::type* __restrict__ tv, int s0, int s1,
+                                          typename cvec<T>::type* a_s, typename cvec<T>::type* t_s, int lane, F emit)
 {
     typedef typename cvec<T>::type V;
     constexpr bool COMP = sizeof(T) == 4;
     constexpr int NP = R * (R + 1) / 2;
     constexpr int NI = NP + R;
     constexpr int IPL = (NI + 31) / 32;
-    constexpr int WPB = 4;
-    __shared__ __align__(16) V a_s[WPB][32 * R];
-    __shared__ V t_s[WPB][32];
-    const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
-    const int f = blockIdx.x * WPB + wib;
-    if (f >= nfib) return;  // whole warp leaves; only warp-level barriers below
-    const int s0 = seg[f], s1 = seg[f + 1];
 
     int ip[IPL], iq[IPL];
 #pragma unroll
@@ -395,23 +389,22 @@ k_outer_gram(const typename cvec<T>::type* __restrict__ A, const typename cvec<T
         // a 16-byte boundary)
         {
             const V* src = A + (size_t)base * R;
-            V* dst = a_s[wib];
             const int nv = cnt * R;
             if constexpr (sizeof(V) == 8 && R % 2 == 0) {
                 for (int x = lane; x < nv / 2; x += 32)
-                    reinterpret_cast<float4*>(dst)[x] = reinterpret_cast<const float4*>(src)[x];
+                    reinterpret_cast<float4*>(a_s)[x] = reinterpret_cast<const float4*>(src)[x];
             } else {
-                for (int x = lane; x < nv; x += 32) dst[x] = src[x];
+                for (int x = lane; x < nv; x += 32) a_s[x] = src[x];
             }
-            if (lane < cnt) t_s[wib][lane] = tv[base + lane];
+            if (lane < cnt) t_s[lane] = tv[base + lane];
         }
         __syncwarp();
         for (int e = 0; e < cnt; ++e) {
-            const V* ae = &a_s[wib][e * R];
+            const V* ae = &a_s[e * R];
 #pragma unroll
             for (int u = 0; u < IPL; ++u) {
                 if (ip[u] >= 0) {   // Gram item (iq >= 0) or right-hand side (iq == -2): one code path
-                    const V* bp = iq[u] >= 0 ? ae + iq[u] : &t_s[wib][e];
+                    const V* bp = iq[u] >= 0 ? ae + iq[u] : &t_s[e];
                     cmacc(acc[u], ae[ip[u]], *bp);
                 }
             }
@@ -430,13 +423,30 @@ k_outer_gram(const typename cvec<T>::type* __restrict__ A, const typename cvec<T
 #pragma unroll
     for (int u = 0; u < IPL; ++u) {
         const int it = lane + 32 * u;
-        if (it < NI) {
-            const double2 v = COMP ? make_double2((double)sum[u].x - (double)cmp[u].x,
-                                                  (double)sum[u].y - (double)cmp[u].y)
-                                   : to_d2(acc[u]);
-            rec[(size_t)f * NI + it] = v;
-        }
+        if (it < NI) emit(it, ip[u], iq[u], COMP ? sum[u] : acc[u], cmp[u]);
     }
+}
+
+// Outer fibers, stage 1: one warp per fiber accumulates K and y (r x r) over
+// the fiber's entries (warp_sums).  A: design vectors in the level order (w_0
+// for the S^1 rows, h_{L+1} for the S^{L+2} columns).
+// Output record per fiber: [K packed (R(R+1)/2) | y (R)] in FP64.
+template <typename T, int R>
+__global__ void __launch_bounds__(128)
+k_outer_gram(const typename cvec<T>::type* __restrict__ A, const typename cvec<T>::type* __restrict__ tv,
+             const int32_t* __restrict__ seg, int nfib, double2* __restrict__ rec)
+{
+    typedef typename cvec<T>::type V;
+    constexpr int NI = R * (R + 1) / 2 + R;
+    constexpr int WPB = 4;
+    __shared__ __align__(16) V a_s[WPB][32 * R];
+    __shared__ V t_s[WPB][32];
+    const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
+    const int f = blockIdx.x * WPB + wib;
+    if (f >= nfib) return;  // whole warp leaves; only warp-level barriers below
+    warp_sums<T, R>(A, tv, seg[f], seg[f + 1], a_s[wib], t_s[wib], lane, [&](int it, int, int, V s, V c) {
+        rec[(size_t)f * NI + it] = make_double2((double)s.x - (double)c.x, (double)s.y - (double)c.y);
+    });
 }
 
 // Outer fibers, stage 2: one thread per fiber solves K + lambda I in FP64

@@ -16,18 +16,23 @@ template <typename T, int R> struct Path {
     typedef typename cvec<T>::type V;
     // the tensor-core Gram exists for the complex64 form with R * R <= 64
     static constexpr bool TC = sizeof(T) == 4 && R <= 8;
-    // the grouped Gram's 4 x 4 tiles need R in {4, 8}
-    static constexpr bool GRP = R == 4 || R == 8;
+    // the grouped Gram (rank 1 has nothing to gain: K is one number)
+    static constexpr bool GRP = R >= 2;
+    // entries per group from which a warp takes one group (k_group_sums_warp)
+    // instead of r threads (k_group_sums): at rank 8 and 29 entries per group
+    // the threads are faster (0.140 against 0.154 ms at n = 65536), at rank 12
+    // and 52 to 420 a block's entries outgrow its staging and the warps are
+    static constexpr int GROUP_WARP = 32;
 
     static cudaError_t set_grp_attr()
     {
         if constexpr (GRP) {
-            cudaError_t e = cudaFuncSetAttribute(k_mid_gram_grp<T, GRP ? R : 4, 0>,
+            cudaError_t e = cudaFuncSetAttribute(k_mid_gram_grp<T, GRP ? R : 2, 0>,
                                                  cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                                 (int)GrpCfg<T, GRP ? R : 4>::SMEM);
+                                                 (int)GrpCfg<T, GRP ? R : 2>::SMEM);
             if (e != cudaSuccess) return e;
-            return cudaFuncSetAttribute(k_mid_gram_grp<T, GRP ? R : 4, 1>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                        (int)GrpCfg<T, GRP ? R : 4>::SMEM);
+            return cudaFuncSetAttribute(k_mid_gram_grp<T, GRP ? R : 2, 1>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                        (int)GrpCfg<T, GRP ? R : 2>::SMEM);
         }
         return cudaSuccess;
     }
@@ -76,6 +81,13 @@ template <typename T, int R> struct Path {
     static size_t fallback_bytes(int64_t S)
     {
         return SolveCfg<T, R>::MIXED ? (size_t)S * SolveCfg<T, R>::NPK * sizeof(double2) : 0;
+    }
+
+    // Bytes of one group record of the grouped Gram (0: no grouped Gram).
+    static size_t group_record_bytes()
+    {
+        if constexpr (GRP) return GrpRec<V, GRP ? R : 2>::RS * sizeof(V);
+        return 0;
     }
 
     // One block-coordinate update of an outer factor (rows: S^1, cols: S^{L+2}).
@@ -148,20 +160,26 @@ template <typename T, int R> struct Path {
                 if constexpr (GRP) {
                     if (grouped(c, m)) {
                         const GroupLevel& gl = c->grp[m];
-                        constexpr int RG = GRP ? R : 4;
+                        constexpr int RG = GRP ? R : 2;
                         typedef GsumCfg<T, RG> GS;
                         static_assert(GS::NTH == 128, "host block partition of the group sums");
-                        // shared memory for the level's largest block (at most CAP entries)
-                        const int cap = (int)std::min<int64_t>(gl.max_block, GS::CAP);
-                        k_group_sums<T, RG><<<nblocks(gl.ngroups, GS::GB), GS::NTH,
-                                              (size_t)cap * (RG + 1) * GS::VS, c->stream>>>(
-                            hin, W + (size_t)m * NR, (const V*)c->tval[m], gl.gstart, (int)gl.ngroups, gl.by_col,
-                            (V*)c->grec, cap);
+                        if (c->N >= (int64_t)GROUP_WARP * gl.ngroups) {
+                            k_group_sums_warp<T, RG><<<nblocks(gl.ngroups, 4), 128, 0, c->stream>>>(
+                                hin, W + (size_t)m * NR, (const V*)c->tval[m], gl.gstart, (int)gl.ngroups, gl.by_col,
+                                (V*)c->grec);
+                        } else {
+                            // shared memory for the level's largest block (at most CAP entries)
+                            const int cap = (int)std::min<int64_t>(gl.max_block, GS::CAP);
+                            k_group_sums<T, RG><<<nblocks(gl.ngroups, GS::GB), GS::NTH,
+                                                  (size_t)cap * (RG + 1) * GS::VS, c->stream>>>(
+                                hin, W + (size_t)m * NR, (const V*)c->tval[m], gl.gstart, (int)gl.ngroups, gl.by_col,
+                                (V*)c->grec, cap);
+                        }
                         if (gl.by_col)
-                            k_mid_gram_grp<T, RG, 1><<<(unsigned)S, GrpCfg<T, RG>::NTH, GrpCfg<T, RG>::SMEM,
+                            k_mid_gram_grp<T, RG, 1><<<(unsigned)S * GrpCfg<T, RG>::NSPLIT, GrpCfg<T, RG>::NTH, GrpCfg<T, RG>::SMEM,
                                                        c->stream>>>((const V*)c->grec, gl.gseg, (V*)c->rec, (int)S);
                         else
-                            k_mid_gram_grp<T, RG, 0><<<(unsigned)S, GrpCfg<T, RG>::NTH, GrpCfg<T, RG>::SMEM,
+                            k_mid_gram_grp<T, RG, 0><<<(unsigned)S * GrpCfg<T, RG>::NSPLIT, GrpCfg<T, RG>::NTH, GrpCfg<T, RG>::SMEM,
                                                        c->stream>>>((const V*)c->grec, gl.gseg, (V*)c->rec, (int)S);
                         ps.add_kernels(1);
                         done = true;
