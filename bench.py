@@ -55,20 +55,21 @@ UNIT = "entries/s"
 WORKLOAD = ("n=65536 L=12 b=16 r=8, exp(i w rho)/rho line-to-line kernel, w=pi n/16, h=1.5, "
             "|Omega|=4 n log2 n (3774874 train / 419430 test), lambda=1e-7")
 TC_FLOPS_PER_ENTRY = 2 * 3 * 128 * 144   # flop, one contraction position x M 128 x N 144 x 3 products
-# DRAM counters of one k_mid_gram_tc launch (ncu, n = 32768, L = 11: 1,769,472
-# entries, 4096 slices), valid for the kernel source with this sha256 prefix
-TC_GRAM_TRAFFIC = {"source": "paper_2510_17734_gb300/csrc/bfc_gram_tc.cuh", "sha": "8159f55fbacf40ac",
-                   "read_bytes": 241.090048e6, "write_bytes": 51.348736e6, "entries": 1769472, "slices": 4096}
+# DRAM counters of k_mid_gram_tc at the n = 65536 workload (ncu, one-pass
+# metrics, mean of three launches of the first sweep: 3,774,874 entries, 8192
+# slices per level), valid for the kernel source with this sha256 prefix
+TC_GRAM_TRAFFIC = {"source": "paper_2510_17734_gb300/csrc/bfc_gram_tc.cuh", "sha": "ca3d3494f519d50b",
+                   "read_bytes": 513.94176e6, "write_bytes": 142.995456e6, "entries": 3774874, "slices": 8192}
 
 
 # DRAM counters of k_mid_solve at the n = 65536 workload itself (ncu, one-pass
-# metrics, mean of two launches of the first sweep: 3,774,874 entries, 8192
+# metrics, mean of three launches of the first sweep: 3,774,874 entries, 8192
 # slices per level), valid for the kernel source with this sha256 prefix
-SOLVE_TRAFFIC = {"source": "paper_2510_17734_gb300/csrc/bfc_kernels.cuh", "sha": "fca9bdd68955b392",
-                 # the kernel and the device functions it calls (warp_chol ... k_mid_solve)
-                 "span": ("// Row of slot s owned by a lane in the warp-level factorization",
-                          "// FP64 fallback of the precision form"),
-                 "read_bytes": 427.399552e6, "write_bytes": 213.848576e6, "entries": 3774874, "slices": 8192}
+SOLVE_TRAFFIC = {"source": "paper_2510_17734_gb300/csrc/bfc_solve.cuh", "sha": "ed8040b484dc97cc",
+                 # the kernel and the device functions it calls (KPair ... k_mid_solve)
+                 "span": ("// Arithmetic on pairs of neighbouring k of two rows",
+                          "// FP64 fallback of the precision form: a CTA"),
+                 "read_bytes": 431.426987e6, "write_bytes": 212.522069e6, "entries": 3774874, "slices": 8192}
 
 
 def kernel_source_sha(rel_path: str, span=None) -> str:
@@ -219,7 +220,7 @@ def kernel_rooflines(prob, prof, stats, peaks, fp32_meas):
         out.append({"kernel": "k_mid_solve", "bound": "hbm", "launch_ms": ms, "bytes": by,
                     "achieved": a, "peak": hbm, "unit": "GB/s", "frac": a / hbm, "traffic": traffic,
                     "traffic_source": "ncu dram__bytes_read.sum + dram__bytes_write.sum per launch at this "
-                                      f"workload (kernel source sha {cap['sha']}: warp_chol through k_mid_solve)",
+                                      f"workload (kernel source sha {cap['sha']}: KPair through k_mid_solve)",
                     "flop": fl, "fp32_achieved_tflops": af, "fp32_peak": fp32_meas, "fp32_frac": af / fp32_meas,
                     "refine_steps_per_slice": steps_avg,
                     "per_unit": f"{(npk + D) * 8 + D * 24} B per slice (normal equations in, slice out) + "
@@ -302,8 +303,8 @@ def gram_rooflines(prob, prof, n_sweeps, c64, tc_levels, grouped, peaks, fp32_me
                            + cap["write_bytes"] * (1 << (prob.L + 1)) / cap["slices"])
             out.append({"kernel": "k_mid_gram_tc", "bound": "tensor", "achieved": a, "peak": peak,
                         "unit": "TFLOP/s", "frac": a / peak, "traffic": traffic,
-                        "traffic_source": "ncu dram__bytes_read.sum + dram__bytes_write.sum of one launch at "
-                                          f"n=32768 (kernel source sha {cap['sha']}), scaled by entries (reads) "
+                        "traffic_source": "ncu dram__bytes_read.sum + dram__bytes_write.sum per launch at "
+                                          f"n=65536 (kernel source sha {cap['sha']}), scaled by entries (reads) "
                                           "and slices (writes)",
                         "launch_ms": ms, "launches_per_sweep": n_plain, "ms_per_sweep": tot / n_sweeps,
                         "flop_per_launch": fl,

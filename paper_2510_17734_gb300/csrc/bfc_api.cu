@@ -358,11 +358,7 @@ static bfc_status build(Ctx* c, const Inputs& in)
     for (const GroupLevel& gl : c->grp)
         if (gl.gstart) gmax = std::max(gmax, gl.ngroups);
     if (gmax > 0) BFC_TRY(dalloc(c, &c->grec, (size_t)gmax * ops->group_record_bytes(), "group records"));
-    const size_t fbb = ops->fallback_bytes(S);
-    if (fbb > 0 && L > 0) {
-        BFC_TRY(dalloc(c, (void**)&c->fb, fbb, "FP64 fallback records"));
-        BFC_TRY(dalloc(c, (void**)&c->fblist, (size_t)S * sizeof(int32_t), "fallback list"));
-    }
+    if (c->fp32 && L > 0) BFC_TRY(dalloc(c, (void**)&c->fblist, (size_t)S * sizeof(int32_t), "fallback list"));
     BFC_TRY(ops->configure(c));
     return sync(c);
 }

@@ -407,10 +407,11 @@ template <typename V, int TT> __device__ __forceinline__ void load_t(V (&d)[TT],
 template <typename T, int R, int BY_COL>
 __global__ void __launch_bounds__(GrpCfg<T, R>::NTH, GrpCfg<T, R>::MINB)
 k_mid_gram_grp(const typename cvec<T>::type* __restrict__ grec, const int32_t* __restrict__ gseg,
-               typename cvec<T>::type* __restrict__ rec, int S)
+               T* __restrict__ rec, int S)
 {
     typedef typename cvec<T>::type V;
     typedef GrpCfg<T, R> C;
+    typedef Rec<T, R> RC;
     constexpr int D = C::D, NPK = C::NPK, CG = C::CG, NTH = C::NTH, RS = C::RS, NST = C::NST;
     constexpr int TT = C::TT, RP = C::RP;
     extern __shared__ __align__(16) unsigned char smem[];
@@ -595,7 +596,7 @@ k_mid_gram_grp(const typename cvec<T>::type* __restrict__ grec, const int32_t* _
                 ys[u].y = __fsub_rn(ys[u].y, yc[u].y);
             }
         }
-        V* out = rec + (size_t)k * (NPK + D);
+        T* out = rec + (size_t)k * RC::SIZE;
         if constexpr (C::G == 1) {
             if (worker) {
 #pragma unroll
@@ -605,15 +606,15 @@ k_mid_gram_grp(const typename cvec<T>::type* __restrict__ grec, const int32_t* _
 #pragma unroll
                     for (int v = 0; v < TT; ++v) {
                         const int q = aJ * R + cJ + v;
-                        if (q <= p && (RP == R || cJ + v < R)) out[tri(p, q)] = s_[u][v];
+                        if (q <= p && (RP == R || cJ + v < R)) RC::put(out, p, q, s_[u][v]);
                     }
-                    if (diag) out[NPK + p] = ys[u];
+                    if (diag) RC::put_y(out, p, ys[u]);
                 }
             } else if (ythread) {
 #pragma unroll
                 for (int x = 0; x < C::YPT; ++x) {
                     const int p = yb + C::NY * x;
-                    if (p < D) out[NPK + p] = ys[x];
+                    if (p < D) RC::put_y(out, p, ys[x]);
                 }
             }
         } else {
@@ -642,7 +643,7 @@ k_mid_gram_grp(const typename cvec<T>::type* __restrict__ grec, const int32_t* _
                 }
                 __syncthreads();
             }
-            for (int q = tid; q < NPK + D; q += NTH) out[q] = from_d2<V>(Kacc[q]);
+            rec_put_packed<T, R>(out, Kacc, tid, NTH);
         }
     }
 }

@@ -4,7 +4,7 @@
 // with a_e = h_e (x) w_e (a[p R + c] = h_p w_c), the left and right
 // environments of entry e (Alg. 1, middle factors; Eq. (BF_tensor_rep)
 // read as a linear function of one slice).  Same output record as the
-// CUDA-core k_mid_gram: K packed lower-triangular, then y.
+// CUDA-core k_mid_gram (Rec).
 //
 // Real form of the complex sums.  Write a = u + i v.  Then
 //     Re K[p][q] = UU[p][q] + VV[p][q],   Im K[p][q] = UV[p][q] - VU[p][q],
@@ -58,6 +58,8 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include "bfc_kernels.cuh"
+
 namespace bfc {
 
 struct TcGram {
@@ -73,7 +75,7 @@ struct TcGram {
     static constexpr int NBUILD = 8;              // operand builder warps
     static constexpr int NFOLD = 8;               // fold warps: 2 per TMEM lane quadrant
     static constexpr int NTH = 32 * (NBUILD + NFOLD + 2);   // + the MMA warp + the input-loader warp
-    static constexpr int RECB = (64 * 65 / 2 + 64) * 8;  // packed record copy (rank 8; a multiple of 16 bytes)
+    static constexpr int RECB = Rec<float, 8>::SIZE * 4;  // record copy (rank 8 is the largest; a multiple of 16 bytes)
     static constexpr int SEGC = 1024;             // cached (start, end) of this CTA's first slices
     static constexpr int NIN = 4;
     static constexpr int NBARS = 9 + 2 * NIN;     // 9 pipeline barriers + 2 x NIN input-ring barriers
@@ -215,15 +217,16 @@ struct TcFold {
 template <int R>
 __global__ void __launch_bounds__(TcGram::NTH, 1)
 k_mid_gram_tc(const float2* __restrict__ H, const float2* __restrict__ Wm, const float2* __restrict__ tv,
-              const int32_t* __restrict__ seg, float2* __restrict__ rec, int S, unsigned long long* err)
+              const int32_t* __restrict__ seg, float* __restrict__ rec, int S, unsigned long long* err)
 {
     static_assert(R >= 1 && R <= 8, "tensor-core Gram needs R*R <= 64");
-    constexpr int D = R * R, NPK = D * (D + 1) / 2, CE = TcGram::CE, NBIG = TcGram::NBIG;
+    typedef Rec<float, R> RC;
+    constexpr int D = R * R, CE = TcGram::CE, NBIG = TcGram::NBIG;
     constexpr int NF = 32 * TcGram::NFOLD;    // fold threads
     extern __shared__ unsigned char smem_raw[];
     const uint32_t raw_s = tc_smem_u32(smem_raw);
     unsigned char* ops = smem_raw + ((1024u - (raw_s & 1023u)) & 1023u);  // 2 operand stages
-    float* recs = (float*)(ops + 2 * TcGram::STAGE);                       // packed record copy
+    float* recs = (float*)(ops + 2 * TcGram::STAGE);                       // record copy
     int2* segc = (int2*)((unsigned char*)recs + TcGram::RECB);             // slice bounds cache
     uint64_t* bars = (uint64_t*)(segc + TcGram::SEGC);
     uint64_t* full = bars;            // [2]     builders -> MMA warp (count NBUILD)
@@ -244,8 +247,7 @@ k_mid_gram_tc(const float2* __restrict__ H, const float2* __restrict__ Wm, const
     for (int x = tid; x < 2 * TcGram::STAGE / 16; x += TcGram::NTH) ((uint4*)ops)[x] = make_uint4(0, 0, 0, 0);
     for (int k = blockIdx.x; k < S; k += gridDim.x)
         if (seg[k + 1] == seg[k])
-            for (int x = tid; x < NPK + D; x += TcGram::NTH)
-                rec[(size_t)k * (NPK + D) + x] = make_float2(0.f, 0.f);
+            for (int x = tid; x < RC::SIZE; x += TcGram::NTH) rec[(size_t)k * RC::SIZE + x] = 0.f;
     for (int i = tid; i < TcGram::SEGC; i += TcGram::NTH) {
         const int k = blockIdx.x + i * gridDim.x;
         if (k >= S) break;
@@ -463,21 +465,29 @@ k_mid_gram_tc(const float2* __restrict__ H, const float2* __restrict__ Wm, const
                 s2[j] = t;
             }
         };
-        // record copy in shared memory: the u lanes write Re, the v lanes Im
+        // record copy in shared memory: the u lanes write Re, the v lanes Im.
+        // Half hh of column block c is panel 2 c + hh of the record: this
+        // lane's 8 values are one half of row p, stored whole (what lies above
+        // the diagonal is not read)
         auto put_half = [&](int c, int hh, const uint64_t* s2, const uint64_t* c2, const float* w) {
+            float v8[8];
 #pragma unroll
             for (int jj = 0; jj < 4; ++jj) {
                 const int j = 4 * hh + jj;
                 float s0, s1, c0, c1;
                 f2unpack(s2[j], s0, s1);
                 f2unpack(c2[j], c0, c1);
-                const float v2[2] = {(s0 - c0) + pair(w[2 * jj], w[8 + 2 * jj]),
-                                     (s1 - c1) + pair(w[2 * jj + 1], w[8 + 2 * jj + 1])};
+                v8[2 * jj] = (s0 - c0) + pair(w[2 * jj], w[8 + 2 * jj]);
+                v8[2 * jj + 1] = (s1 - c1) + pair(w[2 * jj + 1], w[8 + 2 * jj + 1]);
+            }
+            const int J = 2 * c + hh;
+            if (J < RC::NPAN && p < D && p >= 8 * J) {
 #pragma unroll
-                for (int h = 0; h < 2; ++h) {
-                    const int q = 16 * c + 2 * j + h;
-                    if (p < D && q <= p) recs[2 * (p * (p + 1) / 2 + q) + (is_u ? 0 : 1)] = (q == p && !is_u) ? 0.f : v2[h];
-                }
+                for (int q = 0; q < 8; ++q)
+                    if (!is_u && 8 * J + q == p) v8[q] = 0.f;   // Im K[p][p]
+                float4* o = reinterpret_cast<float4*>(recs + RC::row(J, p - 8 * J) + (is_u ? 0 : 8));
+                o[0] = make_float4(v8[0], v8[1], v8[2], v8[3]);
+                o[1] = make_float4(v8[4], v8[5], v8[6], v8[7]);
             }
         };
 
@@ -548,7 +558,7 @@ k_mid_gram_tc(const float2* __restrict__ H, const float2* __restrict__ Wm, const
                     asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
                 }
                 const float yv = (sum_y - comp_y) + pair(v[0], v[1]);
-                if (p < D) recs[2 * (NPK + p) + (is_u ? 0 : 1)] = yv;
+                if (p < D) recs[RC::re(D, p) + (is_u ? 0 : 8)] = is_u ? yv : -yv;   // conj(y)
             }
             asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
             __syncwarp();
@@ -560,11 +570,10 @@ k_mid_gram_tc(const float2* __restrict__ H, const float2* __restrict__ Wm, const
             sum_y = 0.f;
             comp_y = 0.f;
             asm volatile("bar.sync 1, %0;" ::"n"(NF) : "memory");
-            // the record (NPK + D complex values, an even count for D = R^2,
-            // so records start on 16-byte boundaries) in 16-byte pieces
+            // the record (a multiple of 16 bytes) in 16-byte pieces
             const float4* src = (const float4*)recs;
-            float4* out = (float4*)(rec + (size_t)f.k * (NPK + D));
-            for (int x = tid - 32 * TcGram::NBUILD; x < (NPK + D) / 2; x += NF) out[x] = src[x];
+            float4* out = (float4*)(rec + (size_t)f.k * RC::SIZE);
+            for (int x = tid - 32 * TcGram::NBUILD; x < RC::SIZE / 4; x += NF) out[x] = src[x];
             asm volatile("bar.sync 1, %0;" ::"n"(NF) : "memory");
         };
 

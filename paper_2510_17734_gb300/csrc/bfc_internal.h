@@ -77,8 +77,7 @@ struct Ctx {
     void* W = nullptr;
     void* H[2] = {nullptr, nullptr};
     void* Rres[2] = {nullptr, nullptr};  // residual carried along the orders (gradient)
-    void* rec = nullptr;              // per-block normal-equation records [K packed | y]
-    double2* fb = nullptr;            // FP64 refinement / fallback records (precision form)
+    void* rec = nullptr;              // normal-equation records (middle slices: Rec, outer fibers: [K packed | y])
     int32_t* fblist = nullptr;        // slices handed to the FP64 fallback in the current level
 
     // factors: FP64 master and compute-type copies (alias when double)

@@ -92,6 +92,42 @@ __device__ __forceinline__ int slice_of(int pi, int pj, int m, int L)
 // Packed lower-triangular index (p >= q).
 __host__ __device__ __forceinline__ constexpr int tri(int p, int q) { return (p * (p + 1) >> 1) + q; }
 
+// Normal-equation record of one middle slice, from the Gram kernels to the
+// solve: the lower triangle of the (D + 1) x (D + 1) matrix [K y; y^H .],
+// D = R^2, in block columns (panels) of 8 columns.  Panel J holds the rows
+// 8J .. D, each as 8 real parts then 8 imaginary parts; row D is conj(y), so
+// the factorization carries the forward substitution along as one more row.
+// Every four rows are followed by 16 bytes of padding: 8 lanes reading 16
+// bytes of rows four apart then fall into distinct shared-memory banks.
+// Elements above the diagonal and the padding are not written.  Offsets are in
+// values of T, every row starts on a 16-byte boundary, and the solve's copy in
+// shared memory has the same layout.
+template <typename T, int R> struct Rec {
+    static constexpr int D = R * R, DR = D + 1, NPAN = (D + 7) / 8;
+    static constexpr int PADT = 16 / (int)sizeof(T);
+    __host__ __device__ static constexpr int base(int J)
+    {
+        return 16 * (J * DR - 4 * J * (J - 1)) + PADT * (J * ((DR + 3) / 4) - J * (J - 1));
+    }
+    // row 8 J + rho of panel J
+    __host__ __device__ static constexpr int row(int J, int rho) { return base(J) + rho * 16 + (rho >> 2) * PADT; }
+    // real part of element (p, q), p >= q (imaginary part 8 values further); p = D: conj(y_q)
+    __host__ __device__ static constexpr int re(int p, int q) { return row(q >> 3, p - (q & ~7)) + (q & 7); }
+    static constexpr int SIZE = base(NPAN);
+    template <typename V> __device__ static __forceinline__ void put(T* rec, int p, int q, V v)
+    {
+        const int o = re(p, q);
+        rec[o] = (T)v.x;
+        rec[o + 8] = (T)v.y;
+    }
+    template <typename V> __device__ static __forceinline__ void put_y(T* rec, int p, V v)
+    {
+        const int o = re(D, p);
+        rec[o] = (T)v.x;
+        rec[o + 8] = (T)-v.y;
+    }
+};
+
 // ------------------------------------------------------------------------
 // Right environments, one level: w_{m-1} = Z^{m+1}(k) w_m for every entry of
 // slice k (Alg. 1: the right vector v, built from the right end).  One CTA
@@ -557,7 +593,7 @@ k_outer_post(const typename cvec<T>::type* __restrict__ A, const typename cvec<T
 // into the other staging buffer with cp.async.  In float every FOLD chunks
 // the register partials are folded into Kahan-compensated running sums
 // (sums in registers, compensation in shared memory).
-// Output record per slice: [K packed lower | y] in the compute type.
+// Output record per slice: Rec<T, R>.
 template <typename T, int R> struct GramCfg {
     static constexpr int D = R * R;
     static constexpr int DP = (D + 3) / 4 * 4;
@@ -596,14 +632,27 @@ __device__ __forceinline__ void cp_async_v(double2* smem_dst, const double2* gme
 __device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
 __device__ __forceinline__ void cp_async_wait_all() { asm volatile("cp.async.wait_group 0;" ::: "memory"); }
 
+// The record from [K packed lower | y] in FP64 (a block's thread-group sums).
+template <typename T, int R>
+__device__ __forceinline__ void rec_put_packed(T* out, const double2* Kacc, int tid, int nthr)
+{
+    constexpr int D = R * R;
+    for (int x = tid; x < D * D; x += nthr) {
+        const int p = x / D, q = x - p * D;
+        if (q <= p) Rec<T, R>::put(out, p, q, Kacc[tri(p, q)]);
+    }
+    for (int p = tid; p < D; p += nthr) Rec<T, R>::put_y(out, p, Kacc[D * (D + 1) / 2 + p]);
+}
+
 template <typename T, int R>
 __global__ void __launch_bounds__(GramCfg<T, R>::NTH, GramCfg<T, R>::MINB)
 k_mid_gram(const typename cvec<T>::type* __restrict__ H, const typename cvec<T>::type* __restrict__ Wm,
            const typename cvec<T>::type* __restrict__ tv, const int32_t* __restrict__ seg,
-           typename cvec<T>::type* __restrict__ rec, int S)
+           T* __restrict__ rec, int S)
 {
     typedef typename cvec<T>::type V;
     typedef GramCfg<T, R> C;
+    typedef Rec<T, R> RC;
     constexpr int D = C::D, DP = C::DP, NPK = C::NPK, CE = C::CE, NTH = C::NTH;
     extern __shared__ __align__(16) unsigned char smem[];
     V* ring = (V*)smem;                                      // [2][CE][DP]
@@ -740,7 +789,7 @@ k_mid_gram(const typename cvec<T>::type* __restrict__ H, const typename cvec<T>:
                 }
             }
         }
-        V* out = rec + (size_t)k * (NPK + D);
+        T* out = rec + (size_t)k * RC::SIZE;
         if (C::G == 1) {
             if (worker) {
 #pragma unroll
@@ -750,9 +799,9 @@ k_mid_gram(const typename cvec<T>::type* __restrict__ H, const typename cvec<T>:
 #pragma unroll
                         for (int v = 0; v < 4; ++v) {
                             const int q = J * 4 + v;
-                            if (q <= p) out[tri(p, q)] = acc[u][v];
+                            if (q <= p) RC::put(out, p, q, acc[u][v]);
                         }
-                        if (diag) out[NPK + p] = yacc[u];
+                        if (diag) RC::put_y(out, p, yacc[u]);
                     }
                 }
             }
@@ -783,768 +832,8 @@ k_mid_gram(const typename cvec<T>::type* __restrict__ H, const typename cvec<T>:
                 }
                 __syncthreads();
             }
-            for (int q = tid; q < NPK + D; q += NTH) out[q] = from_d2<V>(Kacc[q]);
+            rec_put_packed<T, R>(out, Kacc, tid, NTH);
         }
-    }
-}
-
-// ------------------------------------------------------------------------
-// Row of slot s owned by a lane in the warp-level factorization: even slots
-// take rows 32 s + lane, odd slots mirror them (32 s + 31 - lane), so the two
-// rows of a lane have complementary lengths and the work per lane is balanced.
-__device__ __forceinline__ int owned_row(int s, int lane) { return 32 * s + ((s & 1) ? 31 - lane : lane); }
-
-// Warp-level Hermitian Cholesky (K = L L^H) of a D x D packed lower matrix
-// in shared or global memory, right-looking and blocked by NBK columns:
-//  (1) the NBK x NBK diagonal block is factored column by column;
-//  (2) every panel row r below it, owned by one lane, is solved in registers:
-//      L[r][j0..j1) = K[r][j0..j1) L_dd^{-H};
-//  (3) the trailing matrix gets the rank-NBK update
-//      L[r][q] -= sum_k L[r][j0+k] conj(L[q][j0+k]), the lane holding its
-//      panel row in registers while all lanes read the same panel row q.
-// The diagonal of L is real, so its imaginary slot stores 1 / L_cc for the
-// triangular solves.  Returns false (warp-uniform) when a pivot is <= tol.
-template <typename E, typename S, int NS>
-__device__ bool warp_chol(E* Lm, int D, S tol, int lane)
-{
-    constexpr int NBK = 8;
-    for (int j0 = 0; j0 < D; j0 += NBK) {
-        const int j1 = min(j0 + NBK, D);
-        // (1) diagonal block
-        for (int c = j0; c < j1; ++c) {
-            __syncwarp();
-            const S d = Lm[tri(c, c)].x;
-            if (!(d > tol)) return false;
-            const S piv = sqrt(d), inv = S(1) / piv;
-            __syncwarp();
-            if (lane == 0) {
-                E v;
-                v.x = piv;
-                v.y = inv;
-                Lm[tri(c, c)] = v;
-            }
-            const int r = c + 1 + lane;
-            if (r < j1) {
-                E l = Lm[tri(r, c)];
-                l.x *= inv;
-                l.y *= inv;
-                Lm[tri(r, c)] = l;
-            }
-            __syncwarp();
-            if (r < j1) {
-                const E a = Lm[tri(r, c)];
-                for (int q = c + 1; q <= r; ++q) {
-                    E cur = Lm[tri(r, q)];
-                    csub_mul_conj(cur, a, Lm[tri(q, c)]);
-                    Lm[tri(r, q)] = cur;
-                }
-            }
-        }
-        __syncwarp();
-        if (j1 >= D) break;
-        const int nb = j1 - j0;
-        // (2) panel rows, solved in registers by their owner lanes
-        E x[NS][NBK];
-        if constexpr (sizeof(S) == 4) {
-            // complex64: the same substitution with the terms as packed fused
-            // multiply-adds (the trailing update's form below)
-#pragma unroll
-            for (int s = 0; s < NS; ++s) {
-                const int r = owned_row(s, lane);
-                if (r >= j1 && r < D) {
-                    E* rowp = Lm + tri(r, 0);
-                    uint64_t p1[NBK], p2[NBK];
-#pragma unroll
-                    for (int cc = 0; cc < NBK; ++cc) {
-                        x[s][cc] = E{};
-                        p1[cc] = 0ull;
-                        p2[cc] = 0ull;
-                        if (cc < nb) {
-                            const uint64_t* drow = reinterpret_cast<const uint64_t*>(Lm + tri(j0 + cc, 0) + j0);
-                            const E e0 = rowp[j0 + cc];
-                            uint64_t acc = c2pack(e0.x, e0.y), sw = 0ull;
-#pragma unroll
-                            for (int k = 0; k < cc; ++k) {
-                                const uint64_t b = drow[k];
-                                acc = c2fma(b, p1[k], acc);
-                                sw = c2fma(b, p2[k], sw);
-                            }
-                            float ar, ai, si, sr;
-                            c2unpack(acc, ar, ai);
-                            c2unpack(sw, si, sr);
-                            const S inv = Lm[tri(j0 + cc, j0 + cc)].y;
-                            E v;
-                            v.x = (ar + sr) * inv;
-                            v.y = (ai + si) * inv;
-                            x[s][cc] = v;
-                            p1[cc] = c2pack(-v.x, v.x);
-                            p2[cc] = c2pack(-v.y, -v.y);
-                        }
-                    }
-#pragma unroll
-                    for (int k = 0; k < NBK; ++k)
-                        if (k < nb) rowp[j0 + k] = x[s][k];
-                }
-            }
-        } else {
-#pragma unroll
-        for (int s = 0; s < NS; ++s) {
-            const int r = owned_row(s, lane);
-            if (r >= j1 && r < D) {
-                const E* rowp = Lm + tri(r, 0);
-#pragma unroll
-                for (int k = 0; k < NBK; ++k) x[s][k] = k < nb ? rowp[j0 + k] : E{};
-#pragma unroll
-                for (int cc = 0; cc < NBK; ++cc) {
-                    if (cc < nb) {
-                        const E* drow = Lm + tri(j0 + cc, 0);
-#pragma unroll
-                        for (int k = 0; k < cc; ++k) csub_mul_conj(x[s][cc], x[s][k], drow[j0 + k]);
-                        const S inv = drow[j0 + cc].y;
-                        x[s][cc].x *= inv;
-                        x[s][cc].y *= inv;
-                    }
-                }
-                E* roww = Lm + tri(r, 0);
-#pragma unroll
-                for (int k = 0; k < NBK; ++k)
-                    if (k < nb) roww[j0 + k] = x[s][k];
-            }
-        }
-        }
-        __syncwarp();
-        // (3) rank-NBK trailing update
-        if constexpr (sizeof(S) == 4) {
-            // complex64: L[r][q] -= sum_k x_k conj(l_k) (l = L[q][j0 + k]) as
-            // two packed fused multiply-adds per term, with the factors of
-            // x_k prepared once per row: l (.) (-x.re, x.re) goes into
-            // (re, im) and l (.) (-x.im, -x.im) into a second accumulator
-            // that holds (im, re)
-#pragma unroll
-            for (int s = 0; s < NS; ++s) {
-                const int r = owned_row(s, lane);
-                if (r >= j1 && r < D) {
-                    uint64_t p1[NBK], p2[NBK];
-#pragma unroll
-                    for (int k = 0; k < NBK; ++k) {
-                        const float xr = k < nb ? x[s][k].x : 0.f, xi = k < nb ? x[s][k].y : 0.f;
-                        p1[k] = c2pack(-xr, xr);
-                        p2[k] = c2pack(-xi, -xi);
-                    }
-                    E* rowp = Lm + tri(r, 0);
-                    auto finish = [&](uint64_t acc, uint64_t sw) {
-                        float ar, ai, si, sr;
-                        c2unpack(acc, ar, ai);
-                        c2unpack(sw, si, sr);
-                        E v;
-                        v.x = ar + sr;
-                        v.y = ai + si;
-                        return v;
-                    };
-                    int q = j1;
-                    for (; q + 1 <= r; q += 2) {
-                        const uint64_t* qa = reinterpret_cast<const uint64_t*>(Lm + tri(q, 0) + j0);
-                        const uint64_t* qb = reinterpret_cast<const uint64_t*>(Lm + tri(q + 1, 0) + j0);
-                        const E ea = rowp[q], eb = rowp[q + 1];
-                        uint64_t ca = c2pack(ea.x, ea.y), cb = c2pack(eb.x, eb.y), sa = 0ull, sb = 0ull;
-                        uint64_t va[NBK], vb[NBK];
-#pragma unroll
-                        for (int k = 0; k < NBK; ++k)
-                            if (k < nb) { va[k] = qa[k]; vb[k] = qb[k]; }
-#pragma unroll
-                        for (int k = 0; k < NBK; ++k)
-                            if (k < nb) {
-                                ca = c2fma(va[k], p1[k], ca);
-                                sa = c2fma(va[k], p2[k], sa);
-                                cb = c2fma(vb[k], p1[k], cb);
-                                sb = c2fma(vb[k], p2[k], sb);
-                            }
-                        rowp[q] = finish(ca, sa);
-                        rowp[q + 1] = finish(cb, sb);
-                    }
-                    if (q <= r) {
-                        const uint64_t* qr = reinterpret_cast<const uint64_t*>(Lm + tri(q, 0) + j0);
-                        const E e0 = rowp[q];
-                        uint64_t c0 = c2pack(e0.x, e0.y), s0 = 0ull;
-#pragma unroll
-                        for (int k = 0; k < NBK; ++k)
-                            if (k < nb) {
-                                const uint64_t v = qr[k];
-                                c0 = c2fma(v, p1[k], c0);
-                                s0 = c2fma(v, p2[k], s0);
-                            }
-                        rowp[q] = finish(c0, s0);
-                    }
-                }
-            }
-        } else {
-#pragma unroll
-        for (int s = 0; s < NS; ++s) {
-            const int r = owned_row(s, lane);
-            if (r >= j1 && r < D) {
-                E* rowp = Lm + tri(r, 0);
-                // two columns per step: both elements and both panel rows are
-                // loaded before either element is stored (independent chains)
-                int q = j1;
-                for (; q + 1 <= r; q += 2) {
-                    const E* qa = Lm + tri(q, 0) + j0;
-                    const E* qb = Lm + tri(q + 1, 0) + j0;
-                    E ca = rowp[q], cb = rowp[q + 1];
-                    E va[NBK], vb[NBK];
-#pragma unroll
-                    for (int k = 0; k < NBK; ++k)
-                        if (k < nb) { va[k] = qa[k]; vb[k] = qb[k]; }
-#pragma unroll
-                    for (int k = 0; k < NBK; ++k)
-                        if (k < nb) {
-                            csub_mul_conj(ca, x[s][k], va[k]);
-                            csub_mul_conj(cb, x[s][k], vb[k]);
-                        }
-                    rowp[q] = ca;
-                    rowp[q + 1] = cb;
-                }
-                if (q <= r) {
-                    const E* qrow = Lm + tri(q, 0) + j0;
-                    E cur = rowp[q];
-#pragma unroll
-                    for (int k = 0; k < NBK; ++k)
-                        if (k < nb) csub_mul_conj(cur, x[s][k], qrow[k]);
-                    rowp[q] = cur;
-                }
-            }
-        }
-        }
-    }
-    __syncwarp();
-    return true;
-}
-
-// Column-oriented triangular solves with the right-hand side spread over the
-// lanes: row p lives in slot p / 32 of lane p % 32.  L z = b, then L^H x = z.
-template <typename E, typename S, int NS>
-__device__ __forceinline__ void warp_chol_solve(const E* Lm, int D, E (&bv)[NS], int lane)
-{
-#pragma unroll
-    for (int slot = 0; slot < NS; ++slot) {
-        for (int owner = 0; owner < 32; ++owner) {
-            const int p = slot * 32 + owner;
-            if (p >= D) break;
-            E zp;
-            zp.x = __shfl_sync(0xffffffffu, bv[slot].x, owner);
-            zp.y = __shfl_sync(0xffffffffu, bv[slot].y, owner);
-            const S inv = Lm[tri(p, p)].y;
-            zp.x *= inv;
-            zp.y *= inv;
-            if (lane == owner) bv[slot] = zp;
-#pragma unroll
-            for (int s = 0; s < NS; ++s) {
-                const int q = lane + 32 * s;
-                if (q > p && q < D) {
-                    const E l = Lm[tri(q, p)];
-                    bv[s].x -= l.x * zp.x - l.y * zp.y;
-                    bv[s].y -= l.x * zp.y + l.y * zp.x;
-                }
-            }
-        }
-    }
-#pragma unroll
-    for (int slot = NS - 1; slot >= 0; --slot) {
-        for (int owner = 31; owner >= 0; --owner) {
-            const int p = slot * 32 + owner;
-            if (p >= D) continue;
-            E xp;
-            xp.x = __shfl_sync(0xffffffffu, bv[slot].x, owner);
-            xp.y = __shfl_sync(0xffffffffu, bv[slot].y, owner);
-            const S inv = Lm[tri(p, p)].y;
-            xp.x *= inv;
-            xp.y *= inv;
-            if (lane == owner) bv[slot] = xp;
-#pragma unroll
-            for (int s = 0; s < NS; ++s) {
-                const int q = lane + 32 * s;
-                if (q < p) {
-                    const E l = Lm[tri(p, q)];   // conj(l) * xp
-                    bv[s].x -= l.x * xp.x + l.y * xp.y;
-                    bv[s].y -= l.x * xp.y - l.y * xp.x;
-                }
-            }
-        }
-    }
-}
-
-// Left environment update of slice k: h_{m+1}(e) = h_m(e)^T Z^{m+1}(k) for the
-// slice's entries (lanes over entries), scattered into order m+1.
-template <typename T, int R>
-__device__ __forceinline__ void slice_h_update(const typename cvec<T>::type* __restrict__ H,
-                                               const typename cvec<T>::type* zt_s, const int32_t* __restrict__ nxt,
-                                               typename cvec<T>::type* __restrict__ Hn, int s0, int s1, int lane)
-{
-    typedef typename cvec<T>::type V;
-    constexpr bool VEC = sizeof(V) == 8 && R % 2 == 0;   // rows as 16-byte vectors
-    auto load_row = [&](int p, V* h) {
-        if constexpr (VEC) {
-            const float4* src = reinterpret_cast<const float4*>(H + (size_t)p * R);
-#pragma unroll
-            for (int a = 0; a < R / 2; ++a) {
-                const float4 v = __ldg(src + a);
-                h[2 * a].x = v.x; h[2 * a].y = v.y;
-                h[2 * a + 1].x = v.z; h[2 * a + 1].y = v.w;
-            }
-        } else {
-#pragma unroll
-            for (int a = 0; a < R; ++a) h[a] = H[(size_t)p * R + a];
-        }
-    };
-    auto store_row = [&](size_t o, const V* x) {
-        if constexpr (VEC) {
-            float4* dst = reinterpret_cast<float4*>(Hn + o);
-#pragma unroll
-            for (int a = 0; a < R / 2; ++a) dst[a] = make_float4(x[2 * a].x, x[2 * a].y, x[2 * a + 1].x, x[2 * a + 1].y);
-        } else {
-#pragma unroll
-            for (int a = 0; a < R; ++a) Hn[o + a] = x[a];
-        }
-    };
-    // two entries per lane and step: both loads are in flight together
-    for (int p = s0 + lane; p < s1; p += 64) {
-        const int p2 = p + 32;
-        const bool two = p2 < s1;
-        V h[R], g[R];
-        load_row(p, h);
-        if (two) load_row(p2, g);
-        else
-#pragma unroll
-            for (int a = 0; a < R; ++a) g[a] = czero<V>();
-        const size_t o = (size_t)nxt[p] * R;
-        const size_t o2 = two ? (size_t)nxt[p2] * R : 0;
-        V r1[R], r2[R];
-#pragma unroll
-        for (int c = 0; c < R; ++c) {
-            V acc2 = czero<V>(), acc3 = czero<V>();
-#pragma unroll
-            for (int a = 0; a < R; ++a) {
-                const V z = zt_s[a * R + c];
-                cmac(acc2, h[a], z);
-                cmac(acc3, g[a], z);
-            }
-            r1[c] = acc2;
-            r2[c] = acc3;
-        }
-        store_row(o, r1);
-        if (two) store_row(o2, r2);
-    }
-}
-
-template <typename T, int R> struct SolveCfg {
-    static constexpr int D = R * R;
-    static constexpr int NPK = D * (D + 1) / 2;
-    static constexpr int NS = (D + 31) / 32;
-    static constexpr bool MIXED = sizeof(T) == 4;
-    // per warp: factor (compute type, padded to 16 bytes), FP64 solution
-    // vector, new slice (compute type)
-    static constexpr size_t LBYTES = ((size_t)NPK * sizeof(typename cvec<T>::type) + 15) / 16 * 16;
-    static constexpr size_t WCORE = (LBYTES + (size_t)D * sizeof(double2) +
-                                     (size_t)D * sizeof(typename cvec<T>::type) + (size_t)D * sizeof(T) + 15) /
-                                    16 * 16;
-    // + one mbarrier per warp (the bulk copy of the record), padded to 16 bytes
-    static constexpr size_t WBYTES = WCORE + 16;
-    static constexpr int WPB0 = (int)((96 * 1024) / WBYTES);
-    static constexpr int WPB = WPB0 < 1 ? 1 : (WPB0 > 4 ? 4 : WPB0);
-    static constexpr size_t SMEM = WBYTES * WPB;
-    // CTAs per SM the register budget of k_mid_solve targets (bounded by shared memory)
-    static constexpr int MINB0 = (int)((227 * 1024) / SMEM);
-    static constexpr int MINB = MINB0 < 1 ? 1 : (MINB0 > 3 ? 3 : MINB0);
-};
-
-// Middle level m, stage 2 (solve + left update): one warp per slice.
-// Precision form (float): the slice's K block arrives in shared memory by one
-// bulk copy; complex64 Cholesky of the Jacobi-equilibrated S (K + lambda I) S,
-// complex64 solve, then up to three steps of iterative refinement: the
-// residual y - (K + lambda I) s is formed in double-float arithmetic
-// (TwoSum-compensated float pairs, rows spread over the lanes) against a
-// solution kept as a double-float pair, and the correction goes through the
-// complex64 factor.  If the factorization breaks down or the refinement does
-// not contract, the slice goes on a list for the FP64 Cholesky of
-// k_mid_fallback.  FP64 path (double): FP64 Cholesky directly.  The slice is
-// written row-major in FP64 and the compute type; then
-// h_{m+1}(e) = h_m(e)^T Z^{m+1}(k) for the slice's entries is scattered into
-// order m+1.  A singular system keeps its old slice.
-template <typename T, int R>
-__global__ void __launch_bounds__(32 * SolveCfg<T, R>::WPB, SolveCfg<T, R>::MINB)
-k_mid_solve(const typename cvec<T>::type* __restrict__ rec, const typename cvec<T>::type* __restrict__ H,
-            const int32_t* __restrict__ seg, const int32_t* __restrict__ nxt,
-            typename cvec<T>::type* __restrict__ Hn, double2* __restrict__ Zd,
-            typename cvec<T>::type* __restrict__ Zt, double2* __restrict__ fb, double lambda_in, double ridge,
-            unsigned long long* __restrict__ nsing, unsigned long long* __restrict__ nfb,
-            unsigned long long* __restrict__ nsteps, int32_t* __restrict__ fblist, int S,
-            unsigned long long* __restrict__ terr, int skip_copy)
-{
-    // nfb: slices handed to the FP64 fallback (length of fblist); nsteps: refinement steps;
-    // terr: raised when the bulk copy of a record does not complete within the wait limit;
-    // skip_copy (failure injection of the tests, bfc_inject_fault): the bulk copies are not
-    // issued and the waits give up after a few tries
-    typedef typename cvec<T>::type V;
-    typedef SolveCfg<T, R> C;
-    constexpr int D = C::D, NPK = C::NPK, NS = C::NS;
-    extern __shared__ __align__(16) unsigned char smem[];
-    const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
-    unsigned char* base = smem + (size_t)wib * C::WBYTES;
-    V* Lm = (V*)base;
-    double2* s_d = (double2*)(base + C::LBYTES);
-    V* zt_s = (V*)(s_d + D);
-    T* sc_s = (T*)(zt_s + D);  // Jacobi scaling of the complex64 factorization
-    // The record's K block reaches shared memory by one bulk copy (the copy
-    // engine, completion counted on a per-warp mbarrier) in the precision
-    // form; the wait is bounded.
-    const uint32_t bar = (uint32_t)__cvta_generic_to_shared(base + C::WCORE);
-    constexpr uint32_t KBULK = (uint32_t)((NPK & ~1) * sizeof(V));   // a multiple of 16 bytes
-    constexpr bool BULK = C::MIXED && KBULK >= 16;
-    uint32_t phase = 0;
-    // warp-uniform: bulk copies still in use (cleared for good when a wait
-    // expires); pending: a copy that was issued and then given up on
-    bool use_bulk = BULK;
-    bool pending = false;
-    uint32_t pending_phase = 0;
-    const uint32_t wait_limit = skip_copy ? 64u : (1u << 22);
-    if constexpr (BULK) {
-        if (lane == 0) {
-            asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(bar));
-            asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
-        }
-        __syncwarp();
-    }
-
-    for (int k = blockIdx.x * C::WPB + wib; k < S; k += gridDim.x * C::WPB) {
-        const V* K = rec + (size_t)k * (NPK + D);
-        __syncwarp();
-        bool have = false;
-        if constexpr (BULK) {
-            if (use_bulk) {
-                // the record stride D (D + 3) / 2 is even for D = r^2, so every
-                // record starts on a 16-byte boundary; the previous slice's
-                // accesses to the factor area are ordered before the copy
-                asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-                __syncwarp();
-                if (lane == 0) {
-                    asm volatile("{\n.reg .b64 st;\nmbarrier.arrive.expect_tx.shared::cta.b64 st, [%0], %1;\n}\n"
-                                 ::"r"(bar), "r"(KBULK) : "memory");
-                    if (!skip_copy)
-                        asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];"
-                                     ::"r"((uint32_t)__cvta_generic_to_shared(Lm)), "l"(K), "r"(KBULK), "r"(bar)
-                                     : "memory");
-                }
-                if ((NPK & 1) && lane == 0) Lm[NPK - 1] = K[NPK - 1];
-                bool done = false;
-                for (uint32_t it = 0; it < wait_limit && !done; ++it) {
-                    uint32_t ok;
-                    asm volatile("{\n.reg .pred p;\nmbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2, 1000;\n"
-                                 "selp.u32 %0, 1, 0, p;\n}\n"
-                                 : "=r"(ok) : "r"(bar), "r"(phase) : "memory");
-                    done = ok != 0;
-                }
-                // the phase completes once for all lanes: any lane that saw it
-                // completed makes the copy valid for the warp
-                done = __any_sync(0xffffffffu, done);
-                if (done) {
-                    have = true;
-                } else {
-                    // the copy did not complete: report it, issue no further
-                    // copies on this barrier and load by plain loads from here
-                    // on (the call's results are undefined)
-                    if (lane == 0) atomicExch(terr, 1ull);
-                    use_bulk = false;
-                    pending = !skip_copy;
-                    pending_phase = phase;
-                }
-                phase ^= 1u;
-            }
-        }
-        if (!have) {
-            if constexpr (C::MIXED) {
-                const float4* src = reinterpret_cast<const float4*>(K);
-                float4* dst = reinterpret_cast<float4*>(Lm);
-#pragma unroll 4
-                for (int q = lane; q < NPK / 2; q += 32) dst[q] = src[q];
-                if ((NPK & 1) && lane == 0) Lm[NPK - 1] = K[NPK - 1];
-            } else {
-                for (int q = lane; q < NPK; q += 32) Lm[q] = K[q];
-            }
-        }
-        __syncwarp();
-        double tr = 0.0;
-        for (int p = lane; p < D; p += 32) tr += (double)Lm[tri(p, p)].x;
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) tr += __shfl_xor_sync(0xffffffffu, tr, o);
-        // lambda, raised to the ridge floor (relative to the mean diagonal) when set
-        const double lambda = fmax(lambda_in, ridge * tr / D);
-        const double tol = lambda > 0.0 ? 0.0 : 1e-14 * (tr + D * lambda);
-        if constexpr (C::MIXED) {
-            // equilibrate: factor S (K + lambda I) S with S = diag(K_pp + lambda)^(-1/2)
-            for (int p = lane; p < D; p += 32) {
-                const T dp = Lm[tri(p, p)].x + (T)lambda;
-                sc_s[p] = dp > (T)0 ? rsqrt(dp) : (T)1;
-            }
-            __syncwarp();
-#pragma unroll
-            for (int s = 0; s < NS; ++s) {
-                const int r = owned_row(s, lane);
-                if (r < D) {
-                    V* rowp = Lm + tri(r, 0);
-                    const T sr = sc_s[r];
-                    for (int q = 0; q <= r; ++q) {
-                        V v = rowp[q];
-                        if (q == r) v.x += (T)lambda;
-                        const T f = sr * sc_s[q];
-                        v.x *= f;
-                        v.y *= f;
-                        rowp[q] = v;
-                    }
-                }
-            }
-        } else {
-            for (int p = lane; p < D; p += 32) Lm[tri(p, p)].x += (T)lambda;
-        }
-        __syncwarp();
-        double2 sv[NS];
-        bool ok;
-        if constexpr (C::MIXED) {
-            bool conv = false;
-            if (warp_chol<V, T, NS>(Lm, D, (T)tol, lane)) {
-                V bv[NS];
-                T scl[NS];
-#pragma unroll
-                for (int s = 0; s < NS; ++s) {
-                    const int p = lane + 32 * s;
-                    scl[s] = p < D ? sc_s[p] : (T)0;
-                    bv[s] = p < D ? K[NPK + p] : czero<V>();
-                    bv[s].x *= scl[s];
-                    bv[s].y *= scl[s];
-                }
-                warp_chol_solve<V, T, NS>(Lm, D, bv, lane);
-                // solution as a double-float pair (hi, lo) per component
-                float2 sh[NS], sl[NS];
-#pragma unroll
-                for (int s = 0; s < NS; ++s) {
-                    sh[s] = make_float2(bv[s].x * scl[s], bv[s].y * scl[s]);
-                    sl[s] = make_float2(0.f, 0.f);
-                }
-                float4* s_df = reinterpret_cast<float4*>(s_d);  // {re_hi, im_hi, re_lo, im_lo} per row
-                const float lamf = (float)lambda;
-                float dmax = 0.f, smax = 0.f;
-                for (int it = 0; it < 3; ++it) {
-                    // residual r = y - (K + lambda I) s in double-float arithmetic, rows over the lanes
-                    __syncwarp();
-#pragma unroll
-                    for (int s = 0; s < NS; ++s) {
-                        const int p = lane + 32 * s;
-                        if (p < D) s_df[p] = make_float4(sh[s].x, sh[s].y, sl[s].x, sl[s].y);
-                    }
-                    __syncwarp();
-                    // one pass over q for all rows of the lane: s_q is read once
-                    // for them, and K_pq comes from the stored lower triangle
-                    // (conjugated above the diagonal), so no lane idles
-                    // packed double-float accumulators: (re, im) of hi and of lo
-                    uint64_t ahi[NS], alo[NS];
-#pragma unroll
-                    for (int s = 0; s < NS; ++s) {
-                        const int p = lane + 32 * s;
-                        ahi[s] = 0ull;
-                        alo[s] = 0ull;
-                        if (p < D) {
-                            const V yp = K[NPK + p];
-                            ahi[s] = c2pack(yp.x, yp.y);
-                            df2_sub_cmul(ahi[s], alo[s], make_float2(lamf, 0.f), df2_prep(sh[s], sl[s]));
-                        }
-                    }
-                    // K_pq for 8 columns are fetched (from L2) before their products
-                    constexpr int QB = 8;
-                    for (int q0 = 0; q0 < D; q0 += QB) {
-                        V kv[NS][QB];
-#pragma unroll
-                        for (int i = 0; i < QB; ++i) {
-                            const int q = q0 + i;
-#pragma unroll
-                            for (int s = 0; s < NS; ++s) {
-                                const int p = lane + 32 * s;
-                                kv[s][i] = czero<V>();
-                                if (p < D && q < D) {
-                                    const bool lo = q <= p;
-                                    kv[s][i] = K[lo ? tri(p, q) : tri(q, p)];
-                                    if (!lo) kv[s][i].y = -kv[s][i].y;
-                                }
-                            }
-                        }
-#pragma unroll
-                        for (int i = 0; i < QB; ++i) {
-                            const int q = q0 + i;
-                            if (q < D) {
-                                const float4 sq = s_df[q];
-                                const DfS2 sp = df2_prep(make_float2(sq.x, sq.y), make_float2(sq.z, sq.w));
-#pragma unroll
-                                for (int s = 0; s < NS; ++s)
-                                    if (lane + 32 * s < D) df2_sub_cmul(ahi[s], alo[s], kv[s][i], sp);
-                            }
-                        }
-                    }
-                    float rr[NS][2];
-                    float rmax = 0.f;
-#pragma unroll
-                    for (int s = 0; s < NS; ++s) {
-                        c2unpack(c2add(ahi[s], alo[s]), rr[s][0], rr[s][1]);
-                        rmax = fmaxf(rmax, fmaxf(fabsf(rr[s][0]), fabsf(rr[s][1])));
-                    }
-#pragma unroll
-                    for (int o = 16; o > 0; o >>= 1) rmax = fmaxf(rmax, __shfl_xor_sync(0xffffffffu, rmax, o));
-                    const float sc = rmax > 0.f ? rmax : 1.f;
-                    const float isc = 1.f / sc;
-#pragma unroll
-                    for (int s = 0; s < NS; ++s) {
-                        bv[s].x = rr[s][0] * isc * scl[s];
-                        bv[s].y = rr[s][1] * isc * scl[s];
-                    }
-                    warp_chol_solve<V, T, NS>(Lm, D, bv, lane);
-                    dmax = 0.f;
-                    smax = 0.f;
-#pragma unroll
-                    for (int s = 0; s < NS; ++s) {
-                        const float dx = bv[s].x * scl[s] * sc, dy = bv[s].y * scl[s] * sc;
-                        float t, e;
-                        two_sum(sh[s].x, dx, t, e); sh[s].x = t; sl[s].x += e;
-                        two_sum(sh[s].y, dy, t, e); sh[s].y = t; sl[s].y += e;
-                        dmax = fmaxf(dmax, fmaxf(fabsf(dx), fabsf(dy)));
-                        smax = fmaxf(smax, fmaxf(fabsf(sh[s].x), fabsf(sh[s].y)));
-                    }
-#pragma unroll
-                    for (int o = 16; o > 0; o >>= 1) {
-                        dmax = fmaxf(dmax, __shfl_xor_sync(0xffffffffu, dmax, o));
-                        smax = fmaxf(smax, __shfl_xor_sync(0xffffffffu, smax, o));
-                    }
-                    if (lane == 0) atomicAdd(nsteps, 1ull);
-                    // after a step with relative correction rho the remaining error is
-                    // about rho^2: stop once that is below 1e-10
-                    if (dmax <= 1e-5f * smax) break;
-                }
-#pragma unroll
-                for (int s = 0; s < NS; ++s)
-                    sv[s] = make_double2((double)sh[s].x + (double)sl[s].x, (double)sh[s].y + (double)sl[s].y);
-                conv = dmax <= 1e-4 * smax;
-            }
-            ok = conv;
-            if (!conv) {
-                // solved afterwards in FP64 by k_mid_fallback (slice and its entries untouched here)
-                if (lane == 0) fblist[atomicAdd(nfb, 1ull)] = k;
-                continue;
-            }
-        } else {
-            ok = warp_chol<V, T, NS>(Lm, D, (T)tol, lane);
-            if (ok) {
-#pragma unroll
-                for (int s = 0; s < NS; ++s) {
-                    const int p = lane + 32 * s;
-                    sv[s] = p < D ? to_d2(K[NPK + p]) : make_double2(0.0, 0.0);
-                }
-                warp_chol_solve<V, T, NS>(Lm, D, sv, lane);
-            }
-        }
-        if (!ok && lane == 0) atomicAdd(nsing, 1ull);
-        __syncwarp();
-#pragma unroll
-        for (int s = 0; s < NS; ++s) {
-            const int p = lane + 32 * s;
-            if (p < D) {
-                if (ok) {
-                    Zd[(size_t)k * D + p] = sv[s];
-                    const V st = from_d2<V>(sv[s]);
-                    Zt[(size_t)k * D + p] = st;
-                    zt_s[p] = st;
-                } else {
-                    zt_s[p] = Zt[(size_t)k * D + p];
-                }
-            }
-        }
-        __syncwarp();
-        // left environment update into the next order
-        slice_h_update<T, R>(H, zt_s, nxt, Hn, seg[k], seg[k + 1], lane);
-    }
-    if (pending) {
-        // a copy that was given up on may still land: wait for it (bounded)
-        // before the warp's shared memory is released
-        for (uint32_t it = 0; it < (1u << 22); ++it) {
-            uint32_t ok;
-            asm volatile("{\n.reg .pred p;\nmbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2, 1000;\n"
-                         "selp.u32 %0, 1, 0, p;\n}\n"
-                         : "=r"(ok) : "r"(bar), "r"(pending_phase) : "memory");
-            if (ok) break;
-        }
-    }
-}
-
-// FP64 fallback of the precision form: one warp per slice listed by
-// k_mid_solve (complex64 factorization broke down or refinement did not
-// contract): FP64 Cholesky of K + lambda I in the slice's FP64 record, solve,
-// slice write (or keep the old slice and count it singular), left update.
-template <typename T, int R>
-__global__ void __launch_bounds__(32 * SolveCfg<T, R>::WPB)
-k_mid_fallback(const typename cvec<T>::type* __restrict__ rec, const typename cvec<T>::type* __restrict__ H,
-               const int32_t* __restrict__ seg, const int32_t* __restrict__ nxt,
-               typename cvec<T>::type* __restrict__ Hn, double2* __restrict__ Zd,
-               typename cvec<T>::type* __restrict__ Zt, double2* __restrict__ fb, double lambda_in, double ridge,
-               unsigned long long* __restrict__ nsing, const unsigned long long* __restrict__ nfb,
-               const int32_t* __restrict__ fblist, unsigned long long* __restrict__ nfb_sweep)
-{
-    typedef typename cvec<T>::type V;
-    typedef SolveCfg<T, R> C;
-    constexpr int D = C::D, NPK = C::NPK, NS = C::NS;
-    extern __shared__ __align__(16) unsigned char smem[];
-    const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
-    V* zt_s = (V*)(smem + (size_t)wib * C::WBYTES);
-    const long long count = (long long)*nfb;
-    // the level's fallbacks join the sweep's count (one thread; nothing else
-    // writes it while this kernel runs)
-    if (blockIdx.x == 0 && threadIdx.x == 0) *nfb_sweep += (unsigned long long)count;
-    for (long long idx = (long long)blockIdx.x * C::WPB + wib; idx < count; idx += (long long)gridDim.x * C::WPB) {
-        const int k = fblist[idx];
-        const V* K = rec + (size_t)k * (NPK + D);
-        double tr = 0.0;
-        for (int p = lane; p < D; p += 32) tr += (double)K[tri(p, p)].x;
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) tr += __shfl_xor_sync(0xffffffffu, tr, o);
-        const double lambda = fmax(lambda_in, ridge * tr / D);
-        const double tol = lambda > 0.0 ? 0.0 : 1e-14 * (tr + D * lambda);
-        double2* Kd = fb + (size_t)k * NPK;
-        __syncwarp();
-        for (int q = lane; q < NPK; q += 32) Kd[q] = to_d2(K[q]);
-        __syncwarp();
-        for (int p = lane; p < D; p += 32) Kd[tri(p, p)].x += lambda;
-        double2 sv[NS];
-        const bool ok = warp_chol<double2, double, NS>(Kd, D, tol, lane);
-        if (ok) {
-#pragma unroll
-            for (int s = 0; s < NS; ++s) {
-                const int p = lane + 32 * s;
-                sv[s] = p < D ? to_d2(K[NPK + p]) : make_double2(0.0, 0.0);
-            }
-            warp_chol_solve<double2, double, NS>(Kd, D, sv, lane);
-        } else if (lane == 0) {
-            atomicAdd(nsing, 1ull);
-        }
-        __syncwarp();
-#pragma unroll
-        for (int s = 0; s < NS; ++s) {
-            const int p = lane + 32 * s;
-            if (p < D) {
-                if (ok) {
-                    Zd[(size_t)k * D + p] = sv[s];
-                    const V st = from_d2<V>(sv[s]);
-                    Zt[(size_t)k * D + p] = st;
-                    zt_s[p] = st;
-                } else {
-                    zt_s[p] = Zt[(size_t)k * D + p];
-                }
-            }
-        }
-        __syncwarp();
-        slice_h_update<T, R>(H, zt_s, nxt, Hn, seg[k], seg[k + 1], lane);
     }
 }
 

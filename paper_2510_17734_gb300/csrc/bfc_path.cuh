@@ -6,6 +6,7 @@
 #include "bfc_gram_tc.cuh"
 #include "bfc_internal.h"
 #include "bfc_kernels.cuh"
+#include "bfc_solve.cuh"
 #include "bfc_util.h"
 
 namespace bfc {
@@ -62,7 +63,7 @@ template <typename T, int R> struct Path {
                                      (int)SolveCfg<T, R>::SMEM);
         if (e == cudaSuccess)
             e = cudaFuncSetAttribute(k_mid_fallback<T, R>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                     (int)SolveCfg<T, R>::SMEM);
+                                     (int)SolveCfg<double, R>::SMEM);
         if (e == cudaSuccess && TC) e = set_tc_attr();
         if (e == cudaSuccess && GRP) e = set_grp_attr();
         if (e != cudaSuccess)
@@ -71,16 +72,12 @@ template <typename T, int R> struct Path {
     }
 
     // Bytes of the per-block normal-equation records (the larger of the
-    // middle-slice and the outer-fiber layouts) and of the FP64 fallback area.
+    // middle-slice and the outer-fiber layouts).
     static size_t record_bytes(int64_t n, int64_t S)
     {
-        const size_t mid = (size_t)S * (GramCfg<T, R>::NPK + R * R) * sizeof(V);
+        const size_t mid = (size_t)S * Rec<T, R>::SIZE * sizeof(T);
         const size_t outer = (size_t)n * (R * (R + 1) / 2 + R) * sizeof(double2);
         return mid > outer ? mid : outer;
-    }
-    static size_t fallback_bytes(int64_t S)
-    {
-        return SolveCfg<T, R>::MIXED ? (size_t)S * SolveCfg<T, R>::NPK * sizeof(double2) : 0;
     }
 
     // Bytes of one group record of the grouped Gram (0: no grouped Gram).
@@ -150,7 +147,6 @@ template <typename T, int R> struct Path {
         BFC_TRY(outer_level<false>(c, W, 0, c->z1d, (V*)c->z1t, H0));
         typedef GramCfg<T, R> GC;
         typedef SolveCfg<T, R> SC;
-        const unsigned gsolve = (unsigned)((S + SC::WPB - 1) / SC::WPB);
         for (int m = 1; m <= L; ++m) {
             V* hin = (m - 1) & 1 ? H1 : H0;
             V* hout = m & 1 ? H1 : H0;
@@ -177,10 +173,10 @@ template <typename T, int R> struct Path {
                         }
                         if (gl.by_col)
                             k_mid_gram_grp<T, RG, 1><<<(unsigned)S * GrpCfg<T, RG>::NSPLIT, GrpCfg<T, RG>::NTH, GrpCfg<T, RG>::SMEM,
-                                                       c->stream>>>((const V*)c->grec, gl.gseg, (V*)c->rec, (int)S);
+                                                       c->stream>>>((const V*)c->grec, gl.gseg, (T*)c->rec, (int)S);
                         else
                             k_mid_gram_grp<T, RG, 0><<<(unsigned)S * GrpCfg<T, RG>::NSPLIT, GrpCfg<T, RG>::NTH, GrpCfg<T, RG>::SMEM,
-                                                       c->stream>>>((const V*)c->grec, gl.gseg, (V*)c->rec, (int)S);
+                                                       c->stream>>>((const V*)c->grec, gl.gseg, (T*)c->rec, (int)S);
                         ps.add_kernels(1);
                         done = true;
                     }
@@ -190,30 +186,31 @@ template <typename T, int R> struct Path {
                         const unsigned g = (unsigned)(S < c->num_sms ? S : c->num_sms);
                         k_mid_gram_tc<TC ? R : 1><<<g, TcGram::NTH, TcGram::SMEM, c->stream>>>(
                             (const float2*)hin, (const float2*)(W + (size_t)m * NR), (const float2*)c->tval[m],
-                            c->seg[m], (float2*)c->rec, (int)S, c->d_count + 5);
+                            c->seg[m], (float*)c->rec, (int)S, c->d_count + 5);
                         done = true;
                     }
                 }
                 if (!done)
                     k_mid_gram<T, R><<<(unsigned)S, GC::NTH, GC::SMEM, c->stream>>>(
-                        hin, W + (size_t)m * NR, (const V*)c->tval[m], c->seg[m], (V*)c->rec, (int)S);
+                        hin, W + (size_t)m * NR, (const V*)c->tval[m], c->seg[m], (T*)c->rec, (int)S);
             }
             {
                 ProfScope ps(c, "mid_solve");
                 if (SC::MIXED) cudaMemsetAsync(c->d_count + 3, 0, sizeof(unsigned long long), c->stream);
-                k_mid_solve<T, R><<<gsolve, 32 * SC::WPB, SC::SMEM, c->stream>>>(
-                    (const V*)c->rec, hin, c->seg[m], c->nxt[m], hout, c->Zd + (size_t)(m - 1) * S * R * R,
-                    (V*)c->Zt + (size_t)(m - 1) * S * R * R, c->fb, c->P.lambda, c->ridge, c->d_count,
-                    c->d_count + 3, c->d_count + 2, c->fblist, (int)S, c->d_count + 5, c->inject == 1 ? 1 : 0);
+                k_mid_solve<T, R><<<(unsigned)S, SC::NTH, SC::SMEM, c->stream>>>(
+                    (const T*)c->rec, hin, c->seg[m], c->nxt[m], hout, c->Zd + (size_t)(m - 1) * S * R * R,
+                    (V*)c->Zt + (size_t)(m - 1) * S * R * R, c->P.lambda, c->ridge, c->d_count,
+                    c->d_count + 3, c->d_count + 2, c->fblist, c->d_count + 5, c->inject == 1 ? 1 : 0);
             }
             if (SC::MIXED) {
                 ProfScope ps(c, "mid_fallback");
-                // a grid-stride loop over the listed slices (usually none): one
-                // wave of blocks at most
-                const unsigned gfb = std::min<unsigned>(gsolve, (unsigned)c->num_sms * SC::MINB);
-                k_mid_fallback<T, R><<<gfb, 32 * SC::WPB, SC::SMEM, c->stream>>>(
-                    (const V*)c->rec, hin, c->seg[m], c->nxt[m], hout, c->Zd + (size_t)(m - 1) * S * R * R,
-                    (V*)c->Zt + (size_t)(m - 1) * S * R * R, c->fb, c->P.lambda, c->ridge, c->d_count,
+                // a loop over the listed slices (usually none): about one wave of blocks
+                typedef SolveCfg<double, R> FC;
+                const int per_sm = (int)std::min<size_t>(8, std::max<size_t>(1, 227 * 1024 / (FC::SMEM + 1024)));
+                const unsigned gfb = (unsigned)std::min<int64_t>(S, (int64_t)c->num_sms * per_sm);
+                k_mid_fallback<T, R><<<gfb, FC::FBT, FC::SMEM, c->stream>>>(
+                    (const T*)c->rec, hin, c->seg[m], c->nxt[m], hout, c->Zd + (size_t)(m - 1) * S * R * R,
+                    (V*)c->Zt + (size_t)(m - 1) * S * R * R, c->P.lambda, c->ridge, c->d_count,
                     c->d_count + 3, c->fblist, c->d_count + 1);   // + the fallbacks of the sweep
             }
         }
