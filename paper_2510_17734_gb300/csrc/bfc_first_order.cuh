@@ -45,20 +45,49 @@ template <typename A, int R> __device__ __forceinline__ A pick(const A (&arr)[R]
     return out;
 }
 
+// Entries base .. base + cnt of a level into shared memory: the rows of H as
+// they are, the rows of W as r conj(w).  128 threads, contiguous loads.
+template <typename T, int R>
+__device__ __forceinline__ void stage_rows(const typename cvec<T>::type* __restrict__ H,
+                                           const typename cvec<T>::type* __restrict__ Wm,
+                                           const typename cvec<T>::type* __restrict__ Rc, int base, int cnt,
+                                           typename cvec<T>::type* h_s, typename cvec<T>::type* w_s, int tid)
+{
+    typedef typename cvec<T>::type V;
+    if constexpr (sizeof(V) == 8 && R % 2 == 0) {
+        const float4* h4 = reinterpret_cast<const float4*>(H + (size_t)base * R);
+        const float4* w4 = reinterpret_cast<const float4*>(Wm + (size_t)base * R);
+        for (int x = tid; x < cnt * (R / 2); x += 128) {
+            const float4 w = w4[x];
+            const V r = Rc[base + x / (R / 2)];
+            reinterpret_cast<float4*>(h_s)[x] = h4[x];
+            reinterpret_cast<float4*>(w_s)[x] =
+                make_float4(w.x * r.x + w.y * r.y, w.x * r.y - w.y * r.x, w.z * r.x + w.w * r.y, w.z * r.y - w.w * r.x);
+        }
+    } else {
+        for (int x = tid; x < cnt * R; x += 128) {
+            V rw = czero<V>();
+            cmacc(rw, Wm[(size_t)base * R + x], Rc[base + x / R]);
+            h_s[x] = H[(size_t)base * R + x];
+            w_s[x] = rw;
+        }
+    }
+}
+
 // ------------------------------------------------------------------ ADAM
 
 // Outer factor of Alg. 4 (rows: S^1 with design w_0; columns: S^{L+2} with
 // design h_{L+1}), one warp per fiber: gradient sum (x - t) conj(a) +
 // lambda s at the current fiber, the Alg. 3 update, then (rows) h_1 = the new
-// fiber into order 1 or (columns) the training residual partials with the
-// new fiber.
+// fiber and the residual h_1^T w_0 - t into order 1 or (columns) the training
+// residual partials with the new fiber.
 template <typename T, int R, bool COLS>
 __global__ void __launch_bounds__(256)
 k_adam_outer(const typename cvec<T>::type* __restrict__ A, const typename cvec<T>::type* __restrict__ tv,
              const int32_t* __restrict__ seg, int nfib, double2* __restrict__ zd,
              typename cvec<T>::type* __restrict__ zt, double2* __restrict__ Mo, double2* __restrict__ Vo,
              AdamHyper hp, double lam, const int32_t* __restrict__ nxt, typename cvec<T>::type* __restrict__ Hn,
-             double* __restrict__ part)
+             typename cvec<T>::type* __restrict__ Rn, double* __restrict__ part)
 {
     typedef typename cvec<T>::type V;
     const int lane = threadIdx.x & 31;
@@ -101,8 +130,16 @@ k_adam_outer(const typename cvec<T>::type* __restrict__ A, const typename cvec<T
     if constexpr (!COLS) {
         for (int p = s0 + lane; p < s1; p += 32) {
             const size_t o = (size_t)nxt[p];
+            V a[R];
+            load_row_v<V, R>(A, (size_t)p, a);
+            V x = czero<V>();
 #pragma unroll
-            for (int c = 0; c < R; ++c) Hn[o * R + c] = s[c];
+            for (int c = 0; c < R; ++c) cmac(x, s[c], a[c]);
+            const V t = tv[p];
+            x.x -= t.x;
+            x.y -= t.y;
+            store_row_v<V, R>(Hn, o, s);
+            Rn[o] = x;
         }
     } else {
         double fit = 0.0, den = 0.0;
@@ -129,103 +166,70 @@ k_adam_outer(const typename cvec<T>::type* __restrict__ A, const typename cvec<T
     }
 }
 
-// Middle factor of Alg. 4, one CTA per slice (grid-stride): the residual of
-// every entry with the current slice, the gradient sum (x - t) conj(h (x) w)
-// + lambda Z (threads own components, chunks of entries staged in shared
-// memory), the Alg. 3 update of the slice, then h_{m+1} = h_m^T Z(new) into
-// order m+1.
+// Middle factor of Alg. 4, one CTA per slice (grid-stride): the gradient sum
+// r conj(h (x) w) + lambda Z with the carried residuals (SliceSums, chunks of
+// entries staged with w already multiplied by r), the Alg. 3 update of the
+// slice, then h_{m+1} = h_m^T Z(new) and the residual h_{m+1}^T w_m - t into
+// order m+1 (r products instead of the r^2 of h_m^T Z w_m at the next level).
 template <typename T, int R>
 __global__ void __launch_bounds__(128)
 k_adam_mid(const typename cvec<T>::type* __restrict__ H, const typename cvec<T>::type* __restrict__ Wm,
-           const typename cvec<T>::type* __restrict__ tv, const int32_t* __restrict__ seg,
-           const int32_t* __restrict__ nxt, double2* __restrict__ Zd, typename cvec<T>::type* __restrict__ Zt,
-           double2* __restrict__ Mo, double2* __restrict__ Vo, AdamHyper hp, double lam,
-           typename cvec<T>::type* __restrict__ Hn, int S)
+           const typename cvec<T>::type* __restrict__ Rc, const typename cvec<T>::type* __restrict__ tv,
+           const int32_t* __restrict__ seg, const int32_t* __restrict__ nxt, double2* __restrict__ Zd,
+           typename cvec<T>::type* __restrict__ Zt, double2* __restrict__ Mo, double2* __restrict__ Vo, AdamHyper hp,
+           double lam, typename cvec<T>::type* __restrict__ Hn, typename cvec<T>::type* __restrict__ Rn, int S)
 {
     typedef typename cvec<T>::type V;
+    typedef SliceSums<T, R, true> SS;
     constexpr int D = R * R;
     constexpr int CH = 128;
-    constexpr int NQ = (D + 127) / 128;
-    __shared__ V z_s[D];
-    __shared__ V h_s[CH * R];
-    __shared__ V w_s[CH * R];
-    __shared__ V r_s[CH];
+    constexpr size_t ROWS = (size_t)CH * R * sizeof(V) + 16;
+    __shared__ __align__(16) unsigned char buf[2 * ROWS > SS::RED ? 2 * ROWS : SS::RED];
+    __shared__ __align__(16) V z_s[D];
+    V* h_s = (V*)buf;
+    V* w_s = (V*)(buf + ROWS);
     const int tid = threadIdx.x;
     for (int k = blockIdx.x; k < S; k += gridDim.x) {
         const int s0 = seg[k], s1 = seg[k + 1];
-        __syncthreads();
-        for (int q = tid; q < D; q += blockDim.x) z_s[q] = Zt[(size_t)k * D + q];
-        double2 g[NQ];
-#pragma unroll
-        for (int u = 0; u < NQ; ++u) g[u] = make_double2(0.0, 0.0);
+        SS ss;
+        ss.start(tid);
         for (int base = s0; base < s1; base += CH) {
             const int cnt = min(CH, s1 - base);
             __syncthreads();
-            if (tid < cnt) {
-                const size_t p = (size_t)(base + tid);
-                V h[R], w[R];
-                load_row_v<V, R>(H, p, h);
-                load_row_v<V, R>(Wm, p, w);
-                V x = czero<V>();
-#pragma unroll
-                for (int a = 0; a < R; ++a) {
-                    V hz = czero<V>();
-#pragma unroll
-                    for (int c = 0; c < R; ++c) cmac(hz, z_s[a * R + c], w[c]);
-                    cmac(x, h[a], hz);
-                }
-                const V t = tv[p];
-                V rr;
-                rr.x = x.x - t.x;
-                rr.y = x.y - t.y;
-                r_s[tid] = rr;
-#pragma unroll
-                for (int c = 0; c < R; ++c) {
-                    h_s[tid * R + c] = h[c];
-                    w_s[tid * R + c] = w[c];
-                }
-            }
+            stage_rows<T, R>(H, Wm, Rc, base, cnt, h_s, w_s, tid);
             __syncthreads();
-#pragma unroll
-            for (int u = 0; u < NQ; ++u) {
-                const int q = tid + 128 * u;
-                if (q < D) {
-                    const int pa = q / R, pc = q - pa * R;
-                    V acc = czero<V>();
-                    for (int e = 0; e < cnt; ++e) cmacc(acc, cmul(h_s[e * R + pa], w_s[e * R + pc]), r_s[e]);
-                    g[u].x += (double)acc.x;
-                    g[u].y += (double)acc.y;
-                }
-            }
+            ss.chunk(h_s, w_s, nullptr, cnt);
+            if (ss.full(CH)) ss.reduce(buf, tid);
         }
-        __syncthreads();
-#pragma unroll
-        for (int u = 0; u < NQ; ++u) {
-            const int q = tid + 128 * u;
-            if (q < D) {
-                const size_t o = (size_t)k * D + q;
-                const double2 sd = Zd[o];
-                const double2 gd = make_double2(g[u].x + lam * sd.x, g[u].y + lam * sd.y);
-                const double2 ns = adam_step(sd, gd, Mo + o, Vo + o, hp);
-                Zd[o] = ns;
-                const V st = from_d2<V>(ns);
-                Zt[o] = st;
-                z_s[q] = st;
-            }
-        }
+        ss.finish(buf, tid, [&](int q, double2 g) {
+            const size_t o = (size_t)k * D + q;
+            const double2 sd = Zd[o];
+            const double2 gd = make_double2(g.x + lam * sd.x, g.y + lam * sd.y);
+            const double2 ns = adam_step(sd, gd, Mo + o, Vo + o, hp);
+            Zd[o] = ns;
+            const V st = from_d2<V>(ns);
+            Zt[o] = st;
+            z_s[q] = st;
+        });
         __syncthreads();
         for (int p = s0 + tid; p < s1; p += blockDim.x) {
-            V h[R];
+            V h[R], hn[R];
             load_row_v<V, R>(H, (size_t)p, h);
             const size_t o = (size_t)nxt[p];
+            row_times_slice<V, R>(h, z_s, hn);
+            store_row_v<V, R>(Hn, o, hn);
+            if (Rn) {
+                load_row_v<V, R>(Wm, (size_t)p, h);
+                V x = czero<V>();
 #pragma unroll
-            for (int c = 0; c < R; ++c) {
-                V acc = czero<V>();
-#pragma unroll
-                for (int a = 0; a < R; ++a) cmac(acc, h[a], z_s[a * R + c]);
-                Hn[o * R + c] = acc;
+                for (int c = 0; c < R; ++c) cmac(x, hn[c], h[c]);
+                const V t = tv[p];
+                x.x -= t.x;
+                x.y -= t.y;
+                Rn[o] = x;
             }
         }
+        __syncthreads();   // z_s is read to the end before the next slice's update
     }
 }
 
@@ -345,9 +349,10 @@ k_adf_outer(const typename cvec<T>::type* __restrict__ A, const typename cvec<T>
 }
 
 // Middle factor of Alg. 5, one CTA per slice (grid-stride): the direction
-// N = sum G conj(h (x) w) - lambda Z (threads own components), the exact
-// step alpha = ||N||^2 / (sum |h^T N w|^2 + lambda ||N||^2), Z += alpha N,
-// and the new residual G - alpha h^T N w into order m+1.
+// N = sum G conj(h (x) w) - lambda Z (SliceSums), the exact step
+// alpha = ||N||^2 / (sum |h^T N w|^2 + lambda ||N||^2), Z += alpha N,
+// and the new residual G - alpha h^T N w into order m+1.  The products
+// h^T N w of up to ZC entries of a slice are kept between the two uses.
 template <typename T, int R>
 __global__ void __launch_bounds__(128)
 k_adf_mid(const typename cvec<T>::type* __restrict__ H, const typename cvec<T>::type* __restrict__ Wm,
@@ -356,16 +361,20 @@ k_adf_mid(const typename cvec<T>::type* __restrict__ H, const typename cvec<T>::
           double lam, typename cvec<T>::type* __restrict__ Gn, int S)
 {
     typedef typename cvec<T>::type V;
+    typedef SliceSums<T, R, true> SS;
     constexpr int D = R * R;
     constexpr int CH = 128;
-    constexpr int NQ = (D + 127) / 128;
-    __shared__ V h_s[CH * R];
-    __shared__ V w_s[CH * R];
-    __shared__ V g_s[CH];
+    constexpr size_t ROWS = (size_t)CH * R * sizeof(V) + 16;
+    constexpr size_t BUF = 2 * ROWS > SS::RED ? 2 * ROWS : SS::RED;
+    constexpr int ZC = (int)(BUF / sizeof(V));   // the chunk buffer is free by then
+    __shared__ __align__(16) unsigned char buf[BUF];
     __shared__ double2 n_s[D];
     __shared__ V nt_s[D];   // the direction in the compute type, for the per-entry products
     __shared__ double red[4];
     __shared__ double alpha_s;
+    V* h_s = (V*)buf;
+    V* w_s = (V*)(buf + ROWS);
+    V* zc = (V*)buf;
     const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
     auto block_sum = [&](double v) {
 #pragma unroll
@@ -376,7 +385,10 @@ k_adf_mid(const typename cvec<T>::type* __restrict__ H, const typename cvec<T>::
         return red[0] + red[1] + red[2] + red[3];
     };
     // z_e = h^T N w in the compute type (the entry's own precision)
-    auto zval = [&](const V (&h)[R], const V (&w)[R]) {
+    auto zval = [&](int p) {
+        V h[R], w[R];
+        load_row_v<V, R>(H, (size_t)p, h);
+        load_row_v<V, R>(Wm, (size_t)p, w);
         V z = czero<V>();
 #pragma unroll
         for (int a = 0; a < R; ++a) {
@@ -385,55 +397,36 @@ k_adf_mid(const typename cvec<T>::type* __restrict__ H, const typename cvec<T>::
             for (int c = 0; c < R; ++c) cmac(nw, nt_s[a * R + c], w[c]);
             cmac(z, h[a], nw);
         }
-        return to_d2(z);
+        return z;
     };
     for (int k = blockIdx.x; k < S; k += gridDim.x) {
         const int s0 = seg[k], s1 = seg[k + 1];
-        __syncthreads();   // the previous slice's readers of n_s are done
-        double2 nq[NQ];
-#pragma unroll
-        for (int u = 0; u < NQ; ++u) nq[u] = make_double2(0.0, 0.0);
+        SS ss;
+        ss.start(tid);
         for (int base = s0; base < s1; base += CH) {
             const int cnt = min(CH, s1 - base);
             __syncthreads();
-            for (int x = tid; x < cnt * R; x += blockDim.x) {
-                h_s[x] = H[(size_t)base * R + x];
-                w_s[x] = Wm[(size_t)base * R + x];
-            }
-            for (int x = tid; x < cnt; x += blockDim.x) g_s[x] = Gin[base + x];
+            stage_rows<T, R>(H, Wm, Gin, base, cnt, h_s, w_s, tid);
             __syncthreads();
-#pragma unroll
-            for (int u = 0; u < NQ; ++u) {
-                const int q = tid + 128 * u;
-                if (q < D) {
-                    const int pa = q / R, pc = q - pa * R;
-                    V acc = czero<V>();
-                    for (int e = 0; e < cnt; ++e) cmacc(acc, cmul(h_s[e * R + pa], w_s[e * R + pc]), g_s[e]);
-                    nq[u].x += (double)acc.x;
-                    nq[u].y += (double)acc.y;
-                }
-            }
+            ss.chunk(h_s, w_s, nullptr, cnt);
+            if (ss.full(CH)) ss.reduce(buf, tid);
         }
         double nn = 0.0;
-#pragma unroll
-        for (int u = 0; u < NQ; ++u) {
-            const int q = tid + 128 * u;
-            if (q < D) {
-                const double2 sd = Zd[(size_t)k * D + q];
-                const double2 nv = make_double2(nq[u].x - lam * sd.x, nq[u].y - lam * sd.y);
-                n_s[q] = nv;
-                nt_s[q] = from_d2<V>(nv);
-                nn += nv.x * nv.x + nv.y * nv.y;
-            }
-        }
-        nn = block_sum(nn);   // its first barrier also publishes n_s
+        ss.finish(buf, tid, [&](int q, double2 g) {
+            const double2 sd = Zd[(size_t)k * D + q];
+            const double2 nv = make_double2(g.x - lam * sd.x, g.y - lam * sd.y);
+            n_s[q] = nv;
+            nt_s[q] = from_d2<V>(nv);
+            nn += nv.x * nv.x + nv.y * nv.y;
+        });
+        nn = block_sum(nn);   // its first barrier also publishes n_s and frees buf
         double zz = 0.0;
         for (int p = s0 + tid; p < s1; p += blockDim.x) {
-            V h[R], w[R];
-            load_row_v<V, R>(H, (size_t)p, h);
-            load_row_v<V, R>(Wm, (size_t)p, w);
-            const double2 z = zval(h, w);
-            zz += z.x * z.x + z.y * z.y;
+            asm volatile("" ::: "memory");   // the direction stays in shared memory, not hoisted into registers
+            const V z = zval(p);
+            if (p - s0 < ZC) zc[p - s0] = z;
+            const double2 zd = to_d2(z);
+            zz += zd.x * zd.x + zd.y * zd.y;
         }
         zz = block_sum(zz);
         if (tid == 0) {
@@ -442,25 +435,19 @@ k_adf_mid(const typename cvec<T>::type* __restrict__ H, const typename cvec<T>::
         }
         __syncthreads();
         const double alpha = alpha_s;
-#pragma unroll
-        for (int u = 0; u < NQ; ++u) {
-            const int q = tid + 128 * u;
-            if (q < D) {
-                const size_t o = (size_t)k * D + q;
-                const double2 sd = Zd[o], nv = n_s[q];
-                const double2 ns = make_double2(sd.x + alpha * nv.x, sd.y + alpha * nv.y);
-                Zd[o] = ns;
-                Zt[o] = from_d2<V>(ns);
-            }
+        for (int q = tid; q < D; q += blockDim.x) {
+            const size_t o = (size_t)k * D + q;
+            const double2 sd = Zd[o], nv = n_s[q];
+            const double2 ns = make_double2(sd.x + alpha * nv.x, sd.y + alpha * nv.y);
+            Zd[o] = ns;
+            Zt[o] = from_d2<V>(ns);
         }
         for (int p = s0 + tid; p < s1; p += blockDim.x) {
-            V h[R], w[R];
-            load_row_v<V, R>(H, (size_t)p, h);
-            load_row_v<V, R>(Wm, (size_t)p, w);
-            const double2 z = zval(h, w);
+            const double2 z = to_d2(p - s0 < ZC ? zc[p - s0] : zval(p));
             const V g = Gin[p];
             Gn[nxt[p]] = from_d2<V>(make_double2((double)g.x - alpha * z.x, (double)g.y - alpha * z.y));
         }
+        __syncthreads();   // n_s and zc are read to the end before the next slice
     }
 }
 
@@ -473,7 +460,7 @@ k_h_next(const typename cvec<T>::type* __restrict__ H, const int32_t* __restrict
          typename cvec<T>::type* __restrict__ Hn, int S)
 {
     typedef typename cvec<T>::type V;
-    __shared__ V z_s[R * R];
+    __shared__ __align__(16) V z_s[R * R];
     for (int k = blockIdx.x; k < S; k += gridDim.x) {
         const int s0 = seg[k], s1 = seg[k + 1];
         if (s0 == s1) continue;
@@ -481,16 +468,10 @@ k_h_next(const typename cvec<T>::type* __restrict__ H, const int32_t* __restrict
         for (int q = threadIdx.x; q < R * R; q += blockDim.x) z_s[q] = Zt[(size_t)k * R * R + q];
         __syncthreads();
         for (int p = s0 + threadIdx.x; p < s1; p += blockDim.x) {
-            V h[R];
+            V h[R], hn[R];
             load_row_v<V, R>(H, (size_t)p, h);
-            const size_t o = (size_t)nxt[p];
-#pragma unroll
-            for (int c = 0; c < R; ++c) {
-                V acc = czero<V>();
-#pragma unroll
-                for (int a = 0; a < R; ++a) cmac(acc, h[a], z_s[a * R + c]);
-                Hn[o * R + c] = acc;
-            }
+            row_times_slice<V, R>(h, z_s, hn);
+            store_row_v<V, R>(Hn, (size_t)nxt[p], hn);
         }
     }
 }
@@ -508,11 +489,7 @@ k_h1_rows(const int32_t* __restrict__ seg, int nfib, const typename cvec<T>::typ
     V s[R];
 #pragma unroll
     for (int c = 0; c < R; ++c) s[c] = zt[(size_t)f * R + c];
-    for (int p = seg[f] + lane; p < seg[f + 1]; p += 32) {
-        const size_t o = (size_t)nxt[p];
-#pragma unroll
-        for (int c = 0; c < R; ++c) Hn[o * R + c] = s[c];
-    }
+    for (int p = seg[f] + lane; p < seg[f + 1]; p += 32) store_row_v<V, R>(Hn, (size_t)nxt[p], s);
 }
 
 // ---------------------------------------------------------------- matvec
@@ -652,27 +629,28 @@ template <typename T, int R> struct FirstOrder {
         const double lam = c->P.lambda;
         V* W = (V*)c->W;
         V* Hb[2] = {(V*)c->H[0], (V*)c->H[1]};
+        V* Rb[2] = {(V*)c->Rres[0], (V*)c->Rres[1]};
         BFC_TRY((Path<T, R>::right_envs(c)));
         const size_t offZ = (size_t)n * R, offL = offZ + (size_t)L * S * R * R;
         {
             ProfScope ps(c, "adam_rows");
             k_adam_outer<T, R, false><<<nblocks(n, 8), 256, 0, c->stream>>>(
                 W, (const V*)c->tval[0], c->seg[0], (int)n, c->z1d, (V*)c->z1t, M, Vm, hp, lam, c->nxt[0], Hb[0],
-                nullptr);
+                Rb[0], nullptr);
         }
         for (int m = 1; m <= L; ++m) {
             ProfScope ps(c, "adam_mid");
             const size_t o = offZ + (size_t)(m - 1) * S * R * R;
             k_adam_mid<T, R><<<grid_slices(S), 128, 0, c->stream>>>(
-                Hb[(m - 1) & 1], W + (size_t)m * NR, (const V*)c->tval[m], c->seg[m], c->nxt[m],
+                Hb[(m - 1) & 1], W + (size_t)m * NR, Rb[(m - 1) & 1], (const V*)c->tval[m], c->seg[m], c->nxt[m],
                 c->Zd + (size_t)(m - 1) * S * R * R, (V*)c->Zt + (size_t)(m - 1) * S * R * R, M + o, Vm + o, hp, lam,
-                Hb[m & 1], (int)S);
+                Hb[m & 1], m < L ? Rb[m & 1] : nullptr, (int)S);
         }
         {
             ProfScope ps(c, "adam_cols");
             k_adam_outer<T, R, true><<<nblocks(n, 8), 256, 0, c->stream>>>(
                 Hb[L & 1], (const V*)c->tval[L + 1], c->seg[L + 1], (int)n, c->zLd, (V*)c->zLt, M + offL,
-                Vm + offL, hp, lam, nullptr, nullptr, c->d_red);
+                Vm + offL, hp, lam, nullptr, nullptr, nullptr, c->d_red);
         }
         BFC_LAUNCH_CHECK(c, "adam iteration");
         return BFC_OK;

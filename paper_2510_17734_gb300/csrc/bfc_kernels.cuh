@@ -1066,17 +1066,216 @@ k_grad_rows(const typename cvec<T>::type* __restrict__ W0, const typename cvec<T
     }
 }
 
+// o = h^T Z for one row h and a slice in shared memory (row-major, 16-byte
+// aligned).
+template <typename V, int R> __device__ __forceinline__ void row_times_slice(const V (&h)[R], const V* z_s, V (&o)[R])
+{
+    asm volatile("" ::: "memory");   // the slice is read here, not held in registers across entries
+    if constexpr (sizeof(V) == 8 && R % 2 == 0) {
+        // packed: h z = h.re (z.re, z.im) + h.im (-z.im, z.re), the second
+        // product taken as h.im (z.re, z.im) and turned at the end
+        uint64_t hr[R], hi[R];
+#pragma unroll
+        for (int a = 0; a < R; ++a) {
+            hr[a] = c2pack(h[a].x, h[a].x);
+            hi[a] = c2pack(h[a].y, h[a].y);
+        }
+#pragma unroll
+        for (int c = 0; c < R; c += 2) {
+            uint64_t p0 = 0ull, p1 = 0ull, q0 = 0ull, q1 = 0ull;
+#pragma unroll
+            for (int a = 0; a < R; ++a) {
+                const float4 z = *reinterpret_cast<const float4*>(z_s + a * R + c);
+                const uint64_t z0 = c2pack(z.x, z.y), z1 = c2pack(z.z, z.w);
+                p0 = c2fma(hr[a], z0, p0);
+                q0 = c2fma(hi[a], z0, q0);
+                p1 = c2fma(hr[a], z1, p1);
+                q1 = c2fma(hi[a], z1, q1);
+            }
+            float pr, pi, qr, qi;
+            c2unpack(p0, pr, pi);
+            c2unpack(q0, qr, qi);
+            o[c].x = pr - qi; o[c].y = pi + qr;
+            c2unpack(p1, pr, pi);
+            c2unpack(q1, qr, qi);
+            o[c + 1].x = pr - qi; o[c + 1].y = pi + qr;
+        }
+    } else {
+#pragma unroll
+        for (int c = 0; c < R; ++c) {
+            o[c] = czero<V>();
+#pragma unroll
+            for (int a = 0; a < R; ++a) cmac(o[c], h[a], z_s[a * R + c]);
+        }
+    }
+}
+
+// Row p of an R-column complex array (16-byte moves in complex64 at even rank).
+template <typename V, int R> __device__ __forceinline__ void store_row_v(V* __restrict__ A, size_t p, const V (&v)[R])
+{
+    if constexpr (sizeof(V) == 8 && R % 2 == 0) {
+        float4* d4 = reinterpret_cast<float4*>(A + p * R);
+#pragma unroll
+        for (int c = 0; c < R / 2; ++c) d4[c] = make_float4(v[2 * c].x, v[2 * c].y, v[2 * c + 1].x, v[2 * c + 1].y);
+    } else {
+#pragma unroll
+        for (int c = 0; c < R; ++c) A[p * R + c] = v[c];
+    }
+}
+
+// Sums over a slice's entries of r_e conj(h_e (x) w_e) (a slice's gradient or
+// descent direction) by 128 threads.  A thread owns T x T (2 x 2 from rank 3)
+// of the R x R components and every EG-th entry of a chunk in shared memory, so
+// two values of each factor feed four complex products and the threads are
+// busy at every rank.  (A component per thread left half of them idle at rank
+// 8 and two thirds at rank 6.  Tiles of 4 x 4 read less but take the registers
+// of two more blocks per SM: gradient at n = 65536 2.7 against 2.5 ms of this
+// kernel.)  PRE: w_s holds r_e conj(w_e) already.  In the precision form a
+// thread adds at most 64 terms before its sums are reduced: error-free sums
+// over the EG threads of a component, then FP64.
+template <typename T, int R, bool PRE> struct SliceSums {
+    typedef typename cvec<T>::type V;
+    static constexpr int D = R * R;
+    static constexpr int TT = R <= 2 ? 1 : 2;
+    static constexpr int TR = (R + TT - 1) / TT, NT = TR * TR;
+    static constexpr int EG0 = 128 / NT;
+    static constexpr int EG = EG0 > 32 ? 32 : EG0;
+    static constexpr bool COMP = sizeof(T) == 4;
+    static constexpr int QPT = (D + 127) / 128;      // components per thread of the totals
+    static constexpr int RS = COMP ? 64 : 1 << 30;   // terms of a thread before a reduction
+    // bytes of shared memory of a reduction
+    static constexpr size_t RED = (size_t)EG * NT * TT * TT * sizeof(V);
+    int ti, tj, grp, terms;
+    V acc[TT][TT];
+    double2 tot[QPT];   // components tid, tid + 128, ..
+
+    __device__ __forceinline__ void start(int tid)
+    {
+        const int tile = tid % NT;
+        grp = tid / NT;
+        ti = tile / TR;
+        tj = tile - ti * TR;
+        terms = 0;
+#pragma unroll
+        for (int u = 0; u < TT; ++u)
+#pragma unroll
+            for (int v = 0; v < TT; ++v) acc[u][v] = czero<V>();
+#pragma unroll
+        for (int u = 0; u < QPT; ++u) tot[u] = make_double2(0.0, 0.0);
+    }
+    __device__ __forceinline__ void values(V (&d)[TT], const V* p) const
+    {
+        if constexpr (sizeof(V) == 8 && TT == 4 && R % 2 == 0) {
+            load4(d, p);
+        } else if constexpr (sizeof(V) == 8 && TT == 2 && R % 2 == 0) {
+            const float4 t = *reinterpret_cast<const float4*>(p);
+            d[0].x = t.x; d[0].y = t.y;
+            d[1].x = t.z; d[1].y = t.w;
+        } else {
+#pragma unroll
+            for (int u = 0; u < TT; ++u) d[u] = p[u];
+        }
+    }
+    __device__ __forceinline__ void chunk(const V* h_s, const V* w_s, const V* r_s, int cnt)
+    {
+        if (grp < EG) {
+            for (int e = grp; e < cnt; e += EG) {
+                V h[TT], w[TT];
+                values(h, h_s + e * R + TT * ti);
+                values(w, w_s + e * R + TT * tj);
+                if constexpr (!PRE) {
+                    const V r = r_s[e];
+#pragma unroll
+                    for (int v = 0; v < TT; ++v) {   // r conj(w)
+                        V x = czero<V>();
+                        cmacc(x, w[v], r);
+                        w[v] = x;
+                    }
+                }
+#pragma unroll
+                for (int u = 0; u < TT; ++u)
+#pragma unroll
+                    for (int v = 0; v < TT; ++v) cmacc(acc[u][v], h[u], w[v]);
+            }
+        }
+        terms += (cnt + EG - 1) / EG;
+    }
+    // whether another chunk of `cnt` entries would take a thread past RS terms
+    __device__ __forceinline__ bool full(int cnt) const { return terms + (cnt + EG - 1) / EG > RS; }
+    // thread sums into the totals; red: RED bytes of shared memory that every
+    // thread is done with after a barrier
+    __device__ __forceinline__ void reduce(void* red, int tid)
+    {
+        V* rd = (V*)red;
+        __syncthreads();
+        if (grp < EG) {
+#pragma unroll
+            for (int u = 0; u < TT; ++u)
+#pragma unroll
+                for (int v = 0; v < TT; ++v) {
+                    rd[((u * TT + v) * NT + ti * TR + tj) * EG + grp] = acc[u][v];
+                    acc[u][v] = czero<V>();
+                }
+        }
+        __syncthreads();
+        terms = 0;
+#pragma unroll
+        for (int n = 0; n < QPT; ++n) {
+            const int q = tid + 128 * n;
+            if (q < D) {
+                const int a = q / R, c = q - a * R;
+                const V* src = rd + (((a % TT) * TT + c % TT) * NT + (a / TT) * TR + c / TT) * EG;
+                if constexpr (COMP) {
+                    float sx = 0.f, sy = 0.f, ex = 0.f, ey = 0.f;
+                    for (int g = 0; g < EG; ++g) {
+                        const V x = src[(g + q) % EG];   // (spread over the banks)
+                        float t, e;
+                        two_sum(sx, x.x, t, e);
+                        sx = t;
+                        ex += e;
+                        two_sum(sy, x.y, t, e);
+                        sy = t;
+                        ey += e;
+                    }
+                    tot[n].x += (double)sx + (double)ex;
+                    tot[n].y += (double)sy + (double)ey;
+                } else {
+                    for (int g = 0; g < EG; ++g) {
+                        const V x = src[(g + q) % EG];
+                        tot[n].x += (double)x.x;
+                        tot[n].y += (double)x.y;
+                    }
+                }
+            }
+        }
+    }
+    // out(q, value) for every component q = a R + c, by threads q, q + 128, ..
+    template <typename F> __device__ __forceinline__ void finish(void* red, int tid, F out)
+    {
+        reduce(red, tid);
+#pragma unroll
+        for (int n = 0; n < QPT; ++n)
+            if (tid + 128 * n < D) out(tid + 128 * n, tot[n]);
+    }
+};
+
 // Middle level m: G^{m+1}(k) = sum r conj(h_m (x) w_m); h_{m+1} = h_m^T Z(k); r carried.
 // One CTA per slice at a time (persistent over slices), chunks of CH entries
-// staged in shared memory as contiguous blocks (bulk copies in complex64 at
-// even rank).  For D = R^2 <= 64 the 128
-// threads split the gradient components (q = t mod 64) and the chunk's
-// entries (two interleaved halves, t / 64); the halves are added at the end
-// of the slice.  The carried h rows are read back from global memory (the
-// chunk just loaded them, so they come from L1) and written as 16-byte
-// vectors in complex64 at even rank.
+// staged in shared memory as contiguous blocks; the carried rows a thread per
+// entry, the components by SliceSums.
+//
+// Complex64 at even rank: the h and w rows of a chunk (16-byte multiples)
+// arrive by two bulk copies counted on the mbarrier of their buffer, one chunk
+// ahead of the arithmetic and across slices; residuals, level maps and the next
+// slice's Z are fetched into registers meanwhile.  (With one buffer every
+// chunk's copy was waited for: the kernel stood at 40 % of HBM with 43 % of the
+// issue slots used.)  The waits are bounded; on expiry *terr is raised, the
+// results are undefined, and the CTA issues no further copies: it loads by
+// plain loads from then on.  skip_copy (failure injection of the tests,
+// bfc_inject_fault): the copies are not issued and the waits give up after a
+// few tries.  Otherwise plain loads, with w multiplied by r as it is staged.
 template <typename T, int R>
-__global__ void __launch_bounds__(128, sizeof(T) == 4 ? 8 : 4)
+__global__ void __launch_bounds__(128, sizeof(T) == 4 && R <= 8 ? 6 : 4)
 k_grad_mid(const typename cvec<T>::type* __restrict__ H, const typename cvec<T>::type* __restrict__ Wm,
            const typename cvec<T>::type* __restrict__ Rc, const int32_t* __restrict__ seg,
            const int32_t* __restrict__ nxt, const typename cvec<T>::type* __restrict__ Zt,
@@ -1086,176 +1285,190 @@ k_grad_mid(const typename cvec<T>::type* __restrict__ H, const typename cvec<T>:
     typedef typename cvec<T>::type V;
     constexpr int D = R * R;
     constexpr int CH = 128;
-    constexpr int NG = D <= 64 ? 2 : 1;              // entry groups
-    constexpr int NQ = NG == 2 ? 1 : (D + 127) / 128;  // components per thread
+    constexpr int ZPT = (D + 127) / 128;   // values of a slice per thread
     constexpr bool VEC = sizeof(V) == 8 && R % 2 == 0;
-    __shared__ V z_s[D];
-    __shared__ __align__(16) V h_s[CH * R];
-    __shared__ __align__(16) V w_s[CH * R];
+    typedef SliceSums<T, R, !VEC> SS;
+    // [h rows | w rows] per buffer; a buffer that is done with also takes the
+    // reduction of a slice's sums
+    constexpr size_t ROWS = (size_t)CH * R * sizeof(V) + 16;
+    constexpr size_t BUF = ((2 * ROWS > SS::RED ? 2 * ROWS : SS::RED) + 15) / 16 * 16;
+    __shared__ __align__(16) unsigned char buf[VEC ? 2 : 1][BUF];
+    __shared__ __align__(16) V z_s[D];
     __shared__ V r_s[CH];
-    __shared__ double2 g_s[NG == 2 ? 64 : 1];
-    // complex64 at even rank: a chunk's h and w rows (contiguous, 16-byte
-    // multiples) arrive by two bulk copies counted on one mbarrier (the wait
-    // is bounded; on expiry *terr is raised, the results are undefined, and
-    // the CTA issues no further copies: it loads by plain loads from then on).
-    // skip_copy (failure injection of the tests, bfc_inject_fault): the copies
-    // are not issued and the waits give up after a few tries.
-    __shared__ __align__(8) unsigned long long cbar;
+    __shared__ __align__(8) unsigned long long cbar[2];
     const int tid = threadIdx.x;
-    const int grp = NG == 2 ? tid >> 6 : 0;
-    const int q0 = NG == 2 ? (tid & 63) : tid;
-    const uint32_t bar = (uint32_t)__cvta_generic_to_shared(&cbar);
-    uint32_t phase = 0;
-    bool use_bulk = VEC;          // CTA-uniform
-    bool pending = false;         // copies issued and then given up on
-    uint32_t pending_phase = 0;
-    const uint32_t wait_limit = skip_copy ? 64u : (1u << 22);
+    // the row of this thread's entry (position o in the next order)
+    auto carry = [&](const V* h_s, V r, size_t o) {
+        V hv[R], hn[R];
+        load_row_v<V, R>(h_s, (size_t)tid, hv);
+        row_times_slice<V, R>(hv, z_s, hn);
+        store_row_v<V, R>(Hn, o, hn);
+        Rn[o] = r;
+    };
     if constexpr (VEC) {
+        const uint32_t bar0 = (uint32_t)__cvta_generic_to_shared(&cbar[0]);   // buffer b: bar0 + 8 b
+        uint32_t phases = 0, issued = 0;   // one bit per buffer, CTA-uniform
+        bool use_bulk = true;              // CTA-uniform
+        const uint32_t wait_limit = skip_copy ? 64u : (1u << 22);
         if (tid == 0) {
-            asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(bar));
+            asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(bar0));
+            asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(bar0 + 8));
             asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
         }
         __syncthreads();
-    }
-    for (int k = blockIdx.x; k < S; k += gridDim.x) {
-        const int s0 = seg[k], s1 = seg[k + 1];
-        __syncthreads();
-        for (int q = tid; q < D; q += blockDim.x) z_s[q] = Zt[(size_t)k * D + q];
-        double2 g[NQ];
+        struct Chunk { int k, base, s1; };
+        // first chunk of the first non-empty slice from k on; empty slices have
+        // a zero gradient
+        auto first = [&](int k) {
+            Chunk c{k, 0, 0};
+            for (; c.k < S; c.k += gridDim.x) {
+                c.base = seg[c.k];
+                c.s1 = seg[c.k + 1];
+                if (c.base < c.s1) break;
+                for (int q = tid; q < D; q += 128) Gm[(size_t)c.k * D + q] = make_double2(0.0, 0.0);
+            }
+            return c;
+        };
+        auto issue = [&](int b, const Chunk& c) {
+            if (tid == 0) {
+                const uint32_t bytes = (uint32_t)(min(CH, c.s1 - c.base) * R * sizeof(V));
+                asm volatile("{\n.reg .b64 st;\nmbarrier.arrive.expect_tx.shared::cta.b64 st, [%0], %1;\n}\n"
+                             ::"r"(bar0 + 8 * b), "r"(2 * bytes) : "memory");
+                if (!skip_copy) {
+                    asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];"
+                                 ::"r"((uint32_t)__cvta_generic_to_shared(buf[b])), "l"(H + (size_t)c.base * R),
+                                 "r"(bytes), "r"(bar0 + 8 * b) : "memory");
+                    asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];"
+                                 ::"r"((uint32_t)__cvta_generic_to_shared(buf[b] + ROWS)), "l"(Wm + (size_t)c.base * R),
+                                 "r"(bytes), "r"(bar0 + 8 * b) : "memory");
+                }
+            }
+            issued |= 1u << b;
+        };
+        V rn = czero<V>(), zn[ZPT];
+        int on = 0;
+        auto fetch = [&](const Chunk& c) {
+            const int p = min(c.base + tid, c.s1 - 1);
+            rn = Rc[p];
+            on = nxt[p];
+        };
+        auto fetch_z = [&](const Chunk& c) {
 #pragma unroll
-        for (int u = 0; u < NQ; ++u) g[u] = make_double2(0.0, 0.0);
-        for (int base = s0; base < s1; base += CH) {
-            const int cnt = min(CH, s1 - base);
+            for (int u = 0; u < ZPT; ++u) {
+                const int q = tid + 128 * u;
+                zn[u] = q < D ? Zt[(size_t)c.k * D + q] : czero<V>();
+            }
+        };
+        Chunk c = first(blockIdx.x);
+        if (c.k < S) {
+            issue(0, c);
+            fetch(c);
+            fetch_z(c);
+        }
+        int b = 0;
+        bool fresh = true;
+        SS ss;
+        while (c.k < S) {
+            const int cnt = min(CH, c.s1 - c.base);
+            const V r = rn;
+            const size_t o = (size_t)on;
+            // this buffer's previous reader, the other buffer's readers, z_s and
+            // r_s are done; their accesses come before the copy engine's
+            asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+            __syncthreads();
+            Chunk n = c;
+            n.base += CH;
+            if (n.base >= n.s1) n = first(c.k + gridDim.x);
+            if (n.k < S && use_bulk) issue(b ^ 1, n);
+            if (fresh) {
+#pragma unroll
+                for (int u = 0; u < ZPT; ++u)
+                    if (tid + 128 * u < D) z_s[tid + 128 * u] = zn[u];
+                ss.start(tid);
+            }
+            r_s[tid] = r;
+            if (n.k < S) {
+                fetch(n);
+                if (n.k != c.k) fetch_z(n);
+            }
             bool have = false;
-            if constexpr (VEC) {
-                if (use_bulk) {
-                    // every thread's reads of the previous chunk are ordered
-                    // before the copy engine overwrites the buffers
-                    asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-                    __syncthreads();
-                    if (tid == 0) {
-                        const uint32_t bytes = (uint32_t)(cnt * R * sizeof(V));
-                        asm volatile("{\n.reg .b64 st;\nmbarrier.arrive.expect_tx.shared::cta.b64 st, [%0], %1;\n}\n"
-                                     ::"r"(bar), "r"(2 * bytes) : "memory");
-                        if (!skip_copy) {
-                            asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];"
-                                         ::"r"((uint32_t)__cvta_generic_to_shared(h_s)), "l"(H + (size_t)base * R),
-                                         "r"(bytes), "r"(bar) : "memory");
-                            asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];"
-                                         ::"r"((uint32_t)__cvta_generic_to_shared(w_s)), "l"(Wm + (size_t)base * R),
-                                         "r"(bytes), "r"(bar) : "memory");
-                        }
-                    }
-                    for (int x = tid; x < cnt; x += blockDim.x) r_s[x] = Rc[base + x];
-                    bool done = false;
-                    for (uint32_t it = 0; it < wait_limit && !done; ++it) {
-                        uint32_t ok;
-                        asm volatile("{\n.reg .pred p;\nmbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2, 1000;\n"
-                                     "selp.u32 %0, 1, 0, p;\n}\n"
-                                     : "=r"(ok) : "r"(bar), "r"(phase) : "memory");
-                        done = ok != 0;
-                    }
-                    // the phase completes once for every thread: any thread
-                    // that saw it complete makes the chunk valid for the CTA
-                    done = __syncthreads_or(done) != 0;
-                    if (done) {
-                        have = true;
-                    } else {
-                        if (tid == 0) atomicExch(terr, 1ull);
-                        use_bulk = false;
-                        pending = !skip_copy;
-                        pending_phase = phase;
-                    }
-                    phase ^= 1u;
+            if (issued >> b & 1u) {
+                bool done = false;
+                for (uint32_t it = 0; it < wait_limit && !done; ++it) {
+                    uint32_t ok;
+                    asm volatile("{\n.reg .pred p;\nmbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2, 1000;\n"
+                                 "selp.u32 %0, 1, 0, p;\n}\n"
+                                 : "=r"(ok) : "r"(bar0 + 8 * b), "r"(phases >> b & 1u) : "memory");
+                    done = ok != 0;
                 }
-            }
-            if (!have) {
-                __syncthreads();
-                for (int x = tid; x < cnt * R; x += blockDim.x) {
-                    h_s[x] = H[(size_t)base * R + x];
-                    w_s[x] = Wm[(size_t)base * R + x];
-                }
-                for (int x = tid; x < cnt; x += blockDim.x) r_s[x] = Rc[base + x];
-            }
-            __syncthreads();
-            // gradient components owned by threads
-#pragma unroll
-            for (int u = 0; u < NQ; ++u) {
-                const int q = q0 + 128 * u;
-                if (q < D) {
-                    const int pa = q / R, pc = q - pa * R;
-                    V acc = czero<V>();
-                    for (int e = grp; e < cnt; e += NG) {
-                        const V a = cmul(h_s[e * R + pa], w_s[e * R + pc]);
-                        cmacc(acc, a, r_s[e]);   // conj(a) r
-                    }
-                    g[u].x += (double)acc.x;
-                    g[u].y += (double)acc.y;
-                }
-            }
-            // carry h and r into the next order
-            for (int e = tid; e < cnt; e += blockDim.x) {
-                const size_t o = (size_t)nxt[base + e];
-                const size_t src = (size_t)(base + e) * R;
-                V hv[R];
-                if constexpr (VEC) {
-#pragma unroll
-                    for (int c = 0; c < R / 2; ++c) {
-                        const float4 v4 = reinterpret_cast<const float4*>(H + src)[c];
-                        hv[2 * c].x = v4.x; hv[2 * c].y = v4.y;
-                        hv[2 * c + 1].x = v4.z; hv[2 * c + 1].y = v4.w;
-                    }
+                // the phase completes once for every thread: any thread that
+                // saw it complete makes the chunk valid for the CTA
+                have = __syncthreads_or(done) != 0;
+                if (have) {
+                    issued ^= 1u << b;
+                    phases ^= 1u << b;
                 } else {
-#pragma unroll
-                    for (int c = 0; c < R; ++c) hv[c] = H[src + c];
+                    if (tid == 0) atomicExch(terr, 1ull);
+                    use_bulk = false;
                 }
-                // one pair of output columns at a time, stored at once (not
-                // unrolled, so the slice's R x R values are not all held in
-                // registers across entries)
-#pragma unroll 1
-                for (int c = 0; c < R; c += 2) {
-                    V a0 = czero<V>(), a1 = czero<V>();
-#pragma unroll
-                    for (int a = 0; a < R; ++a) {
-                        cmac(a0, hv[a], z_s[a * R + c]);
-                        if (c + 1 < R) cmac(a1, hv[a], z_s[a * R + c + 1]);
-                    }
-                    if constexpr (VEC) {
-                        reinterpret_cast<float4*>(Hn + o * R)[c / 2] = make_float4(a0.x, a0.y, a1.x, a1.y);
-                    } else {
-                        Hn[o * R + c] = a0;
-                        if (c + 1 < R) Hn[o * R + c + 1] = a1;
-                    }
+            }
+            V* h_s = (V*)buf[b];
+            V* w_s = (V*)(buf[b] + ROWS);
+            if (!have) {
+                // a copy given up on may still land in this buffer or the other:
+                // the results are undefined, the accesses stay in bounds
+                __syncthreads();
+                for (int x = tid; x < cnt * R; x += 128) {
+                    h_s[x] = H[(size_t)c.base * R + x];
+                    w_s[x] = Wm[(size_t)c.base * R + x];
                 }
-                Rn[o] = r_s[e];
+                __syncthreads();
             }
+            if (tid < cnt) carry(h_s, r, o);
+            ss.chunk(h_s, w_s, r_s, cnt);
+            fresh = n.k != c.k;
+            if (fresh) ss.finish(buf[b], tid, [&](int q, double2 g) { Gm[(size_t)c.k * D + q] = g; });
+            else if (ss.full(CH)) ss.reduce(buf[b], tid);
+            c = n;
+            b ^= 1;
         }
-        if constexpr (NG == 2) {
-            // add the second entry group's sums to the first
-            __syncthreads();
-            if (grp == 1 && q0 < D) g_s[q0] = g[0];
-            __syncthreads();
-            if (grp == 0 && q0 < D) {
-                const double2 o2 = g_s[q0];
-                Gm[(size_t)k * D + q0] = make_double2(g[0].x + o2.x, g[0].y + o2.y);
-            }
-        } else {
+        // copies that were given up on may still land: wait for them (bounded)
+        // before the CTA's shared memory is released
+        if (!skip_copy) {
 #pragma unroll
-            for (int u = 0; u < NQ; ++u) {
-                const int q = q0 + 128 * u;
-                if (q < D) Gm[(size_t)k * D + q] = g[u];
-            }
+            for (int q = 0; q < 2; ++q)
+                for (uint32_t it = 0; (issued >> q & 1u) && it < (1u << 22); ++it) {
+                    uint32_t ok;
+                    asm volatile("{\n.reg .pred p;\nmbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2, 1000;\n"
+                                 "selp.u32 %0, 1, 0, p;\n}\n"
+                                 : "=r"(ok) : "r"(bar0 + 8 * q), "r"(phases >> q & 1u) : "memory");
+                    if (ok) break;
+                }
         }
-    }
-    if (pending) {
-        // copies that were given up on may still land: wait for them
-        // (bounded) before the CTA's shared memory is released
-        for (uint32_t it = 0; it < (1u << 22); ++it) {
-            uint32_t ok;
-            asm volatile("{\n.reg .pred p;\nmbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2, 1000;\n"
-                         "selp.u32 %0, 1, 0, p;\n}\n"
-                         : "=r"(ok) : "r"(bar), "r"(pending_phase) : "memory");
-            if (ok) break;
+    } else {
+        V* h_s = (V*)buf[0];
+        V* w_s = (V*)(buf[0] + ROWS);
+        for (int k = blockIdx.x; k < S; k += gridDim.x) {
+            const int s0 = seg[k], s1 = seg[k + 1];
+            __syncthreads();
+            for (int q = tid; q < D; q += 128) z_s[q] = Zt[(size_t)k * D + q];
+            SS ss;
+            ss.start(tid);
+            for (int base = s0; base < s1; base += CH) {
+                const int cnt = min(CH, s1 - base);
+                __syncthreads();
+                for (int x = tid; x < cnt * R; x += 128) {
+                    V rw = czero<V>();
+                    cmacc(rw, Wm[(size_t)base * R + x], Rc[base + x / R]);
+                    h_s[x] = H[(size_t)base * R + x];
+                    w_s[x] = rw;
+                }
+                __syncthreads();
+                if (tid < cnt) carry(h_s, Rc[base + tid], (size_t)nxt[base + tid]);
+                ss.chunk(h_s, w_s, nullptr, cnt);
+                if (ss.full(CH)) ss.reduce(buf[0], tid);
+            }
+            ss.finish(buf[0], tid, [&](int q, double2 g) { Gm[(size_t)k * D + q] = g; });
         }
     }
 }
