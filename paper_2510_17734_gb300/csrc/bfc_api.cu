@@ -1160,17 +1160,21 @@ bfc_status bfc_matvec(bfc_ctx* ctx, int32_t nvec, const double* V, double* U)
     if (!c) return BFC_EINVAL;
     if (nvec < 1 || nvec > 4096 || !V || !U) return fail(c, BFC_EINVAL, "matvec needs 1 <= nvec <= 4096 and vectors");
     auto up = [](size_t x) { return (x + 255) / 256 * 256; };
-    const size_t vb = up((size_t)c->n * nvec * 16);
+    // device vectors are used where they are if the kernels' 16-byte accesses
+    // allow (V is read by the first kernel only, U written by the last)
+    const bool dev_v = c->P.values_on_device && (uintptr_t)V % 16 == 0;
+    const bool dev_u = c->P.values_on_device && (uintptr_t)U % 16 == 0;
+    const size_t bytes = (size_t)c->n * nvec * 16, vb = up(bytes);
     const size_t yb = up((size_t)c->S * nvec * c->r * c->vsz);
-    BFC_TRY(ensure_tmp(c, 2 * vb + 2 * yb));
+    BFC_TRY(ensure_tmp(c, (dev_v ? 0 : vb) + (dev_u ? 0 : vb) + 2 * yb));
     char* base = (char*)c->d_tmp;
-    double2* Vd = (double2*)base;
-    double2* Ud = (double2*)(base + vb);
-    void* y0 = base + 2 * vb;
-    void* y1 = base + 2 * vb + yb;
-    BFC_CK(c, cudaMemcpyAsync(Vd, V, (size_t)c->n * nvec * 16, in_kind(c), c->stream));
+    void* y0 = base;
+    void* y1 = base + yb;
+    const double2* Vd = dev_v ? (const double2*)V : (double2*)(base + 2 * yb);
+    double2* Ud = dev_u ? (double2*)U : (double2*)(base + 2 * yb + (dev_v ? 0 : vb));
+    if (!dev_v) BFC_CK(c, cudaMemcpyAsync((void*)Vd, V, bytes, in_kind(c), c->stream));
     BFC_TRY(get_fo_ops(c->fp32, c->r)->matvec(c, nvec, Vd, Ud, y0, y1));
-    BFC_CK(c, cudaMemcpyAsync(U, Ud, (size_t)c->n * nvec * 16, out_kind(c), c->stream));
+    if (!dev_u) BFC_CK(c, cudaMemcpyAsync(U, Ud, bytes, out_kind(c), c->stream));
     return sync(c);
 }
 

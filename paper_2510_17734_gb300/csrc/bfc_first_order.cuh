@@ -494,7 +494,7 @@ k_h1_rows(const int32_t* __restrict__ seg, int nfib, const typename cvec<T>::typ
 
 // ---------------------------------------------------------------- matvec
 
-// Y_{L+1}[p][q] = sum over the leaf of zL(j)^T v_q(j), p = j / b (the
+// L = 0: Y[p][q] = sum over the leaf of zL(j)^T v_q(j), p = j / b (the
 // contraction of S^{L+2} with the vectors over j_L); one thread per (p, q).
 template <typename T, int R>
 __global__ void k_mv_leaf(const typename cvec<T>::type* __restrict__ zL, const double2* __restrict__ Vin, int b,
@@ -517,67 +517,219 @@ __global__ void k_mv_leaf(const typename cvec<T>::type* __restrict__ zL, const d
     for (int c = 0; c < R; ++c) Y[idx * R + c] = acc[c];
 }
 
-// Level m of the contraction (m = L .. 1): Y_m[k] = Z[m][k] T_m[g(k)], where
-// T_L[g] = Y_{L+1}[g] with g = the column bits of k, and for m < L
-// T_m[g] = Y_{m+1}[2g] + Y_{m+1}[2g + 1] (the sum over j_m) with g = k
-// without its bit m (i_{L-m}).  One thread per (k, q).
+// One pass over several levels.  Y_m[k] = Z[m][k] T_m[g(k)], where T_L[g] =
+// Y_{L+1}[g] with g = the column bits of k (the leaf sums), and for m < L
+// T_m[g] = Y_{m+1}[2g] + Y_{m+1}[2g + 1] (the sum over j_m) with g = k without
+// its bit m (i_{L-m}).  With k = (row bits I, column bits J) a level turns the
+// last column bit into a new last row bit, so s levels close on 2^s elements
+// that share I's first bits and J's first bits, as a stage of an FFT does.  A
+// block takes 16 elements (s = 4 bits x, level t of the pass works on bit t of
+// x: the pair differing there is summed and replaced by the two products; fewer
+// bits: several such groups) for VT vectors through up to four levels: the intermediates pass through memory
+// four times at L = 12 instead of thirteen.  Thread = (pair, TV vectors 16
+// apart): T in registers, Z read from shared memory for TV products each, the
+// next level's 16 slices copied in meanwhile.  The first pass starts from the
+// leaf sums of 8 column prefixes (level L has no sum), the last ends with the
+// rows u(i) = z1(i)^T T_0[p_i].  Intermediates are laid out [k][c][q].
+// n = 65536, r = 8, 64 vectors, complex64: 0.65 ms of kernels before (a thread
+// per slice and vector, a pass per level), now 0.20 (with one group per block
+// 0.22; 0.28 with 64 vectors per block, 2 blocks per SM, 0.24 with 16).
+template <typename T, int R> struct MvCfg {
+    static constexpr size_t VS = sizeof(typename cvec<T>::type);
+    static constexpr int E = 16;                                   // elements of a block
+    static constexpr int CAP = (int)(32768 / (E * R * VS));        // vectors in 32 KB
+    static constexpr int VT = CAP >= 64 ? 64 : CAP >= 32 ? 32 : 16;
+    static constexpr int TV = VT / 16;
+    static constexpr size_t YB = (size_t)E * R * VT * VS;
+    static constexpr size_t ZB = ((size_t)E * R * R * VS + 15) / 16 * 16;
+    static constexpr size_t SMEM = YB + 2 * ZB;
+    static_assert(SMEM <= 227 * 1024, "shared memory of a block");
+};
+
+struct MvPass {
+    int L, M;       // levels of the network; first (highest) level of the pass
+    int s, lv;      // element bits; levels (lv = s, or s - 1 in the last pass)
+    int first, last;
+    int b, nvec;
+};
+
 template <typename T, int R>
-__global__ void k_mv_level(const typename cvec<T>::type* __restrict__ Zm, const typename cvec<T>::type* __restrict__ Yin,
-                           typename cvec<T>::type* __restrict__ Yout, int m, int L, int nvec, int S)
+__global__ void __launch_bounds__(128)
+k_mv_pass(MvPass ps, const typename cvec<T>::type* __restrict__ Z, const typename cvec<T>::type* __restrict__ zL,
+          const typename cvec<T>::type* __restrict__ z1, const double2* __restrict__ Vin,
+          const typename cvec<T>::type* __restrict__ Yin, typename cvec<T>::type* __restrict__ Yout,
+          double2* __restrict__ U)
 {
     typedef typename cvec<T>::type V;
-    const int64_t idx = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (idx >= (int64_t)S * nvec) return;
-    const int k = (int)(idx / nvec), q = (int)(idx - (int64_t)k * nvec);
-    V tv[R];
-    if (m == L) {
-        const int64_t g = k & ((1 << L) - 1);
+    typedef MvCfg<T, R> C;
+    constexpr int VT = C::VT, TV = C::TV, D = R * R;
+    extern __shared__ __align__(16) unsigned char smem[];
+    V* ys = (V*)smem;                                      // [x][c][q]
+    const int s = ps.s, nel = 1 << s, npair = nel >> 1;
+    // C::E >> s groups of 2^s elements; this thread's group, pair and lane
+    const int tid = threadIdx.x, l = tid & 15;
+    const int grp = (tid >> 4) / npair, bf = (tid >> 4) - grp * npair;
+    const int nJ = ps.M + 1 - s;                           // column bits shared by a group
+    const unsigned ngrp = 1u << (ps.L + 1 - s), grp0 = blockIdx.x * (unsigned)(C::E >> s);
+    const bool active = grp0 + grp < ngrp;
+    const int I0 = (int)((grp0 + grp) >> nJ), J0 = (int)((grp0 + grp) & ((1u << nJ) - 1));
+    V* yg = ys + (size_t)grp * nel * R * C::VT;            // the group's elements
+    const int q0 = blockIdx.y * VT, nq = min(VT, ps.nvec - q0);
+    const int nt = (nq + 15) >> 4;                         // vectors of lane 0
+    const size_t S = (size_t)2 << ps.L;
+    // row bits I, then the first `cnt` bits of x
+    auto row_bits = [&](int I, int x, int cnt) {
+        for (int u = 0; u < cnt; ++u) I = I << 1 | ((x >> u) & 1);
+        return I;
+    };
+    // the slices of level t of the pass into buffer t & 1
+    auto stage = [&](int t) {
+        const int m = ps.M - t;
+        V* dst = (V*)(smem + C::YB + (size_t)(t & 1) * C::ZB);
+        constexpr bool W16 = (D * C::VS) % 16 == 0;
+        constexpr int PIECE = W16 ? 16 : 8, PP = (int)(D * C::VS / PIECE);
+        for (int y = tid; y < C::E * PP; y += 128) {
+            const int gx = y / PP, w = y - gx * PP, x = gx & (nel - 1);
+            const unsigned g = grp0 + (unsigned)(gx >> s);
+            if (g >= ngrp) break;
+            const size_t k = ((size_t)row_bits((int)(g >> nJ), x, t + 1) << m) |
+                             ((size_t)(g & ((1u << nJ) - 1)) << (s - 1 - t)) | (size_t)(x >> (t + 1));
+            const unsigned char* src = (const unsigned char*)(Z + ((size_t)(m - 1) * S + k) * D) + (size_t)w * PIECE;
+            unsigned char* d = (unsigned char*)(dst + (size_t)gx * D) + (size_t)w * PIECE;
+            if constexpr (W16) cp_async16(d, src);
+            else cp_async8(d, src);
+        }
+        cp_async_commit();
+    };
+    V tv[R][TV];
+    // the pair's inputs of level t: their sum (the first level of all: one)
+    auto load_pair = [&](int t, int e0, int e1) {
+        const bool expand = ps.first && t == 0;
+        if (expand) {
+            // leaf sums of column prefix J
+            const int J = (J0 << (s - 1)) | (e0 >> 1);
 #pragma unroll
-        for (int c = 0; c < R; ++c) tv[c] = Yin[(g * nvec + q) * R + c];
-    } else {
-        const int64_t g = ((int64_t)(k >> (m + 1)) << m) | (k & ((1 << m) - 1));
+            for (int c = 0; c < R; ++c)
 #pragma unroll
-        for (int c = 0; c < R; ++c) {
-            const V a = Yin[((2 * g) * nvec + q) * R + c], bq = Yin[((2 * g + 1) * nvec + q) * R + c];
-            tv[c].x = a.x + bq.x;
-            tv[c].y = a.y + bq.y;
+                for (int v = 0; v < TV; ++v) tv[c][v] = czero<V>();
+            for (int r = 0; r < ps.b; ++r) {
+                const size_t j = (size_t)J * ps.b + r;
+                V z[R];
+                load_row_v<V, R>(zL, j, z);
+#pragma unroll
+                for (int v = 0; v < TV; ++v)
+                    if (l + 16 * v < nq) {
+                        const V x = from_d2<V>(Vin[j * ps.nvec + q0 + l + 16 * v]);
+#pragma unroll
+                        for (int c = 0; c < R; ++c) cmac(tv[c][v], z[c], x);
+                    }
+            }
+        } else if (t == 0) {
+            const size_t k0 = ((size_t)I0 << (ps.M + 1)) | ((size_t)J0 << s);
+            const V* a = Yin + (k0 + e0) * R * ps.nvec + q0 + l;
+            const V* b = Yin + (k0 + e1) * R * ps.nvec + q0 + l;
+#pragma unroll
+            for (int c = 0; c < R; ++c)
+#pragma unroll
+                for (int v = 0; v < TV; ++v) {
+                    tv[c][v] = czero<V>();
+                    if (l + 16 * v < nq) {
+                        const V x = a[(size_t)c * ps.nvec + 16 * v], y = b[(size_t)c * ps.nvec + 16 * v];
+                        tv[c][v].x = x.x + y.x;
+                        tv[c][v].y = x.y + y.y;
+                    }
+                }
+        } else {
+            const V* a = yg + (size_t)e0 * R * VT + l;
+            const V* b = yg + (size_t)e1 * R * VT + l;
+#pragma unroll
+            for (int c = 0; c < R; ++c)
+#pragma unroll
+                for (int v = 0; v < TV; ++v) {
+                    tv[c][v] = czero<V>();
+                    if (v < nt) {
+                        const V x = a[c * VT + 16 * v], y = b[c * VT + 16 * v];
+                        tv[c][v].x = x.x + y.x;
+                        tv[c][v].y = x.y + y.y;
+                    }
+                }
+        }
+    };
+    if (ps.lv > 0) stage(0);
+    for (int t = 0; t < ps.lv; ++t) {
+        const int e0 = ((bf >> t) << (t + 1)) | (bf & ((1 << t) - 1)), e1 = e0 | 1 << t;
+        // level 0 reads global memory: before the wait for its slices
+        if (t == 0 && active) load_pair(0, e0, e1);
+        cp_async_wait_all();
+        __syncthreads();   // the level's slices and the elements of the level before; the other buffer is free
+        if (t + 1 < ps.lv) stage(t + 1);
+        if (!active) continue;
+        if (t > 0) load_pair(t, e0, e1);
+        const V* zt = (const V*)(smem + C::YB + (size_t)(t & 1) * C::ZB) + (size_t)grp * nel * D;
+        const bool out = t + 1 == s;   // to global memory (not in the last pass)
+#pragma unroll 1
+        for (int i = 0; i < 2; ++i) {
+            const int x = i ? e1 : e0;
+            const V* z = zt + (size_t)x * D;
+            const size_t ko = out ? ((size_t)row_bits(I0, x, s) << nJ) | (size_t)J0 : 0;
+#pragma unroll 1
+            for (int a = 0; a < R; ++a) {
+                V acc[TV], zr[R];
+#pragma unroll
+                for (int v = 0; v < TV; ++v) acc[v] = czero<V>();
+                load_row_v<V, R>(z, (size_t)a, zr);
+#pragma unroll
+                for (int c = 0; c < R; ++c)
+#pragma unroll
+                    for (int v = 0; v < TV; ++v) cmac(acc[v], zr[c], tv[c][v]);
+                if (out) {
+#pragma unroll
+                    for (int v = 0; v < TV; ++v)
+                        if (l + 16 * v < nq) Yout[(ko * R + a) * ps.nvec + q0 + l + 16 * v] = acc[v];
+                } else {
+#pragma unroll
+                    for (int v = 0; v < TV; ++v)
+                        if (v < nt) yg[((size_t)x * R + a) * VT + l + 16 * v] = acc[v];
+                }
+            }
         }
     }
-    const V* Z = Zm + (size_t)k * R * R;
+    if (ps.last) {
+        // rows of the 2^(s-1) leaf prefixes of the block
+        __syncthreads();
+        if (!active) return;
+        const int t = ps.lv;
+        load_pair(t, bf, bf | 1 << t);   // bits 0 .. t - 1 of bf are the new row bits
+        const size_t p = (size_t)row_bits(I0, bf, t);
+        for (int r = 0; r < ps.b; ++r) {
+            const size_t i = p * ps.b + r;
+            V z[R];
+            load_row_v<V, R>(z1, i, z);
 #pragma unroll
-    for (int a = 0; a < R; ++a) {
-        V acc = czero<V>();
+            for (int v = 0; v < TV; ++v)
+                if (l + 16 * v < nq) {
+                    V acc = czero<V>();
 #pragma unroll
-        for (int c = 0; c < R; ++c) cmac(acc, Z[a * R + c], tv[c]);
-        Yout[idx * R + a] = acc;
+                    for (int c = 0; c < R; ++c) cmac(acc, z[c], tv[c][v]);
+                    U[i * ps.nvec + q0 + l + 16 * v] = to_d2(acc);
+                }
+        }
     }
 }
 
-// u_q(i) = z1(i)^T T_0[p_i], T_0[p] = Y_1[2p] + Y_1[2p + 1] (the sum over j_0)
-// for L >= 1, or Y_1[0] (the leaf contraction) for L = 0; one thread per (i, q).
+// u_q(i) = z1(i)^T Y[q], Y the leaf contraction, for L = 0; one thread per (i, q).
 template <typename T, int R>
-__global__ void k_mv_root(const typename cvec<T>::type* __restrict__ z1, const typename cvec<T>::type* __restrict__ Y1,
-                          int b, int L, int nvec, int64_t n, double2* __restrict__ U)
+__global__ void k_mv_root(const typename cvec<T>::type* __restrict__ z1, const typename cvec<T>::type* __restrict__ Y,
+                          int nvec, int64_t n, double2* __restrict__ U)
 {
     typedef typename cvec<T>::type V;
     const int64_t idx = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (idx >= n * nvec) return;
     const int64_t i = idx / nvec;
     const int q = (int)(idx - i * nvec);
-    const int64_t p = i / b;
     V acc = czero<V>();
 #pragma unroll
-    for (int a = 0; a < R; ++a) {
-        V tv;
-        if (L == 0) {
-            tv = Y1[(int64_t)q * R + a];
-        } else {
-            const V x = Y1[((2 * p) * nvec + q) * R + a], y = Y1[((2 * p + 1) * nvec + q) * R + a];
-            tv.x = x.x + y.x;
-            tv.y = x.y + y.y;
-        }
-        cmac(acc, z1[i * R + a], tv);
-    }
+    for (int a = 0; a < R; ++a) cmac(acc, z1[i * R + a], Y[(int64_t)q * R + a]);
     U[idx] = to_d2(acc);
 }
 
@@ -593,29 +745,47 @@ template <typename T, int R> struct FirstOrder {
     static bfc_status matvec(Ctx* c, int nvec, const double2* Vd, double2* Ud, V* Y0, V* Y1)
     {
         const int L = c->L;
-        const int64_t npre = (int64_t)1 << L;
-        const int64_t S = c->S;
-        {
-            ProfScope ps(c, "mv_leaf");
-            const int64_t cnt = npre * nvec;
-            k_mv_leaf<T, R><<<nblocks(cnt, 256), 256, 0, c->stream>>>((const V*)c->zLt, Vd, c->b, nvec, (int)npre, Y0);
+        if (L == 0) {
+            {
+                ProfScope ps(c, "mv_leaf");
+                k_mv_leaf<T, R><<<nblocks(nvec, 256), 256, 0, c->stream>>>((const V*)c->zLt, Vd, c->b, nvec, 1, Y0);
+            }
+            {
+                ProfScope ps(c, "mv_root");
+                k_mv_root<T, R><<<nblocks(c->n * nvec, 256), 256, 0, c->stream>>>((const V*)c->z1t, Y0, nvec, c->n, Ud);
+            }
+            BFC_LAUNCH_CHECK(c, "matvec");
+            return BFC_OK;
         }
-        V* yin = Y0;
-        V* yout = Y1;
-        for (int m = L; m >= 1; --m) {
-            ProfScope ps(c, "mv_level");
-            const int64_t cnt = S * nvec;
-            k_mv_level<T, R><<<nblocks(cnt, 256), 256, 0, c->stream>>>(
-                (const V*)c->Zt + (size_t)(m - 1) * S * R * R, yin, yout, m, L, nvec, (int)S);
-            V* tmp = yin;
+        typedef MvCfg<T, R> MC;
+        BFC_CK(c, cudaFuncSetAttribute(k_mv_pass<T, R>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)MC::SMEM));
+        // the last pass takes up to 3 levels, the first up to 4, the others the
+        // rest in even parts of at most 4
+        const int nlast = std::min(3, L - 1), nfirst = std::min(4, L - nlast);
+        int rest = L - nlast - nfirst, mids = (rest + 3) / 4;
+        V* yin = nullptr;
+        V* yout = Y0;
+        auto pass = [&](int M, int s, int lv, int first, int last) {
+            ProfScope ps(c, "mv_pass");
+            const MvPass mp{L, M, s, lv, first, last, c->b, nvec};
+            const unsigned groups = 1u << (L + 1 - s), per = (unsigned)(MC::E >> s);
+            const dim3 grid((groups + per - 1) / per, (unsigned)((nvec + MC::VT - 1) / MC::VT));
+            k_mv_pass<T, R><<<grid, 128, MC::SMEM, c->stream>>>(mp, (const V*)c->Zt, (const V*)c->zLt,
+                                                                (const V*)c->z1t, Vd, yin, yout, Ud);
+            V* t = yin == nullptr ? Y1 : yin;
             yin = yout;
-            yout = tmp;
+            yout = t;
+        };
+        int M = L;
+        pass(M, nfirst, nfirst, 1, 0);
+        M -= nfirst;
+        for (; mids > 0; --mids) {
+            const int s = (rest + mids - 1) / mids;
+            pass(M, s, s, 0, 0);
+            M -= s;
+            rest -= s;
         }
-        {
-            ProfScope ps(c, "mv_root");
-            const int64_t cnt = c->n * nvec;
-            k_mv_root<T, R><<<nblocks(cnt, 256), 256, 0, c->stream>>>((const V*)c->z1t, yin, c->b, L, nvec, c->n, Ud);
-        }
+        pass(M, nlast + 1, nlast, 0, 1);
         BFC_LAUNCH_CHECK(c, "matvec");
         return BFC_OK;
     }
