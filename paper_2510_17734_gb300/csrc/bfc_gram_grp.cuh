@@ -30,10 +30,12 @@
 //
 // Measured, all middle levels of a sweep, against the per-entry kernels that
 // these levels ran before: n = 4096, L = 8, r = 12, 3.41 M entries, complex64
-// 107.2 -> 3.6 ms (against k_mid_gram); n = 4096, L = 8, r = 6, 265 k entries,
-// FP64 19.1 -> 3.3 ms (k_mid_gram, bound by the FP64 pipe at 1.25 TFLOP/s);
-// n = 3072, L = 8, r = 5, 961 k entries, complex64 1.42 -> 0.87 ms (against
-// k_mid_gram_tc).
+// 107.2 -> 2.9 ms (against k_mid_gram); n = 4096, L = 8, r = 6, 265 k entries,
+// FP64 19.1 -> 2.8 ms (k_mid_gram, bound by the FP64 pipe at 1.25 TFLOP/s);
+// n = 3072, L = 8, r = 5, 961 k entries, complex64 1.42 -> 0.66 ms (against
+// k_mid_gram_tc).  Issue-bound; two groups per compensated step took 3.6 -> 2.9,
+// 0.87 -> 0.66 and (n = 65536, r = 8) 1.70 -> 1.54 ms, the parallel reduction of
+// the thread groups 34 -> 5 us a level at n = 256, r = 4 (32 slices).
 #pragma once
 
 #include "bfc_kernels.cuh"
@@ -254,7 +256,7 @@ k_group_sums_warp(const typename cvec<T>::type* __restrict__ H, const typename c
 {
     typedef typename cvec<T>::type V;
     typedef GrpRec<V, R> RL;
-    __shared__ __align__(16) V a_s[4][32 * R];
+    __shared__ __align__(16) V a_s[4][32 * R + 2];
     __shared__ V t_s[4][32];
     const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
     const int g = blockIdx.x * 4 + wib;
@@ -329,14 +331,16 @@ __device__ __forceinline__ uint64_t g2sub(uint64_t a, uint64_t b)
     return d;
 }
 
-// (s, nc) += x y with packed operands: X1 = (x.re, x.re), X2 = (x.im, x.im),
-// Y = (y.re, y.im), Yr = i y = (-y.im, y.re), so x y = X1 Y + X2 Yr.  s is
-// the Kahan sum and nc its negated compensation (the value is s + nc); the
-// compensation enters inside the fused multiply-adds.
-__device__ __forceinline__ void grp_acc2(uint64_t& s, uint64_t& nc, uint64_t X1, uint64_t X2, uint64_t Y,
-                                         uint64_t Yr)
+// (s, nc) += x y + x' y' with packed operands: X1 = (x.re, x.re), X2 = (x.im,
+// x.im), Y = (y.re, y.im), Yr = i y = (-y.im, y.re), so x y = X1 Y + X2 Yr.  s
+// is the Kahan sum and nc its negated compensation (the value is s + nc); the
+// compensation enters inside the fused multiply-adds.  Two groups per step: the
+// products' roundings, two per group and component, are as many as with one
+// step per group, the three additions of the step are shared.
+__device__ __forceinline__ void grp_acc2(uint64_t& s, uint64_t& nc, uint64_t X1, uint64_t X2, uint64_t Y, uint64_t Yr,
+                                         uint64_t W1, uint64_t W2, uint64_t Z, uint64_t Zr)
 {
-    const uint64_t q = g2fma(X1, Y, g2fma(X2, Yr, nc));   // x y - c
+    const uint64_t q = g2fma(X1, Y, g2fma(X2, Yr, g2fma(W1, Z, g2fma(W2, Zr, nc))));   // x y + x' y' - c
     const uint64_t t = g2add(s, q);
     nc = g2sub(q, g2sub(t, s));
     s = t;
@@ -373,8 +377,8 @@ template <typename T, int R> struct GrpCfg {
     static_assert(RS * VS % 16 == 0, "records must be whole 16-byte pieces");
     static constexpr size_t STAGE = (size_t)CG * RS * VS;
     static constexpr size_t RING = NST * STAGE;
-    static constexpr size_t KBYTES = G > 1 ? (size_t)(NPK + D) * sizeof(double2) : 0;
-    static constexpr size_t SMEM = RING + KBYTES;
+    static constexpr size_t KBYTES = G > 1 ? (size_t)G * (NPK + D) * VS : 0;
+    static constexpr size_t SMEM = RING > KBYTES ? RING : KBYTES;
     static_assert(SMEM <= 227 * 1024, "shared memory of a block");
     // blocks per SM the registers are budgeted for: a tile's sums (and, in the
     // precision form, compensations) take 4 T^2 registers, plus about 64 (25
@@ -417,7 +421,7 @@ k_mid_gram_grp(const typename cvec<T>::type* __restrict__ grec, const int32_t* _
     extern __shared__ __align__(16) unsigned char smem[];
     typedef typename C::RL RL;
     V* ring = (V*)smem;                           // [NST][CG][RS]
-    double2* Kacc = (double2*)(smem + C::RING);   // thread-group reduction (G > 1)
+    V* red = (V*)smem;                            // thread-group reduction (G > 1), after the ring
 
     const int tid = threadIdx.x;
     const int part = C::NSPLIT > 1 ? blockIdx.x % C::NSPLIT : 0;   // this block's share of the tiles
@@ -461,7 +465,7 @@ k_mid_gram_grp(const typename cvec<T>::type* __restrict__ grec, const int32_t* _
                 n2[u][v] = 0ull;
             }
         }
-        __syncthreads();  // previous slice done with the ring and Kacc
+        __syncthreads();  // previous slice done with the ring and the reduction
 #pragma unroll
         for (int c = 0; c < NST - 1; ++c) {
             if (c < nch) issue(c, g0 + c * CG, min(CG, g1 - g0 - c * CG));
@@ -477,50 +481,61 @@ k_mid_gram_grp(const typename cvec<T>::type* __restrict__ grec, const int32_t* _
             const int cnt = min(CG, g1 - g0 - c * CG);
             if constexpr (sizeof(T) == 4) {
               if (worker) {
-                for (int gi = grp; gi < cnt; gi += C::G) {
+                for (int gi = grp; gi < cnt; gi += 2 * C::G) {
                     const V* gr = buf + gi * RS;
+                    // the second group of the step; past the end the first one
+                    // again with a zero factor
+                    const bool two = gi + C::G < cnt;
+                    const V* gs = two ? gr + C::G * RS : gr;
                     if constexpr (!BY_COL) {
                         // X = conj(h) h^T from s = h; Y = M (sums of the w side)
                         const V x = cmul(make_conj(gr[aI]), gr[aJ]);
+                        V w = cmul(make_conj(gs[aI]), gs[aJ]);
+                        if (!two) w = czero<V>();
                         const uint64_t X1 = g2pack(x.x, x.x), X2 = g2pack(x.y, x.y);
+                        const uint64_t W1 = g2pack(w.x, w.x), W2 = g2pack(w.y, w.y);
 #pragma unroll
                         for (int u = 0; u < TT; ++u) {
-                            V yr[TT];
+                            V yr[TT], zr[TT];
                             load_t<V, TT>(yr, gr + RL::m(cI + u, cJ));
+                            load_t<V, TT>(zr, gs + RL::m(cI + u, cJ));
 #pragma unroll
                             for (int v = 0; v < TT; ++v)
                                 grp_acc2(s2[u][v], n2[u][v], X1, X2, g2pack(yr[v].x, yr[v].y),
-                                         g2pack(-yr[v].y, yr[v].x));
+                                         g2pack(-yr[v].y, yr[v].x), W1, W2, g2pack(zr[v].x, zr[v].y),
+                                         g2pack(-zr[v].y, zr[v].x));
                         }
                         if (diag) {
-                            const V xv = make_conj(gr[aI]);
 #pragma unroll
-                            for (int u = 0; u < TT; ++u) grp_acc(ys[u], yc[u], xv, gr[RL::VOFF + cI + u]);
+                            for (int u = 0; u < TT; ++u) {
+                                grp_acc(ys[u], yc[u], make_conj(gr[aI]), gr[RL::VOFF + cI + u]);
+                                if (two) grp_acc(ys[u], yc[u], make_conj(gs[aI]), gs[RL::VOFF + cI + u]);
+                            }
                         }
                     } else {
                         // X = M (sums of the h side); Y = conj(w) w^T from s = w:
                         // term (u, v) = (conj(s_cI+u) x) s_cJ+v
                         const V x = gr[RL::m(aI, aJ)];
-                        V sj[TT], si[TT];
+                        V w = gs[RL::m(aI, aJ)];
+                        if (!two) w = czero<V>();
+                        V sj[TT], tj[TT];
                         load_t<V, TT>(sj, gr + cJ);
-                        load_t<V, TT>(si, gr + cI);
-                        uint64_t Y[TT], Q[TT];
-#pragma unroll
-                        for (int v = 0; v < TT; ++v) {
-                            Y[v] = g2pack(sj[v].x, sj[v].y);
-                            Q[v] = g2pack(-sj[v].y, sj[v].x);
-                        }
+                        load_t<V, TT>(tj, gs + cJ);
 #pragma unroll
                         for (int u = 0; u < TT; ++u) {
-                            const V xa = cmul(make_conj(si[u]), x);
+                            const V si = gr[cI + u], ti = gs[cI + u];
+                            const V xa = cmul(make_conj(si), x), wa = cmul(make_conj(ti), w);
                             const uint64_t X1 = g2pack(xa.x, xa.x), X2 = g2pack(xa.y, xa.y);
+                            const uint64_t W1 = g2pack(wa.x, wa.x), W2 = g2pack(wa.y, wa.y);
 #pragma unroll
-                            for (int v = 0; v < TT; ++v) grp_acc2(s2[u][v], n2[u][v], X1, X2, Y[v], Q[v]);
-                        }
-                        if (diag) {
-                            const V xv = gr[RL::VOFF + aI];
-#pragma unroll
-                            for (int u = 0; u < TT; ++u) grp_acc(ys[u], yc[u], xv, make_conj(si[u]));
+                            for (int v = 0; v < TT; ++v)
+                                grp_acc2(s2[u][v], n2[u][v], X1, X2, g2pack(sj[v].x, sj[v].y),
+                                         g2pack(-sj[v].y, sj[v].x), W1, W2, g2pack(tj[v].x, tj[v].y),
+                                         g2pack(-tj[v].y, tj[v].x));
+                            if (diag) {
+                                grp_acc(ys[u], yc[u], gr[RL::VOFF + aI], make_conj(si));
+                                if (two) grp_acc(ys[u], yc[u], gs[RL::VOFF + aI], make_conj(ti));
+                            }
                         }
                     }
                 }
@@ -619,31 +634,38 @@ k_mid_gram_grp(const typename cvec<T>::type* __restrict__ grec, const int32_t* _
             }
         } else {
             static_assert(C::G == 1 || !C::YSPARE, "the thread-group reduction takes y from the diagonal tiles");
-            for (int q = tid; q < NPK + D; q += NTH) Kacc[q] = make_double2(0.0, 0.0);
+            // every thread group's sums side by side (the ring is done with),
+            // then a thread per element adds them in FP64, in order
             __syncthreads();
-            for (int g = 0; g < C::G; ++g) {  // deterministic order over the thread groups
-                if (worker && grp == g) {
+            if (worker) {
+                V* rg = red + (size_t)grp * (NPK + D);
 #pragma unroll
-                    for (int u = 0; u < TT; ++u) {
-                        const int p = aI * R + cI + u;
-                        if (RP > R && cI + u >= R) continue;   // padding
+                for (int u = 0; u < TT; ++u) {
+                    const int p = aI * R + cI + u;
+                    if (RP > R && cI + u >= R) continue;   // padding
 #pragma unroll
-                        for (int v = 0; v < TT; ++v) {
-                            const int q = aJ * R + cJ + v;
-                            if (q <= p && (RP == R || cJ + v < R)) {
-                                Kacc[tri(p, q)].x += (double)s_[u][v].x;
-                                Kacc[tri(p, q)].y += (double)s_[u][v].y;
-                            }
-                        }
-                        if (diag) {
-                            Kacc[NPK + p].x += (double)ys[u].x;
-                            Kacc[NPK + p].y += (double)ys[u].y;
-                        }
+                    for (int v = 0; v < TT; ++v) {
+                        const int q = aJ * R + cJ + v;
+                        if (q <= p && (RP == R || cJ + v < R)) rg[tri(p, q)] = s_[u][v];
                     }
+                    if (diag) rg[NPK + p] = ys[u];
                 }
-                __syncthreads();
             }
-            rec_put_packed<T, R>(out, Kacc, tid, NTH);
+            __syncthreads();
+            for (int x = tid; x < D * D + D; x += NTH) {
+                const int p = x / D, q = x - p * D;
+                if (p < D && q > p) continue;
+                const V* src = red + (p < D ? tri(p, q) : NPK + q);
+                double2 v = make_double2(0.0, 0.0);
+#pragma unroll 4
+                for (int g = 0; g < C::G; ++g) {
+                    const V t = src[(size_t)g * (NPK + D)];
+                    v.x += (double)t.x;
+                    v.y += (double)t.y;
+                }
+                if (p < D) RC::put(out, p, q, v);
+                else RC::put_y(out, q, v);
+            }
         }
     }
 }

@@ -380,19 +380,145 @@ __device__ __forceinline__ bool thread_chol_solve(double2 (&K)[R * (R + 1) / 2],
 }
 
 // ------------------------------------------------------------------------
+// The complex64 form of warp_sums (see there).
+template <int R, typename F>
+__device__ __forceinline__ void warp_sums_tiles(const float2* __restrict__ A, const float2* __restrict__ tv, int s0,
+                                                int s1, float2* a_s, float2* t_s, int lane, F emit)
+{
+    constexpr int NB = (R + 1) / 2, NTK = NB * (NB + 1) / 2, NTW = NTK + NB;   // tiles of K, and with y
+    static_assert(NTW <= 32, "a tile per lane");
+    constexpr int EG = 32 / NTW;
+    constexpr bool EVEN = R % 2 == 0;
+    const int tile = lane % NTW, grp = lane / NTW;
+    const bool is_y = tile >= NTK;
+    int I = 0;
+    if (is_y) {
+        I = tile - NTK;
+    } else {
+        while ((I + 1) * (I + 2) / 2 <= tile) ++I;
+    }
+    const int J = is_y ? 0 : tile - I * (I + 1) / 2;
+    float2 acc[2][2], sum[2][2], cmp[2][2];
+#pragma unroll
+    for (int u = 0; u < 2; ++u)
+#pragma unroll
+        for (int v = 0; v < 2; ++v) acc[u][v] = sum[u][v] = cmp[u][v] = make_float2(0.f, 0.f);
+    for (int base = s0; base < s1; base += 32) {
+        const int cnt = min(32, s1 - base);
+        __syncwarp();
+        // the chunk's rows are contiguous: copy them as one coalesced block
+        {
+            const float2* src = A + (size_t)base * R;
+            const int nv = cnt * R;
+            if constexpr (EVEN) {
+                for (int x = lane; x < nv / 2; x += 32)
+                    reinterpret_cast<float4*>(a_s)[x] = reinterpret_cast<const float4*>(src)[x];
+            } else {
+                for (int x = lane; x < nv; x += 32) a_s[x] = src[x];
+            }
+            if (lane < cnt) t_s[lane] = tv[base + lane];
+        }
+        __syncwarp();
+        if (grp < EG) {
+            for (int e = grp; e < cnt; e += EG) {
+                const float2* ae = a_s + e * R;
+                float2 a[2], b[2];
+                if constexpr (EVEN) {
+                    const float4 x = *reinterpret_cast<const float4*>(ae + 2 * I);
+                    a[0] = make_float2(x.x, x.y);
+                    a[1] = make_float2(x.z, x.w);
+                    if (is_y) {
+                        b[0] = b[1] = t_s[e];
+                    } else {
+                        const float4 y = *reinterpret_cast<const float4*>(ae + 2 * J);
+                        b[0] = make_float2(y.x, y.y);
+                        b[1] = make_float2(y.z, y.w);
+                    }
+                } else {
+                    const float2* be = is_y ? t_s + e : ae + 2 * J;   // past an odd rank's end: not emitted
+                    a[0] = ae[2 * I];
+                    a[1] = ae[2 * I + 1];
+                    b[0] = be[0];
+                    b[1] = is_y ? b[0] : be[1];
+                }
+#pragma unroll
+                for (int u = 0; u < 2; ++u)
+#pragma unroll
+                    for (int v = 0; v < 2; ++v) cmacc(acc[u][v], a[u], b[v]);
+            }
+        }
+#pragma unroll
+        for (int u = 0; u < 2; ++u)
+#pragma unroll
+            for (int v = 0; v < 2; ++v) {
+                kahan(sum[u][v].x, cmp[u][v].x, acc[u][v].x);
+                kahan(sum[u][v].y, cmp[u][v].y, acc[u][v].y);
+                acc[u][v] = make_float2(0.f, 0.f);
+            }
+    }
+    // the EG shares of a tile into its first lane
+#pragma unroll
+    for (int g = 1; g < EG; ++g) {
+        const int src = tile + g * NTW;   // (only the first NTW lanes use it)
+#pragma unroll
+        for (int u = 0; u < 2; ++u)
+#pragma unroll
+            for (int v = 0; v < 2; ++v) {
+                const float ox = __shfl_sync(0xffffffffu, sum[u][v].x, src & 31);
+                const float oy = __shfl_sync(0xffffffffu, sum[u][v].y, src & 31);
+                const float cx = __shfl_sync(0xffffffffu, cmp[u][v].x, src & 31);
+                const float cy = __shfl_sync(0xffffffffu, cmp[u][v].y, src & 31);
+                if (grp == 0) {
+                    float t, e;
+                    two_sum(sum[u][v].x, ox, t, e);
+                    sum[u][v].x = t;
+                    cmp[u][v].x += cx - e;
+                    two_sum(sum[u][v].y, oy, t, e);
+                    sum[u][v].y = t;
+                    cmp[u][v].y += cy - e;
+                }
+            }
+    }
+    if (grp == 0) {
+#pragma unroll
+        for (int u = 0; u < 2; ++u) {
+            const int p = 2 * I + u;
+            if (!EVEN && p >= R) continue;
+            if (is_y) {
+                emit(R * (R + 1) / 2 + p, p, -2, sum[u][0], cmp[u][0]);
+            } else {
+#pragma unroll
+                for (int v = 0; v < 2; ++v) {
+                    const int q = 2 * J + v;
+                    if (q <= p) emit(tri(p, q), p, q, sum[u][v], cmp[u][v]);
+                }
+            }
+        }
+    }
+}
+
 // Sums of one warp over the rows s0 .. s1 of A (R values each) and the values
-// tv: K[p][q] = sum conj(a_p) a_q for p >= q and y[p] = sum conj(a_p) t.  Lanes
-// own the R(R+1)/2 + R items; chunks of 32 rows pass through the warp's own
-// shared memory (a_s: 32 R values, t_s: 32); in float the per-chunk partials
-// are folded into Kahan-compensated sums.  emit(item, p, q, sum, comp) hands
-// out every item once (q = -2: y), its value being sum - comp.
+// tv: K[p][q] = sum conj(a_p) a_q for p >= q and y[p] = sum conj(a_p) t.
+// Chunks of 32 rows pass through the warp's own shared memory (a_s: 32 R + 2
+// values, t_s: 32).  emit(item, p, q, sum, comp) hands out every item once, in
+// the order K packed, y (q = -2), its value being sum - comp.
+// FP64: lanes own the R(R+1)/2 + R items (the FP64 pipe counts instructions of
+// a warp).  Complex64: lanes own 2 x 2 tiles of the lower triangle and 2 x 1
+// tiles of y, EG rows at a time side by side; per-chunk partials are folded into
+// Kahan-compensated sums, the EG shares added by error-free sums.  (With an item
+// per lane the two 8-byte reads for each product made the shared-memory return
+// path, 128 bytes a cycle, the bound: n = 4096, r = 12, 3.4 M entries 0.189 ->
+// 0.147 ms; n = 65536, r = 8, 57 entries a row, 0.141 -> 0.151.)
 template <typename T, int R, typename F>
 __device__ __forceinline__ void warp_sums(const typename cvec<T>::type* __restrict__ A,
                                           const typename cvec<T>::type* __restrict__ tv, int s0, int s1,
                                           typename cvec<T>::type* a_s, typename cvec<T>::type* t_s, int lane, F emit)
 {
     typedef typename cvec<T>::type V;
-    constexpr bool COMP = sizeof(T) == 4;
+    if constexpr (sizeof(T) == 4) {
+        warp_sums_tiles<R>(A, tv, s0, s1, a_s, t_s, lane, emit);
+        return;
+    }
     constexpr int NP = R * (R + 1) / 2;
     constexpr int NI = NP + R;
     constexpr int IPL = (NI + 31) / 32;
@@ -413,25 +539,17 @@ __device__ __forceinline__ void warp_sums(const typename cvec<T>::type* __restri
             iq[u] = -2;  // right-hand side item
         }
     }
-    V acc[IPL], sum[IPL], cmp[IPL];
+    V acc[IPL];
 #pragma unroll
-    for (int u = 0; u < IPL; ++u) { acc[u] = czero<V>(); sum[u] = czero<V>(); cmp[u] = czero<V>(); }
+    for (int u = 0; u < IPL; ++u) acc[u] = czero<V>();
 
     for (int base = s0; base < s1; base += 32) {
         const int cnt = min(32, s1 - base);
         __syncwarp();
         // the chunk's rows are contiguous: copy them as one coalesced block
-        // (16-byte moves in complex64 at even rank, where every row starts on
-        // a 16-byte boundary)
         {
             const V* src = A + (size_t)base * R;
-            const int nv = cnt * R;
-            if constexpr (sizeof(V) == 8 && R % 2 == 0) {
-                for (int x = lane; x < nv / 2; x += 32)
-                    reinterpret_cast<float4*>(a_s)[x] = reinterpret_cast<const float4*>(src)[x];
-            } else {
-                for (int x = lane; x < nv; x += 32) a_s[x] = src[x];
-            }
+            for (int x = lane; x < cnt * R; x += 32) a_s[x] = src[x];
             if (lane < cnt) t_s[lane] = tv[base + lane];
         }
         __syncwarp();
@@ -445,21 +563,11 @@ __device__ __forceinline__ void warp_sums(const typename cvec<T>::type* __restri
                 }
             }
         }
-        if (COMP) {
-#pragma unroll
-            for (int u = 0; u < IPL; ++u) {
-                float sx = (float)sum[u].x, sy = (float)sum[u].y, cx = (float)cmp[u].x, cy = (float)cmp[u].y;
-                kahan(sx, cx, (float)acc[u].x);
-                kahan(sy, cy, (float)acc[u].y);
-                sum[u].x = sx; sum[u].y = sy; cmp[u].x = cx; cmp[u].y = cy;
-                acc[u] = czero<V>();
-            }
-        }
     }
 #pragma unroll
     for (int u = 0; u < IPL; ++u) {
         const int it = lane + 32 * u;
-        if (it < NI) emit(it, ip[u], iq[u], COMP ? sum[u] : acc[u], cmp[u]);
+        if (it < NI) emit(it, ip[u], iq[u], acc[u], czero<V>());
     }
 }
 
@@ -475,7 +583,7 @@ k_outer_gram(const typename cvec<T>::type* __restrict__ A, const typename cvec<T
     typedef typename cvec<T>::type V;
     constexpr int NI = R * (R + 1) / 2 + R;
     constexpr int WPB = 4;
-    __shared__ __align__(16) V a_s[WPB][32 * R];
+    __shared__ __align__(16) V a_s[WPB][32 * R + 2];
     __shared__ V t_s[WPB][32];
     const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
     const int f = blockIdx.x * WPB + wib;

@@ -20,10 +20,12 @@ template <typename T, int R> struct Path {
     // the grouped Gram (rank 1 has nothing to gain: K is one number)
     static constexpr bool GRP = R >= 2;
     // entries per group from which a warp takes one group (k_group_sums_warp)
-    // instead of r threads (k_group_sums): at rank 8 and 29 entries per group
-    // the threads are faster (0.140 against 0.154 ms at n = 65536), at rank 12
-    // and 52 to 420 a block's entries outgrow its staging and the warps are
-    static constexpr int GROUP_WARP = 32;
+    // instead of r threads (k_group_sums).  Complex64: at rank 8 and 29 entries
+    // per group the threads are faster (0.140 against 0.154 ms at n = 65536), at
+    // rank 12 and 52 to 420 a block's entries outgrow its staging and the warps
+    // are.  FP64: the warps form only the lower triangle, which the FP64 pipe
+    // shows at every size (n = 4096, r = 6: 71 against 145 to 170 us a level)
+    static constexpr int GROUP_WARP = sizeof(T) == 8 ? 2 : 32;
 
     static cudaError_t set_grp_attr()
     {

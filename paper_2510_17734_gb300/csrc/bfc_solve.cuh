@@ -331,6 +331,43 @@ template <typename T, int R> __device__ __forceinline__ void solve_tile(T* Lm, i
     }
 }
 
+// The row of conj(y) (row D) of the trailing matrix, columns 8J + 8 + 4 Jt ..
+// + 3, where D is a multiple of 4 (otherwise it lies in the last full tiles).
+template <typename T, int R> __device__ __forceinline__ void solve_y_tile(T* Lm, int J, int Jt)
+{
+    typedef Rec<T, R> RC;
+    typedef KPair<T> K;
+    typedef typename K::P P;
+    const T* xp = Lm + RC::row(J, RC::D - 8 * J);
+    const T* lp = Lm + RC::row(J, 8 + 4 * Jt);
+    P xr[4], xi[4], nr[4];
+    load8(xp, xr);
+    load8(xp + 8, xi);
+#pragma unroll
+    for (int t = 0; t < 4; ++t) nr[t] = K::neg(xr[t]);
+    T a[4], b[4];
+    const int c = 8 * J + 8 + 4 * Jt, Jd = c >> 3;
+    T* dp = Lm + RC::row(Jd, RC::D - 8 * Jd) + (c & 7);
+    ld4(dp, a);
+    ld4(dp + 8, b);
+#pragma unroll
+    for (int v = 0; v < 4; ++v) {
+        P lr[4], li[4];
+        load8(lp + 16 * v, lr);
+        load8(lp + 16 * v + 8, li);
+        typename K::A sr = K::zero(), si = K::zero();
+#pragma unroll
+        for (int t = 0; t < 4; ++t) {
+            sr = K::fma(K::fma(sr, xr[t], lr[t]), xi[t], li[t]);
+            si = K::fma(K::fma(si, xi[t], lr[t]), nr[t], li[t]);
+        }
+        a[v] -= K::sum(sr);
+        b[v] -= K::sum(si);
+    }
+    st4(dp, a);
+    st4(dp + 8, b);
+}
+
 // Factorization of the record in Lm by all threads of the CTA.  In the
 // precision form the diagonal blocks end inverted, in FP64 as L (1 / L_cc in
 // the imaginary slot of the diagonal).  False (CTA-uniform) when a pivot is
@@ -361,9 +398,12 @@ __device__ __forceinline__ bool solve_chol(T* Lm, T tol, volatile int* fail, int
                 rp[8] = xi[0]; rp[9] = xi[1];
             }
         }
-        // tile columns hold columns < D, tile rows also the row of conj(y)
-        const int mc = max(0, (D - 8 * J - 5) / 4), mr = (RC::DR - 8 * J - 5) / 4;
-        const int nt = mc * (mc + 1) / 2 + (mr > mc ? mc : 0);
+        // tile columns hold columns < D; the row of conj(y) is in the last tile
+        // row, or (D a multiple of 4) has tiles of one row, by the last threads
+        // (as full tiles they would take a round of their own)
+        const int mc = max(0, (D - 8 * J - 5) / 4), nt = mc * (mc + 1) / 2;
+        if constexpr (D % 4 == 0)
+            for (int x = nthr - 1 - tid; x < mc; x += nthr) solve_y_tile<T, R>(Lm, J, x);
         for (int x = tid; x < nt; x += nthr) {
             int I = (int)((sqrtf(8.f * (float)x + 1.f) - 1.f) * 0.5f);
             if (I * (I + 1) / 2 > x) --I;
