@@ -125,8 +125,10 @@ typedef struct {
     double group_ratio;     /* gram_impl 0: groups-per-entry threshold of the
                                grouped Gram.  0 selects the default (next to
                                the tensor-core kernel 0.1 (8 / r)^4, at most
-                               0.9; 0.9 next to the CUDA-core one); < 0 never
-                               groups; > 0 is used as given                             */
+                               0.9; next to the CUDA-core one 0.9, in the
+                               precision form only levels whose slices span
+                               at least r rows / columns); < 0 never groups;
+                               > 0 is used as given                             */
 } bfc_params;
 
 typedef struct {

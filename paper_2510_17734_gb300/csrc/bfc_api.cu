@@ -275,7 +275,13 @@ static bfc_status build(Ctx* c, const Inputs& in)
             gl.by_col = by_col;
             gl.ngroups = G;
             const double ratio = c->gram_tc ? c->grp_max_ratio : c->grp_cuda_ratio;
-            if (c->r >= 2 && c->P.gram_impl == 0 && (double)G < ratio * (double)N) {
+            // slices of fewer than r rows (columns) are rank deficient and solved
+            // at the ridge floor: there the coherent rounding of a few large
+            // group terms (2-norm error of K 1.8 times that of k_mid_gram) makes
+            // more of them indefinite (n = 4096, b = 4, r = 12: 24 of 20,480
+            // systems of a sweep kept their old slice, with k_mid_gram 2)
+            const bool floor_bound = c->fp32 && c->r > 8 && loc < c->r && !(c->P.group_ratio > 0.0);
+            if (c->r >= 2 && c->P.gram_impl == 0 && !floor_bound && (double)G < ratio * (double)N) {
                 gst.push_back((int32_t)N);
                 // the largest entry range of a k_group_sums block (its shared-memory staging)
                 const int64_t gpb = 128 / c->r;
