@@ -132,6 +132,27 @@ static bfc_status sync(Ctx* c)
 static cudaMemcpyKind in_kind(const Ctx* c) { return c->P.values_on_device ? cudaMemcpyDeviceToDevice : cudaMemcpyHostToDevice; }
 static cudaMemcpyKind out_kind(const Ctx* c) { return c->P.values_on_device ? cudaMemcpyDeviceToDevice : cudaMemcpyDeviceToHost; }
 
+// p is an address in device memory of the current device.
+static bool device_address(const void* p)
+{
+    cudaPointerAttributes a;
+    int dev = -1;
+    if (cudaPointerGetAttributes(&a, p) != cudaSuccess || cudaGetDevice(&dev) != cudaSuccess) {
+        cudaGetLastError();
+        return false;
+    }
+    return a.type == cudaMemoryTypeDevice && a.device == dev;
+}
+
+// A caller's device array that kernels may use in place: of this device from
+// the first to the last byte and aligned.  Any other goes through a copy, which
+// takes every kind of memory that the runtime can copy and refuses the rest.
+static bool in_place(const Ctx* c, const void* p, size_t bytes, size_t align)
+{
+    return c->P.values_on_device && (uintptr_t)p % align == 0 && device_address(p) &&
+           device_address((const char*)p + bytes - 1);
+}
+
 // Refresh the compute-type copies of the factors from the FP64 masters.
 static bfc_status refresh_copies(Ctx* c)
 {
@@ -475,7 +496,7 @@ static bfc_status test_error(Ctx* c, int slot)
     if (c->NT <= 0) return BFC_OK;
     const Ops* ops = get_ops(c->fp32, c->r);
     const int nb = (int)std::min<int64_t>(1216, (c->NT + 255) / 256);
-    BFC_TRY(ops->eval(c, c->d_it, c->d_jt, c->NT, nullptr, c->d_tt, c->d_red, nb));
+    BFC_TRY(ops->eval(c, c->d_it, c->d_jt, c->NT, nullptr, c->d_tt, c->d_red, nb, nullptr));
     {
         ProfScope ps(c, "reduce");
         launch_reduce_pairs(c->d_red, nb, c->d_scalars + slot, c->stream);
@@ -821,24 +842,56 @@ bfc_status bfc_eval(bfc_ctx* ctx, int64_t m, const int32_t* i, const int32_t* j,
     if (!c) return BFC_EINVAL;
     if (m < 0 || (m > 0 && (!i || !j || !out))) return fail(c, BFC_EINVAL, "bad eval arguments");
     if (m == 0) return BFC_OK;
-    const size_t ib = ((size_t)m * 4 + 255) / 256 * 256;
-    BFC_TRY(ensure_tmp(c, 2 * ib + (size_t)m * 16 + 256));
-    int32_t* di = (int32_t*)c->d_tmp;
-    int32_t* dj = (int32_t*)((char*)c->d_tmp + ib);
-    double2* dout = (double2*)((char*)c->d_tmp + 2 * ib);
-    BFC_CK(c, cudaMemcpyAsync(di, i, m * 4, in_kind(c), c->stream));
-    BFC_CK(c, cudaMemcpyAsync(dj, j, m * 4, in_kind(c), c->stream));
-    int* dflag = (int*)(c->d_count + 4);
-    BFC_CK(c, cudaMemsetAsync(dflag, 0, sizeof(int), c->stream));
-    launch_check_entries(di, dj, nullptr, m, c->n, dflag, c->stream);
-    int hflag = 0;
-    BFC_CK(c, cudaMemcpyAsync(&hflag, dflag, sizeof(int), cudaMemcpyDeviceToHost, c->stream));
-    BFC_TRY(sync(c));
-    if (hflag) return fail(c, BFC_EINVAL, "an index is outside [0, n)");
+    // Device arrays are used in place (an output that overlaps the indices goes
+    // through scratch).  Host indices of a small call are checked here; otherwise
+    // a kernel checks them and the evaluation does nothing when it found a bad
+    // one, so one wait is enough and nothing is written on an error.
+    const size_t ob = (size_t)m * 16, ib = (size_t)m * 4;
+    auto apart = [&](const int32_t* x) {
+        return (uintptr_t)out + ob <= (uintptr_t)x || (uintptr_t)x + ib <= (uintptr_t)out;
+    };
+    const bool idx = in_place(c, i, ib, 4) && in_place(c, j, ib, 4);
+    const bool direct = idx && in_place(c, out, ob, 16) && apart(i) && apart(j);
+    const bool host_check = !c->P.values_on_device && m <= 65536 && !device_address(i) && !device_address(j);
+    if (host_check)
+        for (int64_t e = 0; e < m; ++e)
+            if (i[e] < 0 || i[e] >= c->n || j[e] < 0 || j[e] >= c->n)
+                return fail(c, BFC_EINVAL, "an index is outside [0, n)");
+    // scratch: [out | i | j]
+    BFC_TRY(ensure_tmp(c, (direct ? 0 : ob) + (idx ? 0 : 2 * ib) + 256));
+    double2* dout = direct ? (double2*)out : (double2*)c->d_tmp;
+    const int32_t *di = i, *dj = j;
+    if (!idx) {
+        int32_t* d = (int32_t*)((char*)c->d_tmp + ob);
+        di = d;
+        dj = d + m;
+        if (host_check && m <= 4096) {
+            int32_t both[8192];   // one copy for both index arrays
+            memcpy(both, i, ib);
+            memcpy(both + m, j, ib);
+            BFC_CK(c, cudaMemcpyAsync(d, both, 2 * ib, cudaMemcpyHostToDevice, c->stream));
+        } else {
+            BFC_CK(c, cudaMemcpyAsync(d, i, ib, in_kind(c), c->stream));
+            BFC_CK(c, cudaMemcpyAsync(d + m, j, ib, in_kind(c), c->stream));
+        }
+    }
+    int* dflag = nullptr;
+    if (!host_check) {
+        dflag = (int*)(c->d_count + 4);
+        BFC_CK(c, cudaMemsetAsync(dflag, 0, sizeof(int), c->stream));
+        launch_check_entries(di, dj, nullptr, m, c->n, dflag, c->stream);
+    }
     const Ops* ops = get_ops(c->fp32, c->r);
     const int nb = (int)std::min<int64_t>(1216 * 4, (m + 255) / 256);
-    BFC_TRY(ops->eval(c, di, dj, m, dout, nullptr, nullptr, nb));
-    BFC_CK(c, cudaMemcpyAsync(out, dout, (size_t)m * 16, out_kind(c), c->stream));
+    BFC_TRY(ops->eval(c, di, dj, m, dout, nullptr, nullptr, nb, dflag));
+    if (dflag) {
+        int hflag = 0;
+        BFC_CK(c, cudaMemcpyAsync(&hflag, dflag, sizeof(int), cudaMemcpyDeviceToHost, c->stream));
+        BFC_TRY(sync(c));
+        if (hflag) return fail(c, BFC_EINVAL, "an index is outside [0, n)");
+        if (direct) return BFC_OK;
+    }
+    BFC_CK(c, cudaMemcpyAsync(out, dout, ob, out_kind(c), c->stream));
     return sync(c);
 }
 
@@ -1038,7 +1091,7 @@ static bfc_status train_rel_err(Ctx* c, double* err)
 {
     const Ops* ops = get_ops(c->fp32, c->r);
     const int nb = (int)std::min<int64_t>(1216, (c->N + 255) / 256);
-    BFC_TRY(ops->eval(c, c->d_i, c->d_j, c->N, nullptr, c->d_t, c->d_red, nb));
+    BFC_TRY(ops->eval(c, c->d_i, c->d_j, c->N, nullptr, c->d_t, c->d_red, nb, nullptr));
     launch_reduce_pairs(c->d_red, nb, c->d_scalars + 12, c->stream);
     BFC_LAUNCH_CHECK(c, "reduce");
     double hs[2];
@@ -1168,9 +1221,8 @@ bfc_status bfc_matvec(bfc_ctx* ctx, int32_t nvec, const double* V, double* U)
     auto up = [](size_t x) { return (x + 255) / 256 * 256; };
     // device vectors are used where they are if the kernels' 16-byte accesses
     // allow (V is read by the first kernel only, U written by the last)
-    const bool dev_v = c->P.values_on_device && (uintptr_t)V % 16 == 0;
-    const bool dev_u = c->P.values_on_device && (uintptr_t)U % 16 == 0;
     const size_t bytes = (size_t)c->n * nvec * 16, vb = up(bytes);
+    const bool dev_v = in_place(c, V, bytes, 16), dev_u = in_place(c, U, bytes, 16);
     const size_t yb = up((size_t)c->S * nvec * c->r * c->vsz);
     BFC_TRY(ensure_tmp(c, (dev_v ? 0 : vb) + (dev_u ? 0 : vb) + 2 * yb));
     char* base = (char*)c->d_tmp;

@@ -983,8 +983,10 @@ __global__ void __launch_bounds__(256)
 k_eval(const int32_t* __restrict__ ii, const int32_t* __restrict__ jj, int64_t M,
        const typename cvec<T>::type* __restrict__ z1, const typename cvec<T>::type* __restrict__ Z,
        const typename cvec<T>::type* __restrict__ zL, int L, int b, int64_t S,
-       double2* __restrict__ out, const double2* __restrict__ tref, double* __restrict__ part)
+       double2* __restrict__ out, const double2* __restrict__ tref, double* __restrict__ part,
+       const int* __restrict__ skip)
 {
+    if (skip && *skip) return;   // an index was found out of range before this kernel
     // A group of GS >= R lanes evaluates one entry: lane c keeps h_c and
     // forms column c of h^T Z^{m}(k), so the group reads each slice row as
     // one contiguous segment; h is passed around the group by shuffles.  The

@@ -10,7 +10,8 @@ struct Ops {
     bfc_status (*configure)(Ctx*);
     bfc_status (*sweep)(Ctx*);
     bfc_status (*grad)(Ctx*, double2*, double*);
-    bfc_status (*eval)(Ctx*, const int32_t*, const int32_t*, int64_t, double2*, const double2*, double*, int);
+    bfc_status (*eval)(Ctx*, const int32_t*, const int32_t*, int64_t, double2*, const double2*, double*, int,
+                       const int* skip);
     size_t (*record_bytes)(int64_t n, int64_t S);
     size_t (*group_record_bytes)();
 };

@@ -266,12 +266,13 @@ template <typename T, int R> struct Path {
     }
 
     // Entry evaluation of M pairs (device arrays); out and/or residual partials.
+    // skip (may be NULL): a device word; nothing is read or written unless it is 0.
     static bfc_status eval(Ctx* c, const int32_t* di, const int32_t* dj, int64_t M, double2* out,
-                           const double2* tref, double* part, int nblk)
+                           const double2* tref, double* part, int nblk, const int* skip)
     {
         ProfScope ps(c, "eval");
         k_eval<T, R><<<nblk, 256, 0, c->stream>>>(di, dj, M, (const V*)c->z1t, (const V*)c->Zt, (const V*)c->zLt,
-                                                   c->L, c->b, c->S, out, tref, part);
+                                                   c->L, c->b, c->S, out, tref, part, skip);
         BFC_LAUNCH_CHECK(c, "eval");
         return BFC_OK;
     }
