@@ -65,7 +65,7 @@ TC_GRAM_TRAFFIC = {"source": "paper_2510_17734_gb300/csrc/bfc_gram_tc.cuh", "sha
 # DRAM counters of k_mid_solve at the n = 65536 workload itself (ncu, one-pass
 # metrics, mean of three launches of the first sweep: 3,774,874 entries, 8192
 # slices per level), valid for the kernel source with this sha256 prefix
-SOLVE_TRAFFIC = {"source": "paper_2510_17734_gb300/csrc/bfc_solve.cuh", "sha": "e7fd6aa90b7ac4e2",
+SOLVE_TRAFFIC = {"source": "paper_2510_17734_gb300/csrc/bfc_solve.cuh", "sha": "60826c85247253b6",
                  # the kernel and the device functions it calls (KPair ... k_mid_solve)
                  "span": ("// Arithmetic on pairs of neighbouring k of two rows",
                           "// FP64 fallback of the precision form: a CTA"),

@@ -120,8 +120,11 @@ template <typename T, int R> struct SolveCfg {
     typedef Rec<T, R> RC;
     // Warps of a slice's CTA: shared memory holds 9 records of rank 8 per SM, 2
     // of rank 12, and the diagonal blocks and triangular solves are chains of
-    // one warp
-    static constexpr int NW = R <= 8 ? 2 : R <= 10 ? 4 : 8;
+    // one warp.  FP64 at r = 6: the entries' left update is most of the work, 2
+    // warps leave its loads exposed and 8 lose the CTAs per SM that overlap
+    // (S = 512: 208 / 209 / 281 us per launch with 2 / 4 / 8, S = 128: 316 / 204
+    // / 199 us; 256 and 360 us with 2 warps and 4 x 4 tiles)
+    static constexpr int NW = R <= 8 ? (MIXED ? 2 : 4) : R <= 10 ? 4 : 8;
     static constexpr int NTH = 32 * NW;
     static constexpr int MINB = MIXED ? 512 / NTH : 1;   // 128 registers in the precision form
     static constexpr int FBT = 128;      // threads of a k_mid_fallback CTA
@@ -368,6 +371,54 @@ template <typename T, int R> __device__ __forceinline__ void solve_y_tile(T* Lm,
     st4(dp + 8, b);
 }
 
+// FP64: a 2 x 2 tile (I, Jt) of the trailing matrix of panel J.  A warp
+// instruction takes the FP64 pipe as long with one active lane as with 32, and
+// 4 x 4 tiles leave most lanes of the later panels idle.
+template <int R> __device__ __forceinline__ void solve_tile2(double* Lm, int J, int I, int Jt)
+{
+    typedef Rec<double, R> RC;
+    const double* xp = Lm + RC::row(J, 8 + 2 * I);
+    const double* lp = Lm + RC::row(J, 8 + 2 * Jt);
+    double sr[2][2] = {}, si[2][2] = {};
+#pragma unroll
+    for (int h = 0; h < 4; ++h) {
+        double2 lr[2], li[2];
+#pragma unroll
+        for (int v = 0; v < 2; ++v) {
+            lr[v] = *reinterpret_cast<const double2*>(lp + 16 * v + 2 * h);
+            li[v] = *reinterpret_cast<const double2*>(lp + 16 * v + 8 + 2 * h);
+        }
+#pragma unroll
+        for (int u = 0; u < 2; ++u) {
+            const double2 xr = *reinterpret_cast<const double2*>(xp + 16 * u + 2 * h);
+            const double2 xi = *reinterpret_cast<const double2*>(xp + 16 * u + 8 + 2 * h);
+#pragma unroll
+            for (int v = 0; v < 2; ++v) {
+                sr[u][v] += xr.x * lr[v].x;
+                si[u][v] += xi.x * lr[v].x;
+                sr[u][v] += xi.x * li[v].x;
+                si[u][v] -= xr.x * li[v].x;
+                sr[u][v] += xr.y * lr[v].y;
+                si[u][v] += xi.y * lr[v].y;
+                sr[u][v] += xi.y * li[v].y;
+                si[u][v] -= xr.y * li[v].y;
+            }
+        }
+    }
+    const int c = 8 * J + 8 + 2 * Jt, Jd = c >> 3, r0 = 8 * J + 8 + 2 * I;
+    double* dp = Lm + RC::row(Jd, r0 - 8 * Jd) + (c & 7);
+#pragma unroll
+    for (int u = 0; u < 2; ++u) {
+        if (r0 + u <= RC::D) {
+            double2* a = reinterpret_cast<double2*>(dp + 16 * u);
+            double2* b = reinterpret_cast<double2*>(dp + 16 * u + 8);
+            const double2 av = *a, bv = *b;
+            *a = make_double2(av.x - sr[u][0], av.y - sr[u][1]);
+            *b = make_double2(bv.x - si[u][0], bv.y - si[u][1]);
+        }
+    }
+}
+
 // Factorization of the record in Lm by all threads of the CTA.  In the
 // precision form the diagonal blocks end inverted, in FP64 as L (1 / L_cc in
 // the imaginary slot of the diagonal).  False (CTA-uniform) when a pivot is
@@ -401,13 +452,29 @@ __device__ __forceinline__ bool solve_chol(T* Lm, T tol, volatile int* fail, int
         // tile columns hold columns < D; the row of conj(y) is in the last tile
         // row, or (D a multiple of 4) has tiles of one row, by the last threads
         // (as full tiles they would take a round of their own)
+        auto tri = [](int x) {   // the row of element x of a packed lower triangle
+            int I = (int)((sqrtf(8.f * (float)x + 1.f) - 1.f) * 0.5f);
+            if (I * (I + 1) / 2 > x) --I;
+            if ((I + 1) * (I + 2) / 2 <= x) ++I;
+            return I;
+        };
+        if constexpr (sizeof(T) == 8) {
+            // columns 8J + 8 .. D - 1 in pairs, rows to D: with an even number of
+            // columns the row of conj(y) is a row of tiles of its own
+            const int M = max(0, D - 8 * J - 8), mc = (M + 1) / 2;
+            const int nt = mc * (mc + 1) / 2 + (M % 2 == 0 ? mc : 0);
+            for (int x = tid; x < nt; x += nthr) {
+                const int I = tri(x);
+                solve_tile2<R>(Lm, J, I, x - I * (I + 1) / 2);
+            }
+            __syncthreads();
+            continue;
+        }
         const int mc = max(0, (D - 8 * J - 5) / 4), nt = mc * (mc + 1) / 2;
         if constexpr (D % 4 == 0)
             for (int x = nthr - 1 - tid; x < mc; x += nthr) solve_y_tile<T, R>(Lm, J, x);
         for (int x = tid; x < nt; x += nthr) {
-            int I = (int)((sqrtf(8.f * (float)x + 1.f) - 1.f) * 0.5f);
-            if (I * (I + 1) / 2 > x) --I;
-            if ((I + 1) * (I + 2) / 2 <= x) ++I;
+            const int I = tri(x);
             solve_tile<T, R>(Lm, J, I, x - I * (I + 1) / 2);
         }
         __syncthreads();
