@@ -214,9 +214,9 @@ __global__ void k_env_init(typename cvec<T>::type* __restrict__ WL,
 // Normal equations of Alg. 1 (complex form): for a block (one fiber of S^1 or
 // S^{L+2}, or one slice of a middle factor) with design vectors a_e,
 //   K = sum conj(a_e) a_e^T + lambda I,   y = sum conj(a_e) t_e,   K s = y.
-// Every kernel that accumulates K and y writes them, packed lower-triangular
-// (element (p, q), p >= q, at tri(p, q)) followed by y, to a per-block
-// record; a solve kernel then factors and solves.
+// Every kernel that accumulates K and y writes them to a per-block record; a
+// solve kernel then factors and solves.  Outer factors: packed lower-triangular
+// (element (p, q), p >= q, at tri(p, q)) followed by y; middle factors: Rec.
 //
 // FP64 on this GPU runs at 1/64 of the FP32 rate and a warp-wide FP64
 // instruction holds an SM sub-partition's FP64 pipe for tens of cycles

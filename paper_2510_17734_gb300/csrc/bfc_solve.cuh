@@ -10,7 +10,7 @@
 //  (2) a thread per row solves the panel rows below it, conj(y) among them;
 //  (3) threads own 4 x 4 tiles of the trailing matrix: 8 rows of the panel are
 //      read as 16-byte pieces for 64 complex multiply-adds, done as packed
-//      pairs of neighbouring k (f32x2 in the precision form).
+//      pairs of neighbouring k (f32x2 in the precision form; 2 x 2 tiles in FP64).
 // The row of conj(y) ends as conj(z), z the forward solution, so only the
 // backward substitution is left; the refinement's solves run in warp 0, block
 // by block, with the inverted diagonal blocks.
@@ -21,7 +21,7 @@
 // line throughput 61 %).  Measured, all middle levels of a sweep, against the
 // kernel before (one warp per slice on a packed triangle, a lane per row):
 // n = 65536, r = 8 6.48 -> 5.74 ms; n = 4096, r = 12 8.8 -> 3.1 ms; n = 4096,
-// r = 6, FP64 3.75 -> 2.0 ms; n = 3072, r = 5 0.47 -> 0.38 ms.  One warp per
+// r = 6, FP64 3.75 -> 1.67 ms; n = 3072, r = 5 0.47 -> 0.38 ms.  One warp per
 // slice: 7.3 ms at n = 65536, three: 6.8 (r = 12: 7.2 and 4.0, eight: 3.3).
 // Also slower or no faster: lanes sharing the rows of the left update (the
 // lines of a load or store fewer, the shuffles more), two lanes per row of the
