@@ -106,8 +106,7 @@ typedef struct {
     int32_t gram_impl;      /* per-slice normal equations of the middle
                                levels.  0 = automatic: for r >= 2, a
                                level whose row (or column) groups are few
-                               against its entries (below group_ratio of
-                               them) runs the grouped Gram (the entries of one row
+                               against its entries (group_ratio) runs the grouped Gram (the entries of one row
                                / column of a slice share an environment, so
                                the sums are taken per group and the Gram is
                                the sum of Kronecker products of the group
@@ -123,12 +122,14 @@ typedef struct {
     int32_t lr2bf_oversample; /* oversampling p of Alg. 2 for init_kind 2
                                (0 selects 5); r + p <= 32                   */
     double group_ratio;     /* gram_impl 0: groups-per-entry threshold of the
-                               grouped Gram.  0 selects the default (next to
-                               the tensor-core kernel 0.1 (8 / r)^4, at most
-                               0.9; next to the CUDA-core one 0.9, in the
-                               precision form only levels whose slices span
-                               at least r rows / columns); < 0 never groups;
-                               > 0 is used as given                             */
+                               grouped Gram.  0 selects the default: next to
+                               the tensor-core kernel the levels where grouping
+                               saves time by a model of both (entries, groups
+                               and slices of the level, r); next to the
+                               CUDA-core one 0.9, in the precision form only
+                               levels whose slices span at least r rows /
+                               columns.  < 0 never groups; > 0 is used as
+                               given                                        */
 } bfc_params;
 
 typedef struct {

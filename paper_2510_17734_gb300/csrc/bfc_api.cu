@@ -192,6 +192,44 @@ struct Inputs {
     cudaMemcpyKind kind;
 };
 
+// Whether a middle level whose entries form G row / column groups (slices of
+// loc rows / columns) runs the grouped Gram.  group_ratio > 0: below that many
+// groups per entry.  Default:
+//  * next to the tensor-core kernel, where a model of both says that grouping
+//    saves time.  Whole-chip ns per slice: 0.105 per entry more on the tensor
+//    cores, `group` per group and the difference `base` of the fixed parts for
+//    the grouped kernel (rank 2 .. 8; ranks 3 .. 6 pay for the sum over thread
+//    groups), from sweeps with -1, 0.05 .. 0.9 of the entries as the line at
+//    n = 256 .. 32768, 130 .. 1037 entries per slice.  Examples, ms for all
+//    levels with none / all / the model's levels grouped: n = 32768, b = 8,
+//    r = 4 2.78 / 4.44 / 2.99; r = 7 4.43 / 5.84 / 3.55; n = 4096, b = 16,
+//    r = 5 0.85 / 0.58 / 0.58; n = 65536, b = 16, r = 8: four levels.  Its two
+//    kernels cost 5 us more than one.  At ranks 4 and 8 also below 0.1 groups
+//    per entry, for the compensated sums: n = 32768, r = 4, Radon data, error of
+//    the factors after a sweep 7.2e-7, and 8.5e-7 without those levels;
+//  * next to the per-entry CUDA-core kernel, whose work per entry is that of a
+//    group, below 0.9 groups per entry.  In the precision form (r > 8) not
+//    where slices have fewer than r rows (columns): they are rank deficient and
+//    solved at the ridge floor, and the coherent rounding of a few large group
+//    terms (2-norm error of K 1.8 times that of k_mid_gram) makes more of them
+//    indefinite (n = 4096, b = 4, r = 12: 24 of 20,480 systems of a sweep kept
+//    their old slice, with k_mid_gram 2).
+static bool group_level(const Ctx* c, int64_t G, int64_t loc)
+{
+    if (c->r < 2 || c->P.gram_impl != 0) return false;
+    const double g = (double)G, N = (double)c->N, S = (double)c->S, given = c->P.group_ratio;
+    if (given != 0.0) return g < given * N;
+    if (c->gram_tc) {
+        static const double base[7] = {1.0, -12.0, -25.0, -49.0, -8.5, 19.0, 19.0};
+        static const double group[7] = {0.025, 0.1, 0.1, 0.375, 0.4, 1.0, 1.25};
+        const double gain = base[c->r - 2] * S + 0.105 * N - group[c->r - 2] * g;
+        // with fewer slices than SMs both leave the rest idle
+        return gain * std::max(1.0, 152.0 / S) > 5000.0 || ((c->r == 4 || c->r == 8) && g < 0.1 * N);
+    }
+    if (c->fp32 && loc < c->r) return false;
+    return g < 0.9 * N;
+}
+
 static bfc_status build(Ctx* c, const Inputs& in)
 {
     const int64_t N = c->N, n = c->n, S = c->S;
@@ -295,14 +333,7 @@ static bfc_status build(Ctx* c, const Inputs& in)
             GroupLevel& gl = c->grp[l];
             gl.by_col = by_col;
             gl.ngroups = G;
-            const double ratio = c->gram_tc ? c->grp_max_ratio : c->grp_cuda_ratio;
-            // slices of fewer than r rows (columns) are rank deficient and solved
-            // at the ridge floor: there the coherent rounding of a few large
-            // group terms (2-norm error of K 1.8 times that of k_mid_gram) makes
-            // more of them indefinite (n = 4096, b = 4, r = 12: 24 of 20,480
-            // systems of a sweep kept their old slice, with k_mid_gram 2)
-            const bool floor_bound = c->fp32 && c->r > 8 && loc < c->r && !(c->P.group_ratio > 0.0);
-            if (c->r >= 2 && c->P.gram_impl == 0 && !floor_bound && (double)G < ratio * (double)N) {
+            if (group_level(c, G, loc)) {
                 gst.push_back((int32_t)N);
                 // the largest entry range of a k_group_sums block (its shared-memory staging)
                 const int64_t gpb = 128 / c->r;
@@ -425,18 +456,6 @@ static bfc_status create_impl(const bfc_params* params, const Inputs& in, bfc_ct
     c->vsz = c->fp32 ? 8 : 16;
     c->ridge = p.ridge_rel > 0.0 ? p.ridge_rel : (p.ridge_rel == 0.0 && c->fp32 ? 9.5367431640625e-07 : 0.0);
     c->gram_tc = c->fp32 && p.gram_impl != 1 && p.r <= 8;
-    // grouped Gram (gram_impl 0) at the middle levels with few row / column
-    // groups per entry.  Against the per-entry CUDA-core kernel, whose work per
-    // entry is that of a group, below 0.9.  Against the tensor-core kernel,
-    // which costs the same per entry at every rank (it pads to rank 8), the
-    // line moves with the r^4 of a group's Kronecker update: 0.1 at rank 8 (at
-    // n = 65536 a level of 0.07 groups per entry is faster grouped, one of 0.14
-    // on the tensor cores), times (8 / r)^4, at most 0.9
-    double tc_ratio = 0.1;
-    for (int q = 0; q < 4; ++q) tc_ratio *= 8.0 / p.r;
-    tc_ratio = std::min(std::max(tc_ratio, 0.1), 0.9);
-    c->grp_max_ratio = p.group_ratio > 0.0 ? p.group_ratio : (p.group_ratio < 0.0 ? 0.0 : tc_ratio);
-    c->grp_cuda_ratio = p.group_ratio > 0.0 ? p.group_ratio : (p.group_ratio < 0.0 ? 0.0 : 0.9);
     bfc_status st = build(c, in);
     if (st != BFC_OK) {
         g_create_err = c->err;
@@ -784,8 +803,7 @@ bool level_grouped(const Ctx* c, int m)
     if (m < 1 || m > c->L || (int)c->grp.size() <= m) return false;
     const GroupLevel& gl = c->grp[m];
     if (!gl.gstart) return false;   // level order not grouped at build time
-    const double ratio = c->gram_tc ? c->grp_max_ratio : c->grp_cuda_ratio;
-    return gl.ngroups > 0 && (double)gl.ngroups < ratio * (double)c->N;
+    return gl.ngroups > 0;
 }
 
 }  // namespace bfc

@@ -69,9 +69,6 @@ struct Ctx {
     std::vector<int32_t*> perm;  // L+2: entry index at each position of order l
     std::vector<GroupLevel> grp; // L+2: row / column groups of the middle levels (empty otherwise)
     void* grec = nullptr;        // group records [s | M | v] of the level being solved (grouped Gram)
-    double grp_max_ratio = 0.0;  // a middle level's Gram runs per group when groups / entries < this
-                                 // (next to the tensor-core kernel)
-    double grp_cuda_ratio = 0.0; // the same next to the per-entry CUDA-core kernel
 
     // environments (compute type): W[l] (l = 0..L) in order l, two H buffers
     void* W = nullptr;

@@ -54,13 +54,20 @@ def test_grouped_sweep_parity(r, few, prec):
 
 @pytest.mark.parametrize("r", [3, 5, 6, 7, 10, 12])
 def test_default_grouping_by_rank(r):
-    """Default thresholds: every level whose groups are below 0.9 of the entries
-    in FP64 and above rank 8; 0.1 (8 / r)^4 of them, at most 0.9, next to the
-    tensor-core kernel."""
+    """Default rule: every level whose groups are below 0.9 of the entries in
+    FP64 and above rank 8; next to the tensor-core kernel the levels for which
+    the cost model (ns per slice, entry and group by rank) sees a gain."""
     n, L, b, lam, i, j, t, _ = problem(r, False)
+    S = 2 << L
     for prec in (bfc.PREC_FP64, bfc.PREC_C64):
-        ratio = 0.9 if prec == bfc.PREC_FP64 or r > 8 else min(0.9, max(0.1, 0.1 * (8 / r) ** 4))
         with bfc.Completion(n, L, b, r, lam, i, j, t, prec=prec) as c:
             for m in range(1, L + 1):
                 groups, on = c.level_groups(m)
-                assert on == (groups < ratio * len(i))
+                if prec == bfc.PREC_FP64 or r > 8:
+                    want = groups < 0.9 * len(i)
+                else:
+                    base = (1.0, -12.0, -25.0, -49.0, -8.5, 19.0, 19.0)[r - 2]
+                    per = (0.025, 0.1, 0.1, 0.375, 0.4, 1.0, 1.25)[r - 2]
+                    want = (base * S + 0.105 * len(i) - per * groups) * max(1.0, 152.0 / S) > 5000.0
+                    want = want or (r in (4, 8) and groups < 0.1 * len(i))
+                assert on == want
