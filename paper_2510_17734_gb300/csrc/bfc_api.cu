@@ -144,6 +144,18 @@ static bool device_address(const void* p)
     return a.type == cudaMemoryTypeDevice && a.device == dev;
 }
 
+// p can be read by the host: not device memory of any device, nor the device's
+// address of page-locked memory.
+static bool host_address(const void* p)
+{
+    cudaPointerAttributes a;
+    if (cudaPointerGetAttributes(&a, p) != cudaSuccess) {
+        cudaGetLastError();
+        return false;
+    }
+    return a.type != cudaMemoryTypeDevice && (a.type != cudaMemoryTypeHost || a.hostPointer == p);
+}
+
 // A caller's device array that kernels may use in place: of this device from
 // the first to the last byte and aligned.  Any other goes through a copy, which
 // takes every kind of memory that the runtime can copy and refuses the rest.
@@ -861,20 +873,30 @@ bfc_status bfc_eval(bfc_ctx* ctx, int64_t m, const int32_t* i, const int32_t* j,
     if (m < 0 || (m > 0 && (!i || !j || !out))) return fail(c, BFC_EINVAL, "bad eval arguments");
     if (m == 0) return BFC_OK;
     // Device arrays are used in place (an output that overlaps the indices goes
-    // through scratch).  Host indices of a small call are checked here; otherwise
-    // a kernel checks them and the evaluation does nothing when it found a bad
-    // one, so one wait is enough and nothing is written on an error.
+    // through scratch).  Host indices of a small call are copied and checked
+    // here, once the stream's pending work (which may write them) is done;
+    // otherwise a kernel checks them and the evaluation does nothing when it
+    // found a bad one, so one wait is enough and nothing is written on an error.
+    // The line lies at 8192 pairs (n = 4096, r = 6, complex64; checked here / by a
+    // kernel): 4096 pairs 58 / 73 us, 8000 pairs 72 / 75 us, 65536 pairs 140 / 97 us.
     const size_t ob = (size_t)m * 16, ib = (size_t)m * 4;
     auto apart = [&](const int32_t* x) {
         return (uintptr_t)out + ob <= (uintptr_t)x || (uintptr_t)x + ib <= (uintptr_t)out;
     };
     const bool idx = in_place(c, i, ib, 4) && in_place(c, j, ib, 4);
     const bool direct = idx && in_place(c, out, ob, 16) && apart(i) && apart(j);
-    const bool host_check = !c->P.values_on_device && m <= 65536 && !device_address(i) && !device_address(j);
-    if (host_check)
-        for (int64_t e = 0; e < m; ++e)
-            if (i[e] < 0 || i[e] >= c->n || j[e] < 0 || j[e] >= c->n)
-                return fail(c, BFC_EINVAL, "an index is outside [0, n)");
+    const bool host_check = !c->P.values_on_device && m <= 8192 && host_address(i) && host_address(j);
+    int32_t both[16384];   // [i | j] of a small call: what is checked is what is copied, in one piece
+    if (host_check) {
+        if (cudaStreamQuery(c->stream) != cudaSuccess) {
+            cudaGetLastError();   // (not ready)
+            BFC_TRY(sync(c));
+        }
+        memcpy(both, i, ib);
+        memcpy(both + m, j, ib);
+        for (int64_t e = 0; e < 2 * m; ++e)
+            if (both[e] < 0 || both[e] >= c->n) return fail(c, BFC_EINVAL, "an index is outside [0, n)");
+    }
     // scratch: [out | i | j]
     BFC_TRY(ensure_tmp(c, (direct ? 0 : ob) + (idx ? 0 : 2 * ib) + 256));
     double2* dout = direct ? (double2*)out : (double2*)c->d_tmp;
@@ -883,10 +905,7 @@ bfc_status bfc_eval(bfc_ctx* ctx, int64_t m, const int32_t* i, const int32_t* j,
         int32_t* d = (int32_t*)((char*)c->d_tmp + ob);
         di = d;
         dj = d + m;
-        if (host_check && m <= 4096) {
-            int32_t both[8192];   // one copy for both index arrays
-            memcpy(both, i, ib);
-            memcpy(both + m, j, ib);
+        if (host_check) {
             BFC_CK(c, cudaMemcpyAsync(d, both, 2 * ib, cudaMemcpyHostToDevice, c->stream));
         } else {
             BFC_CK(c, cudaMemcpyAsync(d, i, ib, in_kind(c), c->stream));
