@@ -1502,7 +1502,7 @@ k_grad_mid(const typename cvec<T>::type* __restrict__ H, const typename cvec<T>:
                 if (n.k != c.k) fetch_z(n);
             }
             bool have = false;
-            if (issued >> b & 1u) {
+            if (use_bulk && (issued >> b & 1u)) {   // (given up on once: no second wait before the end)
                 bool done = false;
                 for (uint32_t it = 0; it < wait_limit && !done; ++it) {
                     uint32_t ok;
