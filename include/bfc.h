@@ -129,7 +129,11 @@ typedef struct {
                                CUDA-core one 0.9, in the precision form only
                                levels whose slices span at least r rows /
                                columns.  < 0 never groups; > 0 is used as
-                               given                                        */
+                               given.  The group records of a level take at
+                               most 256 MiB, 1/16 of the right environments
+                               or the largest slice's, whichever is most; a
+                               problem that does not fit the memory with
+                               grouped levels is created without             */
 } bfc_params;
 
 typedef struct {

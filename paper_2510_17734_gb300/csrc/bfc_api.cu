@@ -228,7 +228,7 @@ struct Inputs {
 //    their old slice, with k_mid_gram 2).
 static bool group_level(const Ctx* c, int64_t G, int64_t loc)
 {
-    if (c->r < 2 || c->P.gram_impl != 0) return false;
+    if (c->r < 2 || c->P.gram_impl != 0 || c->no_groups) return false;
     const double g = (double)G, N = (double)c->N, S = (double)c->S, given = c->P.group_ratio;
     if (given != 0.0) return g < given * N;
     if (c->gram_tc) {
@@ -241,6 +241,35 @@ static bool group_level(const Ctx* c, int64_t G, int64_t loc)
     if (c->fp32 && loc < c->r) return false;
     return g < 0.9 * N;
 }
+
+// The slices of a grouped level in consecutive batches of about equal numbers
+// of groups, at most `cap` of them (a slice with more has its own).  gst: first
+// entry of each group, then N; gsg: first group of each slice, then G; gpb:
+// groups of a k_group_sums block.
+static std::vector<GroupBatch> group_batches(const std::vector<int32_t>& gst, const std::vector<int32_t>& gsg,
+                                             int64_t cap, int64_t gpb)
+{
+    const int64_t S = (int64_t)gsg.size() - 1, G = gsg[S];
+    const int64_t count = std::max<int64_t>(1, (G + cap - 1) / cap), per = (G + count - 1) / count;
+    std::vector<GroupBatch> out;
+    for (int64_t k = 0; k < S;) {
+        GroupBatch b;
+        b.k0 = (int32_t)k;
+        b.g0 = gsg[k];
+        for (++k; k < S && (gsg[k] == G || (gsg[k] - b.g0 < per && gsg[k + 1] - b.g0 <= cap));) ++k;
+        b.k1 = (int32_t)k;
+        b.g1 = gsg[k];
+        for (int64_t g = b.g0; g < b.g1; g += gpb)
+            b.max_block = std::max(b.max_block, (int64_t)gst[std::min(g + gpb, b.g1)] - gst[g]);
+        out.push_back(b);
+    }
+    return out;
+}
+
+// Group records of a level, unless its largest slice or 1/16 of the right
+// environments take more.  Without a bound a level of 0.9 groups per entry at r
+// = 12 needs as much memory as all right environments.
+static const size_t GROUP_BYTES = (size_t)256 << 20;
 
 static bfc_status build(Ctx* c, const Inputs& in)
 {
@@ -310,6 +339,11 @@ static bfc_status build(Ctx* c, const Inputs& in)
     c->prv.assign(L + 1, nullptr);
     c->grp.assign(NL, GroupLevel{});
     std::vector<uint32_t> hkeys;
+    const Ops* ops = get_ops(c->fp32, r);
+    // groups whose records fill the buffer of a level: GROUP_BYTES, or 1/16 of
+    // the right environments where that is more
+    const size_t wbytes = (size_t)(L + 1) * N * r * c->vsz, grec_bytes = std::max<size_t>(ops->group_record_bytes(), 1);
+    const int64_t batch_groups = (int64_t)(std::max(GROUP_BYTES, wbytes / 16) / grec_bytes);
     for (int l = 0; l < NL; ++l) {
         const int64_t K = (l == 0 || l == L + 1) ? n : S;
         BFC_TRY(dalloc(c, (void**)&perm[l], N * 4, "perm"));
@@ -347,15 +381,12 @@ static bfc_status build(Ctx* c, const Inputs& in)
             gl.ngroups = G;
             if (group_level(c, G, loc)) {
                 gst.push_back((int32_t)N);
-                // the largest entry range of a k_group_sums block (its shared-memory staging)
-                const int64_t gpb = 128 / c->r;
-                for (int64_t g0 = 0; g0 < G; g0 += gpb)
-                    gl.max_block = std::max(gl.max_block, (int64_t)gst[std::min(g0 + gpb, G)] - gst[g0]);
                 int64_t g = 0;
                 for (int64_t k = 0; k <= S; ++k) {
                     while (g < G && (int64_t)(hkeys[gst[g]] / (uint64_t)loc) < k) ++g;
                     gsg[k] = (int32_t)g;
                 }
+                gl.batches = group_batches(gst, gsg, batch_groups, 128 / r);
                 BFC_TRY(dalloc(c, (void**)&gl.gstart, (size_t)(G + 1) * 4, "group offsets"));
                 BFC_TRY(dalloc(c, (void**)&gl.gseg, (size_t)(S + 1) * 4, "slice group offsets"));
                 BFC_CK(c, cudaMemcpyAsync(gl.gstart, gst.data(), (size_t)(G + 1) * 4, cudaMemcpyHostToDevice,
@@ -420,14 +451,13 @@ static bfc_status build(Ctx* c, const Inputs& in)
         c->Zt = c->Zd;
         c->zLt = c->zLd;
     }
-    const Ops* ops = get_ops(c->fp32, r);
     BFC_TRY(dalloc(c, &c->rec, ops->record_bytes(n, S), "normal-equation records"));
     // group records [s | M | v] of the grouped Gram: sized for the largest
-    // level whose order was grouped
+    // batch of a level whose order was grouped
     int64_t gmax = 0;
     for (const GroupLevel& gl : c->grp)
-        if (gl.gstart) gmax = std::max(gmax, gl.ngroups);
-    if (gmax > 0) BFC_TRY(dalloc(c, &c->grec, (size_t)gmax * ops->group_record_bytes(), "group records"));
+        for (const GroupBatch& gb : gl.batches) gmax = std::max(gmax, gb.g1 - gb.g0);
+    if (gmax > 0) BFC_TRY(dalloc(c, &c->grec, (size_t)gmax * grec_bytes, "group records"));
     if (c->fp32 && L > 0) BFC_TRY(dalloc(c, (void**)&c->fblist, (size_t)S * sizeof(int32_t), "fallback list"));
     BFC_TRY(ops->configure(c));
     return sync(c);
@@ -454,28 +484,36 @@ static bfc_status create_impl(const bfc_params* params, const Inputs& in, bfc_ct
     if (in.ntest < 0 || in.ntest >= ((int64_t)1 << 31) - 1) return fail(nullptr, BFC_EINVAL, "bad ntest");
     if (!in.i || !in.j || !in.t) return fail(nullptr, BFC_EINVAL, "null training data");
     if (in.ntest > 0 && (!in.it || !in.jt || !in.tt)) return fail(nullptr, BFC_EINVAL, "null test data");
-    Ctx* c = new Ctx();
-    c->P = p;
-    c->n = p.n;
-    c->L = p.L;
-    c->b = p.b;
-    c->r = p.r;
-    c->S = (int64_t)1 << (p.L + 1);
-    c->N = in.nnz;
-    c->NT = in.ntest;
-    c->Pn = bfc_num_params(p.n, p.L, p.b, p.r);
-    c->fp32 = p.prec == BFC_PREC_C64_FP64SOLVE;
-    c->vsz = c->fp32 ? 8 : 16;
-    c->ridge = p.ridge_rel > 0.0 ? p.ridge_rel : (p.ridge_rel == 0.0 && c->fp32 ? 9.5367431640625e-07 : 0.0);
-    c->gram_tc = c->fp32 && p.gram_impl != 1 && p.r <= 8;
-    bfc_status st = build(c, in);
-    if (st != BFC_OK) {
+    // where the memory does not suffice with grouped levels, once more without
+    // (their offsets and records are all that the per-entry kernels do without)
+    for (const bool no_groups : {false, true}) {
+        Ctx* c = new Ctx();
+        c->P = p;
+        c->n = p.n;
+        c->L = p.L;
+        c->b = p.b;
+        c->r = p.r;
+        c->S = (int64_t)1 << (p.L + 1);
+        c->N = in.nnz;
+        c->NT = in.ntest;
+        c->Pn = bfc_num_params(p.n, p.L, p.b, p.r);
+        c->fp32 = p.prec == BFC_PREC_C64_FP64SOLVE;
+        c->vsz = c->fp32 ? 8 : 16;
+        c->ridge = p.ridge_rel > 0.0 ? p.ridge_rel : (p.ridge_rel == 0.0 && c->fp32 ? 9.5367431640625e-07 : 0.0);
+        c->gram_tc = c->fp32 && p.gram_impl != 1 && p.r <= 8;
+        c->no_groups = no_groups;
+        const bfc_status st = build(c, in);
+        if (st == BFC_OK) {
+            *out = (bfc_ctx*)c;
+            return BFC_OK;
+        }
+        bool grouped = false;
+        for (const GroupLevel& gl : c->grp) grouped = grouped || !gl.batches.empty();
         g_create_err = c->err;
         bfc_destroy((bfc_ctx*)c);
-        return st;
+        if (st != BFC_ENOMEM || !grouped) return st;
     }
-    *out = (bfc_ctx*)c;
-    return BFC_OK;
+    return BFC_ENOMEM;
 }
 
 // ---------------------------------------------------------------- sweeps

@@ -401,7 +401,8 @@ template <typename V, int TT> __device__ __forceinline__ void load_t(V (&d)[TT],
 }
 
 // Per-slice normal equations from the group records of k_group_sums (NSPLIT
-// blocks per slice; the grid is a multiple of NSPLIT, grid-stride).  Chunks of CG records stream through an
+// blocks per slice; the grid is a multiple of NSPLIT, grid-stride).  grec starts
+// with group gbase of the level, the first of the S slices.  Chunks of CG records stream through an
 // NST-stage shared-memory ring by 16-byte cp.async copies; per group, the
 // shared side's outer product is formed in registers (conj(s_a) s_a' for row
 // groups; conj(s_c) s_c' for column groups) and multiplied with the other
@@ -410,7 +411,7 @@ template <typename V, int TT> __device__ __forceinline__ void load_t(V (&d)[TT],
 // the slice's sum).
 template <typename T, int R, int BY_COL>
 __global__ void __launch_bounds__(GrpCfg<T, R>::NTH, GrpCfg<T, R>::MINB)
-k_mid_gram_grp(const typename cvec<T>::type* __restrict__ grec, const int32_t* __restrict__ gseg,
+k_mid_gram_grp(const typename cvec<T>::type* __restrict__ grec, const int32_t* __restrict__ gseg, int gbase,
                T* __restrict__ rec, int S)
 {
     typedef typename cvec<T>::type V;
@@ -447,7 +448,7 @@ k_mid_gram_grp(const typename cvec<T>::type* __restrict__ grec, const int32_t* _
     };
 
     for (int k = blockIdx.x / C::NSPLIT; k < S; k += gridDim.x / C::NSPLIT) {
-        const int g0 = gseg[k], g1 = gseg[k + 1];
+        const int g0 = gseg[k] - gbase, g1 = gseg[k + 1] - gbase;
         const int nch = (g1 - g0 + CG - 1) / CG;
         // tiles: s_/c_ (Kahan pairs); right-hand side: ys/yc (diagonal tiles
         // or spare threads)

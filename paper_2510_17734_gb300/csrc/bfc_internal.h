@@ -27,6 +27,14 @@ struct ProfPending {
 struct Ctx;
 bfc_status fail(Ctx* ctx, bfc_status st, const std::string& msg);
 
+// Slices k0 .. k1 - 1 and groups g0 .. g1 - 1 of a grouped level whose records
+// are formed and summed together; max_block: most entries of a k_group_sums
+// block (128 / r consecutive groups).
+struct GroupBatch {
+    int32_t k0 = 0, k1 = 0;
+    int64_t g0 = 0, g1 = 0, max_block = 0;
+};
+
 // The entries of one middle level, inside every slice, in groups that share
 // one environment: one row (by_col = 0, they share h_m) or one column
 // (by_col = 1, they share w_m).  gstart[g] .. gstart[g+1] are the positions
@@ -36,7 +44,7 @@ struct GroupLevel {
     int64_t ngroups = 0;
     int32_t* gstart = nullptr;
     int32_t* gseg = nullptr;
-    int64_t max_block = 0;   // most entries of a k_group_sums block (128 / r consecutive groups)
+    std::vector<GroupBatch> batches;   // the level's slices in the pieces that the record buffer takes
 };
 
 // Device buffers of one completion problem.  Level l = 0 is the S^1 (row)
@@ -68,7 +76,8 @@ struct Ctx {
     int32_t* jL = nullptr;       // column index of the entries in order L
     std::vector<int32_t*> perm;  // L+2: entry index at each position of order l
     std::vector<GroupLevel> grp; // L+2: row / column groups of the middle levels (empty otherwise)
-    void* grec = nullptr;        // group records [s | M | v] of the level being solved (grouped Gram)
+    void* grec = nullptr;        // group records [s | M | v] of the batch being summed (grouped Gram)
+    bool no_groups = false;      // no grouped levels: their buffers did not fit
 
     // environments (compute type): W[l] (l = 0..L) in order l, two H buffers
     void* W = nullptr;

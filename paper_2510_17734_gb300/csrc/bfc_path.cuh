@@ -161,25 +161,28 @@ template <typename T, int R> struct Path {
                         constexpr int RG = GRP ? R : 2;
                         typedef GsumCfg<T, RG> GS;
                         static_assert(GS::NTH == 128, "host block partition of the group sums");
-                        if (c->N >= (int64_t)GROUP_WARP * gl.ngroups) {
-                            k_group_sums_warp<T, RG><<<nblocks(gl.ngroups, 4), 128, 0, c->stream>>>(
-                                hin, W + (size_t)m * NR, (const V*)c->tval[m], gl.gstart, (int)gl.ngroups, gl.by_col,
-                                (V*)c->grec);
-                        } else {
-                            // shared memory for the level's largest block (at most CAP entries)
-                            const int cap = (int)std::min<int64_t>(gl.max_block, GS::CAP);
-                            k_group_sums<T, RG><<<nblocks(gl.ngroups, GS::GB), GS::NTH,
-                                                  (size_t)cap * (RG + 1) * GS::VS, c->stream>>>(
-                                hin, W + (size_t)m * NR, (const V*)c->tval[m], gl.gstart, (int)gl.ngroups, gl.by_col,
-                                (V*)c->grec, cap);
+                        // a level whose records outgrow their buffer in batches of slices
+                        for (const GroupBatch& gb : gl.batches) {
+                            const int32_t* gstart = gl.gstart + gb.g0;
+                            const int G = (int)(gb.g1 - gb.g0);
+                            const unsigned grid = (unsigned)(gb.k1 - gb.k0) * GrpCfg<T, RG>::NSPLIT;
+                            T* rec = (T*)c->rec + (size_t)gb.k0 * Rec<T, R>::SIZE;
+                            if (G > 0 && c->N >= (int64_t)GROUP_WARP * gl.ngroups) {
+                                k_group_sums_warp<T, RG><<<nblocks(G, 4), 128, 0, c->stream>>>(
+                                    hin, W + (size_t)m * NR, (const V*)c->tval[m], gstart, G, gl.by_col, (V*)c->grec);
+                            } else if (G > 0) {
+                                // shared memory for the batch's largest block (at most CAP entries)
+                                const int cap = (int)std::min<int64_t>(gb.max_block, GS::CAP);
+                                k_group_sums<T, RG><<<nblocks(G, GS::GB), GS::NTH,
+                                                      (size_t)cap * (RG + 1) * GS::VS, c->stream>>>(
+                                    hin, W + (size_t)m * NR, (const V*)c->tval[m], gstart, G, gl.by_col, (V*)c->grec,
+                                    cap);
+                            }
+                            const auto gram = gl.by_col ? k_mid_gram_grp<T, RG, 1> : k_mid_gram_grp<T, RG, 0>;
+                            gram<<<grid, GrpCfg<T, RG>::NTH, GrpCfg<T, RG>::SMEM, c->stream>>>(
+                                (const V*)c->grec, gl.gseg + gb.k0, (int)gb.g0, rec, gb.k1 - gb.k0);
                         }
-                        if (gl.by_col)
-                            k_mid_gram_grp<T, RG, 1><<<(unsigned)S * GrpCfg<T, RG>::NSPLIT, GrpCfg<T, RG>::NTH, GrpCfg<T, RG>::SMEM,
-                                                       c->stream>>>((const V*)c->grec, gl.gseg, (T*)c->rec, (int)S);
-                        else
-                            k_mid_gram_grp<T, RG, 0><<<(unsigned)S * GrpCfg<T, RG>::NSPLIT, GrpCfg<T, RG>::NTH, GrpCfg<T, RG>::SMEM,
-                                                       c->stream>>>((const V*)c->grec, gl.gseg, (T*)c->rec, (int)S);
-                        ps.add_kernels(1);
+                        ps.add_kernels(2 * (int)gl.batches.size() - 1);
                         done = true;
                     }
                 }
