@@ -267,7 +267,7 @@ k_group_sums_warp(const typename cvec<T>::type* __restrict__ H, const typename c
     V* o = out + (size_t)g * RL::RS;
     if (lane < R) o[lane] = Sv[(size_t)e0 * R + lane];
     if (RL::RP > R) grp_zero_padding<V, R>(o, lane, 32);
-    warp_sums<T, R>(Uv, tv, e0, gstart[g + 1], a_s[wib], t_s[wib], lane, [&](int, int p, int q, V s, V c) {
+    warp_sums<T, R, sizeof(T) == 4>(Uv, tv, e0, gstart[g + 1], a_s[wib], t_s[wib], lane, [&](int, int p, int q, V s, V c) {
         if constexpr (sizeof(T) == 4) {
             s.x = __fsub_rn(s.x, c.x);
             s.y = __fsub_rn(s.y, c.y);

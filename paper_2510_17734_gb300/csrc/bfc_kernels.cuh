@@ -502,23 +502,23 @@ __device__ __forceinline__ void warp_sums_tiles(const float2* __restrict__ A, co
 // Chunks of 32 rows pass through the warp's own shared memory (a_s: 32 R + 2
 // values, t_s: 32).  emit(item, p, q, sum, comp) hands out every item once, in
 // the order K packed, y (q = -2), its value being sum - comp.
-// FP64: lanes own the R(R+1)/2 + R items (the FP64 pipe counts instructions of
-// a warp).  Complex64: lanes own 2 x 2 tiles of the lower triangle and 2 x 1
-// tiles of y, EG rows at a time side by side; per-chunk partials are folded into
-// Kahan-compensated sums, the EG shares added by error-free sums.  (With an item
-// per lane the two 8-byte reads for each product made the shared-memory return
-// path, 128 bytes a cycle, the bound: n = 4096, r = 12, 3.4 M entries 0.189 ->
-// 0.147 ms; n = 65536, r = 8, 57 entries a row, 0.141 -> 0.151.)
-template <typename T, int R, typename F>
+// Items (FP64 always: the FP64 pipe counts instructions of a warp): lanes own
+// the R(R+1)/2 + R items.  TILES (complex64): lanes own 2 x 2 tiles of the lower
+// triangle and 2 x 1 tiles of y, EG rows at a time side by side; the EG shares
+// are added by error-free sums.  In complex64 per-chunk partials are folded into
+// Kahan-compensated sums.
+template <typename T, int R, bool TILES, typename F>
 __device__ __forceinline__ void warp_sums(const typename cvec<T>::type* __restrict__ A,
                                           const typename cvec<T>::type* __restrict__ tv, int s0, int s1,
                                           typename cvec<T>::type* a_s, typename cvec<T>::type* t_s, int lane, F emit)
 {
     typedef typename cvec<T>::type V;
-    if constexpr (sizeof(T) == 4) {
+    if constexpr (TILES) {
+        static_assert(sizeof(T) == 4, "tiles are a complex64 form");
         warp_sums_tiles<R>(A, tv, s0, s1, a_s, t_s, lane, emit);
         return;
     }
+    constexpr bool COMP = sizeof(T) == 4;
     constexpr int NP = R * (R + 1) / 2;
     constexpr int NI = NP + R;
     constexpr int IPL = (NI + 31) / 32;
@@ -539,9 +539,9 @@ __device__ __forceinline__ void warp_sums(const typename cvec<T>::type* __restri
             iq[u] = -2;  // right-hand side item
         }
     }
-    V acc[IPL];
+    V acc[IPL], sum[IPL], cmp[IPL];
 #pragma unroll
-    for (int u = 0; u < IPL; ++u) acc[u] = czero<V>();
+    for (int u = 0; u < IPL; ++u) acc[u] = sum[u] = cmp[u] = czero<V>();
 
     for (int base = s0; base < s1; base += 32) {
         const int cnt = min(32, s1 - base);
@@ -549,7 +549,12 @@ __device__ __forceinline__ void warp_sums(const typename cvec<T>::type* __restri
         // the chunk's rows are contiguous: copy them as one coalesced block
         {
             const V* src = A + (size_t)base * R;
-            for (int x = lane; x < cnt * R; x += 32) a_s[x] = src[x];
+            if constexpr (sizeof(V) == 8 && R % 2 == 0) {
+                for (int x = lane; x < cnt * R / 2; x += 32)
+                    reinterpret_cast<float4*>(a_s)[x] = reinterpret_cast<const float4*>(src)[x];
+            } else {
+                for (int x = lane; x < cnt * R; x += 32) a_s[x] = src[x];
+            }
             if (lane < cnt) t_s[lane] = tv[base + lane];
         }
         __syncwarp();
@@ -563,19 +568,39 @@ __device__ __forceinline__ void warp_sums(const typename cvec<T>::type* __restri
                 }
             }
         }
+        if constexpr (COMP) {
+#pragma unroll
+            for (int u = 0; u < IPL; ++u) {
+                kahan(sum[u].x, cmp[u].x, acc[u].x);
+                kahan(sum[u].y, cmp[u].y, acc[u].y);
+                acc[u] = czero<V>();
+            }
+        }
     }
 #pragma unroll
     for (int u = 0; u < IPL; ++u) {
         const int it = lane + 32 * u;
-        if (it < NI) emit(it, ip[u], iq[u], acc[u], czero<V>());
+        if (it < NI) emit(it, ip[u], iq[u], COMP ? sum[u] : acc[u], cmp[u]);
     }
 }
+
+// Average rows per fiber from which k_outer_gram takes tiles in complex64.  An
+// item per lane reads two 8-byte values for each product (the shared-memory
+// return path, 128 bytes a cycle, is its bound); tiles read less, but spend up
+// to 2 us per thousand fibers on adding their shares.  us per launch, items /
+// tiles: r = 1, n = 32768, 20 rows 19 / 62, n = 4096, 300 rows 24 / 23; r = 4, n =
+// 4096, 90 rows 17 / 21, 150 rows 24 / 25, 300 rows 39 / 31; r = 8, n = 32768, 60
+// rows 82 / 85, 90 rows 112 / 103; r = 10, 40 rows 75 / 74; r = 12, n = 4096, 40
+// rows 18.5 / 19.8, 800 rows 184 / 143.
+template <int R> struct OuterTiles {
+    static constexpr int ROWS = R == 1 ? 300 : R <= 7 ? 160 : R == 8 ? 90 : R <= 10 ? 70 : 40;
+};
 
 // Outer fibers, stage 1: one warp per fiber accumulates K and y (r x r) over
 // the fiber's entries (warp_sums).  A: design vectors in the level order (w_0
 // for the S^1 rows, h_{L+1} for the S^{L+2} columns).
 // Output record per fiber: [K packed (R(R+1)/2) | y (R)] in FP64.
-template <typename T, int R>
+template <typename T, int R, bool TILES>
 __global__ void __launch_bounds__(128)
 k_outer_gram(const typename cvec<T>::type* __restrict__ A, const typename cvec<T>::type* __restrict__ tv,
              const int32_t* __restrict__ seg, int nfib, double2* __restrict__ rec)
@@ -588,7 +613,7 @@ k_outer_gram(const typename cvec<T>::type* __restrict__ A, const typename cvec<T
     const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
     const int f = blockIdx.x * WPB + wib;
     if (f >= nfib) return;  // whole warp leaves; only warp-level barriers below
-    warp_sums<T, R>(A, tv, seg[f], seg[f + 1], a_s[wib], t_s[wib], lane, [&](int it, int, int, V s, V c) {
+    warp_sums<T, R, TILES>(A, tv, seg[f], seg[f + 1], a_s[wib], t_s[wib], lane, [&](int it, int, int, V s, V c) {
         rec[(size_t)f * NI + it] = make_double2((double)s.x - (double)c.x, (double)s.y - (double)c.y);
     });
 }

@@ -97,8 +97,10 @@ template <typename T, int R> struct Path {
         double2* rec = (double2*)c->rec;
         {
             ProfScope ps(c, COLS ? "outer_cols_gram" : "outer_rows_gram");
-            k_outer_gram<T, R><<<nblocks(n, 4), 128, 0, c->stream>>>(A, (const V*)c->tval[level], c->seg[level],
-                                                                      (int)n, rec);
+            auto gram = k_outer_gram<T, R, false>;
+            if constexpr (sizeof(T) == 4)
+                if (c->N >= OuterTiles<R>::ROWS * n) gram = k_outer_gram<T, R, true>;
+            gram<<<nblocks(n, 4), 128, 0, c->stream>>>(A, (const V*)c->tval[level], c->seg[level], (int)n, rec);
         }
         {
             ProfScope ps(c, COLS ? "outer_cols_solve" : "outer_rows_solve");

@@ -1,0 +1,42 @@
+"""Both sides of lines of the sweep's dispatch, against the oracle: rows per
+fiber from which k_outer_gram takes tiles (complex64).  Tolerances as in test_gpu_group_ranks.py: FP64 1e-10 relative on
+entry values and the objective; complex64 max(1e-4, kappa_max 2^-24)."""
+import numpy as np
+import pytest
+
+import oracle
+import paper_2510_17734_gb300 as bfc
+import synth
+from helpers import block_conditions, rel_dev
+
+pytestmark = pytest.mark.gpu
+
+RIDGE = {bfc.PREC_FP64: 0.0, bfc.PREC_C64: 2.0 ** -20}
+
+
+def check(n, L, b, r, count, prec, lam=1e-1, **kw):
+    i, j = synth.draw_pairs(n, count, 30 + r)
+    X = synth.random_factors(n, L, r, 900 + r)
+    t = oracle.eval_entries(n, L, b, r, X, i, j)
+    X0 = synth.random_factors(n, L, r, 300 + r)
+    Xo, st_o = oracle.als_sweep(n, L, b, r, lam, X0, i, j, t, ridge_rel=RIDGE[prec])
+    with bfc.Completion(n, L, b, r, lam, i, j, t, prec=prec, **kw) as c:
+        groups = [c.level_groups(m) for m in range(1, L + 1)]
+        c.set_factors(X0)
+        st = c.sweep()
+        Xg = c.get_factors()
+    tol = 1e-10
+    if prec == bfc.PREC_C64:
+        kappa = max(float(v.max()) for v in block_conditions(X0, Xo, i, j, t, n, L, b, r, lam, 2.0 ** -20) if v.size)
+        tol = max(1e-4, kappa * 2.0 ** -24)
+    assert abs(st["objective"] - st_o["objective"]) <= tol * abs(st_o["objective"])
+    assert rel_dev(oracle.eval_entries(n, L, b, r, Xg, i, j), oracle.eval_entries(n, L, b, r, Xo, i, j)) <= tol
+    return groups
+
+
+@pytest.mark.parametrize("side", [-1, 0])
+@pytest.mark.parametrize("r", range(1, 13))
+def test_outer_gram_forms(r, side):
+    rows = 300 if r == 1 else 160 if r <= 7 else 90 if r == 8 else 70 if r <= 10 else 40
+    n = 2 * rows
+    check(n, 0, n, r, rows * n + side, bfc.PREC_C64, lam=1e-6)
