@@ -61,7 +61,7 @@ template <typename T, int R> struct Path {
         cudaError_t e = cudaFuncSetAttribute(k_mid_gram<T, R>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                              (int)GramCfg<T, R>::SMEM);
         if (e == cudaSuccess)
-            e = cudaFuncSetAttribute(k_mid_solve<T, R>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+            e = cudaFuncSetAttribute(k_mid_solve<T, R, SolveCfg<T, R>::NW>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                      (int)SolveCfg<T, R>::SMEM);
         if (e == cudaSuccess)
             e = cudaFuncSetAttribute(k_mid_fallback<T, R>, cudaFuncAttributeMaxDynamicSharedMemorySize,
@@ -204,7 +204,14 @@ template <typename T, int R> struct Path {
             {
                 ProfScope ps(c, "mid_solve");
                 if (SC::MIXED) cudaMemsetAsync(c->d_count + 3, 0, sizeof(unsigned long long), c->stream);
-                k_mid_solve<T, R><<<(unsigned)S, SC::NTH, SC::SMEM, c->stream>>>(
+                auto solve = k_mid_solve<T, R, SC::NW>;
+                unsigned nth = SC::NTH;
+                if constexpr (SC::ONE_WARP)
+                    if (S > (int64_t)SC::ONE_WARP_FROM * c->num_sms) {
+                        solve = k_mid_solve<T, R, 1>;
+                        nth = 32;
+                    }
+                solve<<<(unsigned)S, nth, SC::SMEM, c->stream>>>(
                     (const T*)c->rec, hin, c->seg[m], c->nxt[m], hout, c->Zd + (size_t)(m - 1) * S * R * R,
                     (V*)c->Zt + (size_t)(m - 1) * S * R * R, c->P.lambda, c->ridge, c->d_count,
                     c->d_count + 3, c->d_count + 2, c->fblist, c->d_count + 5, c->inject == 1 ? 1 : 0);

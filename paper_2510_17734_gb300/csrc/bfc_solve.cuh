@@ -124,9 +124,16 @@ template <typename T, int R> struct SolveCfg {
     // warps leave its loads exposed and 8 lose the CTAs per SM that overlap
     // (S = 512: 208 / 209 / 281 us per launch with 2 / 4 / 8, S = 128: 316 / 204
     // / 199 us; 256 and 360 us with 2 warps and 4 x 4 tiles)
-    static constexpr int NW = R <= 8 ? (MIXED ? 2 : 4) : R <= 10 ? 4 : 8;
+    static constexpr int NW = R <= 8 ? (MIXED || R <= 2 ? 2 : 4) : R <= 10 ? 4 : 8;
+    // Small ranks also in a form of one warp, for levels with more slices than
+    // CTAs of two warps are resident (8 per SM): the second warp finds little to
+    // do between the barriers.  us per launch, two warps / one: r = 3, S = 4096, 20
+    // entries per row 49 / 32, S = 512, 300 entries per row 32 / 40; r = 5, S =
+    // 16384 358 / 196, S = 512, 300 entries 53 / 60; FP64, r = 1, S = 4096 (four
+    // warps / one) 31 / 20
+    static constexpr bool ONE_WARP = R <= (MIXED ? 5 : 2);
+    static constexpr int ONE_WARP_FROM = 8;   // slices per SM
     static constexpr int NTH = 32 * NW;
-    static constexpr int MINB = MIXED ? 512 / NTH : 1;   // 128 registers in the precision form
     static constexpr int FBT = 128;      // threads of a k_mid_fallback CTA
     // record (+ slack: short blocks and tiles read, but do not write, rows past its
     // end), solution (double-float or FP64), residual / new slice, exchange
@@ -790,8 +797,8 @@ __device__ __forceinline__ void slice_h_update(const typename cvec<T>::type* __r
 // directly.  The slice is written row-major in FP64 and the compute type; then
 // h_{m+1}(e) = h_m(e)^T Z^{m+1}(k) for the slice's entries is scattered into
 // order m+1.  A singular system keeps its old slice.
-template <typename T, int R>
-__global__ void __launch_bounds__(SolveCfg<T, R>::NTH, SolveCfg<T, R>::MINB)
+template <typename T, int R, int NW>
+__global__ void __launch_bounds__(32 * NW, sizeof(T) == 4 ? 16 / NW : 1)   // 128 registers in the precision form
 k_mid_solve(const T* __restrict__ rec, const typename cvec<T>::type* __restrict__ H,
             const int32_t* __restrict__ seg, const int32_t* __restrict__ nxt,
             typename cvec<T>::type* __restrict__ Hn, double2* __restrict__ Zd,
@@ -809,7 +816,7 @@ k_mid_solve(const T* __restrict__ rec, const typename cvec<T>::type* __restrict_
     typedef Rec<T, R> RC;
     constexpr int D = C::D, NS = C::NS;
     extern __shared__ __align__(16) unsigned char smem[];
-    constexpr int nthr = C::NTH;
+    constexpr int nthr = 32 * NW;
     const int tid = threadIdx.x, lane = tid & 31, k = blockIdx.x;
     T* Lm = (T*)smem;
     float4* s_df = (float4*)(smem + C::LBYTES);      // double-float solution

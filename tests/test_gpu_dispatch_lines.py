@@ -1,5 +1,6 @@
 """Both sides of lines of the sweep's dispatch, against the oracle: rows per
-fiber from which k_outer_gram takes tiles (complex64).  Tolerances as in test_gpu_group_ranks.py: FP64 1e-10 relative on
+fiber from which k_outer_gram takes tiles (complex64), slices per level from
+which k_mid_solve takes one warp.  Tolerances as in test_gpu_group_ranks.py: FP64 1e-10 relative on
 entry values and the objective; complex64 max(1e-4, kappa_max 2^-24)."""
 import numpy as np
 import pytest
@@ -40,3 +41,11 @@ def test_outer_gram_forms(r, side):
     rows = 300 if r == 1 else 160 if r <= 7 else 90 if r == 8 else 70 if r <= 10 else 40
     n = 2 * rows
     check(n, 0, n, r, rows * n + side, bfc.PREC_C64, lam=1e-6)
+
+
+@pytest.mark.parametrize("L", [9, 10])      # 1024 and 2048 slices; 8 per SM lie between
+@pytest.mark.parametrize("r,prec", [(1, bfc.PREC_C64), (2, bfc.PREC_C64), (3, bfc.PREC_C64), (4, bfc.PREC_C64),
+                                    (5, bfc.PREC_C64), (1, bfc.PREC_FP64), (2, bfc.PREC_FP64)])
+def test_solve_warps(r, prec, L):
+    b = max(2, r)
+    check(b << L, L, b, r, 30 * (2 << L), prec)
