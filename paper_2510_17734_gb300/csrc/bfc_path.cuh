@@ -19,13 +19,21 @@ template <typename T, int R> struct Path {
     static constexpr bool TC = sizeof(T) == 4 && R <= 8;
     // the grouped Gram (rank 1 has nothing to gain: K is one number)
     static constexpr bool GRP = R >= 2;
-    // entries per group from which a warp takes one group (k_group_sums_warp)
-    // instead of r threads (k_group_sums).  Complex64: at rank 8 and 29 entries
-    // per group the threads are faster (0.140 against 0.154 ms at n = 65536), at
+    // Whether a warp takes one group of the level (k_group_sums_warp) instead of
+    // r threads (k_group_sums).  Complex64: from 32 entries per group: at rank 8
+    // and 29 the threads are faster (0.140 against 0.154 ms at n = 65536), at
     // rank 12 and 52 to 420 a block's entries outgrow its staging and the warps
-    // are.  FP64: the warps form only the lower triangle, which the FP64 pipe
-    // shows at every size (n = 4096, r = 6: 71 against 145 to 170 us a level)
-    static constexpr int GROUP_WARP = sizeof(T) == 8 ? 2 : 32;
+    // are.  FP64: from 2, the warps form only the lower triangle, which the FP64
+    // pipe shows (n = 4096, r = 6: 71 against 145 to 170 us a level); but at rank
+    // 2 only 5 of 32 lanes have an item, which costs more than that once the
+    // groups outnumber the warps that are resident (64 per SM; all levels, warps
+    // / threads: n = 1024, 184 k entries 0.39 / 0.45 ms, n = 8192, 3.3 M 6.54 / 2.28)
+    static bool group_warp(const Ctx* c, const GroupLevel& gl)
+    {
+        if (sizeof(T) == 4) return c->N >= 32 * gl.ngroups;
+        if (R == 2 && gl.ngroups > (int64_t)64 * c->num_sms) return false;
+        return c->N >= 2 * gl.ngroups;
+    }
 
     static cudaError_t set_grp_attr()
     {
@@ -169,7 +177,7 @@ template <typename T, int R> struct Path {
                             const int G = (int)(gb.g1 - gb.g0);
                             const unsigned grid = (unsigned)(gb.k1 - gb.k0) * GrpCfg<T, RG>::NSPLIT;
                             T* rec = (T*)c->rec + (size_t)gb.k0 * Rec<T, R>::SIZE;
-                            if (G > 0 && c->N >= (int64_t)GROUP_WARP * gl.ngroups) {
+                            if (G > 0 && group_warp(c, gl)) {
                                 k_group_sums_warp<T, RG><<<nblocks(G, 4), 128, 0, c->stream>>>(
                                     hin, W + (size_t)m * NR, (const V*)c->tval[m], gstart, G, gl.by_col, (V*)c->grec);
                             } else if (G > 0) {

@@ -1,6 +1,7 @@
-"""Both sides of lines of the sweep's dispatch, against the oracle: rows per
-fiber from which k_outer_gram takes tiles (complex64), slices per level from
-which k_mid_solve takes one warp.  Tolerances as in test_gpu_group_ranks.py: FP64 1e-10 relative on
+"""Both sides of three lines of the sweep's dispatch, against the oracle: rows
+per fiber from which k_outer_gram takes tiles (complex64), slices per level from
+which k_mid_solve takes one warp, groups per level from which FP64 rank 2 sums
+by threads.  Tolerances as in test_gpu_group_ranks.py: FP64 1e-10 relative on
 entry values and the objective; complex64 max(1e-4, kappa_max 2^-24)."""
 import numpy as np
 import pytest
@@ -49,3 +50,9 @@ def test_outer_gram_forms(r, side):
 def test_solve_warps(r, prec, L):
     b = max(2, r)
     check(b << L, L, b, r, 30 * (2 << L), prec)
+
+
+def test_group_sums_fp64_rank2():
+    groups = check(4096, 10, 4, 2, 45_000, bfc.PREC_FP64, group_ratio=2.0)
+    few, many = [g for g, _ in groups if g <= 64 * 148], [g for g, _ in groups if g > 64 * 160]
+    assert all(on for _, on in groups) and few and many     # warps and threads
