@@ -1024,13 +1024,17 @@ k_eval(const int32_t* __restrict__ ii, const int32_t* __restrict__ jj, int64_t M
     const bool col = c < R;
     const int64_t warp0 = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
     const int64_t nwarps = ((int64_t)gridDim.x * blockDim.x) >> 5;
+    const unsigned top = ((unsigned)b << L) - 1u;   // n - 1
     // a group leader sums about a dozen entries in the compute type; the
     // reductions across lanes and warps run in FP64
     T numl = T(0), denl = T(0);
     for (int64_t base = warp0 * GPW; base < M; base += nwarps * GPW) {   // warp-uniform
         const int64_t e = base + g;
         const bool valid = e < M;
-        const int i = valid ? ii[e] : 0, j = valid ? jj[e] : 0;   // entry 0's indices stand in for the tail
+        // (0 stands in for the tail).  The caller's own arrays are read here again
+        // after their check: an index that another stream changes meanwhile must
+        // not lead outside the factors
+        const int i = valid ? (int)min((unsigned)ii[e], top) : 0, j = valid ? (int)min((unsigned)jj[e], top) : 0;
         V h = col ? z1[(size_t)i * R + c] : czero<V>();
         const int pi = i / b, pj = j / b;
         // the slice of every level depends only on (i, j): level m + 1's
