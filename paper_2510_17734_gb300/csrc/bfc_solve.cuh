@@ -920,7 +920,8 @@ k_mid_solve(const T* __restrict__ rec, const typename cvec<T>::type* __restrict_
                     }
 #pragma unroll
                     for (int o = 16; o > 0; o >>= 1) rmax = fmaxf(rmax, __shfl_xor_sync(0xffffffffu, rmax, o));
-                    const float sc = rmax > 0.f ? rmax : 1.f;
+                    // (a residual below the normal range: its reciprocal would be infinite)
+                    const float sc = fmaxf(rmax, 1.17549435e-38f);
                     const float isc = 1.f / sc;
 #pragma unroll
                     for (int s = 0; s < NS; ++s) { bv[s].x *= isc; bv[s].y *= isc; }
