@@ -218,14 +218,19 @@ struct Inputs {
 //    r = 5 0.85 / 0.58 / 0.58; n = 65536, b = 16, r = 8: four levels.  Its two
 //    kernels cost 5 us more than one.  At ranks 4 and 8 also below 0.1 groups
 //    per entry, for the compensated sums: n = 32768, r = 4, Radon data, error of
-//    the factors after a sweep 7.2e-7, and 8.5e-7 without those levels;
+//    the factors after a sweep 7.2e-7, and 8.5e-7 without those levels.  Slices of
+//    fewer than r rows (columns) group as well: with b = 1 .. 4 < r, four sweeps
+//    of ten problems each, all levels on the tensor cores / grouped leave 165 / 0
+//    (r = 5), 1591 / 6 (r = 6), 7821 / 27 (r = 7) and 21027 / 335 (r = 8) singular
+//    systems;
 //  * next to the per-entry CUDA-core kernel, whose work per entry is that of a
 //    group, below 0.9 groups per entry.  In the precision form (r > 8) not
 //    where slices have fewer than r rows (columns): they are rank deficient and
 //    solved at the ridge floor, and the coherent rounding of a few large group
-//    terms (2-norm error of K 1.8 times that of k_mid_gram) makes more of them
-//    indefinite (n = 4096, b = 4, r = 12: 24 of 20,480 systems of a sweep kept
-//    their old slice, with k_mid_gram 2).
+//    terms (2-norm error of K 1.8 times that of k_mid_gram) can make more of them
+//    indefinite (Radon data, n = 4096, b = 4, r = 12: 24 of 20,480 systems of a
+//    sweep kept their old slice, with k_mid_gram 2; on the line kernel's data it
+//    is the other way round, b = 4, r = 12, eight sweeps 10,235 with this rule and 5,160 without).
 static bool group_level(const Ctx* c, int64_t G, int64_t loc)
 {
     if (c->r < 2 || c->P.gram_impl != 0 || c->no_groups) return false;
@@ -236,7 +241,7 @@ static bool group_level(const Ctx* c, int64_t G, int64_t loc)
         static const double group[7] = {0.025, 0.1, 0.1, 0.375, 0.4, 1.0, 1.25};
         const double gain = base[c->r - 2] * S + 0.105 * N - group[c->r - 2] * g;
         // with fewer slices than SMs both leave the rest idle
-        return gain * std::max(1.0, 152.0 / S) > 5000.0 || ((c->r == 4 || c->r == 8) && g < 0.1 * N);
+        return gain * std::max(1.0, (double)c->num_sms / S) > 5000.0 || ((c->r == 4 || c->r == 8) && g < 0.1 * N);
     }
     if (c->fp32 && loc < c->r) return false;
     return g < 0.9 * N;

@@ -298,39 +298,6 @@ __device__ __forceinline__ void grp_acc(float2& s, float2& c, float2 x, float2 y
 }
 __device__ __forceinline__ void grp_acc(double2& s, double2&, double2 x, double2 y) { cmac(s, x, y); }
 
-// Packed (re, im) pairs of FP32 values and the f32x2 arithmetic of sm_100
-// and later: one instruction acts on both components.
-__device__ __forceinline__ uint64_t g2pack(float a, float b)
-{
-    uint64_t r;
-    asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(a), "f"(b));
-    return r;
-}
-__device__ __forceinline__ float2 g2unpack(uint64_t r)
-{
-    float2 v;
-    asm("mov.b64 {%0, %1}, %2;" : "=f"(v.x), "=f"(v.y) : "l"(r));
-    return v;
-}
-__device__ __forceinline__ uint64_t g2fma(uint64_t a, uint64_t b, uint64_t c)
-{
-    uint64_t d;
-    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(d) : "l"(a), "l"(b), "l"(c));
-    return d;
-}
-__device__ __forceinline__ uint64_t g2add(uint64_t a, uint64_t b)
-{
-    uint64_t d;
-    asm("add.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
-    return d;
-}
-__device__ __forceinline__ uint64_t g2sub(uint64_t a, uint64_t b)
-{
-    uint64_t d;
-    asm("sub.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
-    return d;
-}
-
 // (s, nc) += x y + x' y' with packed operands: X1 = (x.re, x.re), X2 = (x.im,
 // x.im), Y = (y.re, y.im), Yr = i y = (-y.im, y.re), so x y = X1 Y + X2 Yr.  s
 // is the Kahan sum and nc its negated compensation (the value is s + nc); the
@@ -340,9 +307,9 @@ __device__ __forceinline__ uint64_t g2sub(uint64_t a, uint64_t b)
 __device__ __forceinline__ void grp_acc2(uint64_t& s, uint64_t& nc, uint64_t X1, uint64_t X2, uint64_t Y, uint64_t Yr,
                                          uint64_t W1, uint64_t W2, uint64_t Z, uint64_t Zr)
 {
-    const uint64_t q = g2fma(X1, Y, g2fma(X2, Yr, g2fma(W1, Z, g2fma(W2, Zr, nc))));   // x y + x' y' - c
-    const uint64_t t = g2add(s, q);
-    nc = g2sub(q, g2sub(t, s));
+    const uint64_t q = c2fma(X1, Y, c2fma(X2, Yr, c2fma(W1, Z, c2fma(W2, Zr, nc))));   // x y + x' y' - c
+    const uint64_t t = c2add(s, q);
+    nc = c2sub(q, c2sub(t, s));
     s = t;
 }
 
@@ -493,8 +460,8 @@ k_mid_gram_grp(const typename cvec<T>::type* __restrict__ grec, const int32_t* _
                         const V x = cmul(make_conj(gr[aI]), gr[aJ]);
                         V w = cmul(make_conj(gs[aI]), gs[aJ]);
                         if (!two) w = czero<V>();
-                        const uint64_t X1 = g2pack(x.x, x.x), X2 = g2pack(x.y, x.y);
-                        const uint64_t W1 = g2pack(w.x, w.x), W2 = g2pack(w.y, w.y);
+                        const uint64_t X1 = c2pack(x.x, x.x), X2 = c2pack(x.y, x.y);
+                        const uint64_t W1 = c2pack(w.x, w.x), W2 = c2pack(w.y, w.y);
 #pragma unroll
                         for (int u = 0; u < TT; ++u) {
                             V yr[TT], zr[TT];
@@ -502,9 +469,9 @@ k_mid_gram_grp(const typename cvec<T>::type* __restrict__ grec, const int32_t* _
                             load_t<V, TT>(zr, gs + RL::m(cI + u, cJ));
 #pragma unroll
                             for (int v = 0; v < TT; ++v)
-                                grp_acc2(s2[u][v], n2[u][v], X1, X2, g2pack(yr[v].x, yr[v].y),
-                                         g2pack(-yr[v].y, yr[v].x), W1, W2, g2pack(zr[v].x, zr[v].y),
-                                         g2pack(-zr[v].y, zr[v].x));
+                                grp_acc2(s2[u][v], n2[u][v], X1, X2, c2pack(yr[v].x, yr[v].y),
+                                         c2pack(-yr[v].y, yr[v].x), W1, W2, c2pack(zr[v].x, zr[v].y),
+                                         c2pack(-zr[v].y, zr[v].x));
                         }
                         if (diag) {
 #pragma unroll
@@ -526,13 +493,13 @@ k_mid_gram_grp(const typename cvec<T>::type* __restrict__ grec, const int32_t* _
                         for (int u = 0; u < TT; ++u) {
                             const V si = gr[cI + u], ti = gs[cI + u];
                             const V xa = cmul(make_conj(si), x), wa = cmul(make_conj(ti), w);
-                            const uint64_t X1 = g2pack(xa.x, xa.x), X2 = g2pack(xa.y, xa.y);
-                            const uint64_t W1 = g2pack(wa.x, wa.x), W2 = g2pack(wa.y, wa.y);
+                            const uint64_t X1 = c2pack(xa.x, xa.x), X2 = c2pack(xa.y, xa.y);
+                            const uint64_t W1 = c2pack(wa.x, wa.x), W2 = c2pack(wa.y, wa.y);
 #pragma unroll
                             for (int v = 0; v < TT; ++v)
-                                grp_acc2(s2[u][v], n2[u][v], X1, X2, g2pack(sj[v].x, sj[v].y),
-                                         g2pack(-sj[v].y, sj[v].x), W1, W2, g2pack(tj[v].x, tj[v].y),
-                                         g2pack(-tj[v].y, tj[v].x));
+                                grp_acc2(s2[u][v], n2[u][v], X1, X2, c2pack(sj[v].x, sj[v].y),
+                                         c2pack(-sj[v].y, sj[v].x), W1, W2, c2pack(tj[v].x, tj[v].y),
+                                         c2pack(-tj[v].y, tj[v].x));
                             if (diag) {
                                 grp_acc(ys[u], yc[u], gr[RL::VOFF + aI], make_conj(si));
                                 if (two) grp_acc(ys[u], yc[u], gs[RL::VOFF + aI], make_conj(ti));
@@ -604,9 +571,7 @@ k_mid_gram_grp(const typename cvec<T>::type* __restrict__ grec, const int32_t* _
             for (int u = 0; u < TT; ++u) {
 #pragma unroll
                 for (int v = 0; v < TT; ++v) {
-                    const float2 t = g2unpack(g2add(s2[u][v], n2[u][v]));
-                    s_[u][v].x = t.x;
-                    s_[u][v].y = t.y;
+                    c2unpack(c2add(s2[u][v], n2[u][v]), s_[u][v].x, s_[u][v].y);
                 }
                 ys[u].x = __fsub_rn(ys[u].x, yc[u].x);
                 ys[u].y = __fsub_rn(ys[u].y, yc[u].y);

@@ -1304,9 +1304,7 @@ template <typename T, int R, bool PRE> struct SliceSums {
     }
     __device__ __forceinline__ void values(V (&d)[TT], const V* p) const
     {
-        if constexpr (sizeof(V) == 8 && TT == 4 && R % 2 == 0) {
-            load4(d, p);
-        } else if constexpr (sizeof(V) == 8 && TT == 2 && R % 2 == 0) {
+        if constexpr (sizeof(V) == 8 && TT == 2 && R % 2 == 0) {
             const float4 t = *reinterpret_cast<const float4*>(p);
             d[0].x = t.x; d[0].y = t.y;
             d[1].x = t.z; d[1].y = t.w;

@@ -70,17 +70,12 @@ template <> struct KPair<double> {
     static __device__ __forceinline__ P make(double x, double y) { return make_double2(x, y); }
     static __device__ __forceinline__ P neg(P x) { return make_double2(-x.x, -x.y); }
     static __device__ __forceinline__ double sum(A a) { return a; }
-    static __device__ __forceinline__ void load4(const double* p, P (&d)[2])
-    {
-        d[0] = *reinterpret_cast<const double2*>(p);
-        d[1] = *reinterpret_cast<const double2*>(p + 2);
-    }
 };
-template <typename T> __device__ __forceinline__ void load8(const T* p, typename KPair<T>::P (&d)[4])
+__device__ __forceinline__ void load8(const float* p, uint64_t (&d)[4])
 {
-    typename KPair<T>::P a[2], b[2];
-    KPair<T>::load4(p, a);
-    KPair<T>::load4(p + 4, b);
+    uint64_t a[2], b[2];
+    KPair<float>::load4(p, a);
+    KPair<float>::load4(p + 4, b);
     d[0] = a[0]; d[1] = a[1]; d[2] = b[0]; d[3] = b[1];
 }
 // four consecutive values of shared memory
@@ -284,16 +279,16 @@ template <typename T, int R> __device__ __forceinline__ void solve_panel_row(T* 
     }
 }
 
-// (3) Tile (I, Jt) of the trailing matrix of panel J: rows 8J + 8 + 4 I .. + 3,
+// (3) Precision form: tile (I, Jt) of the trailing matrix of panel J: rows 8J + 8 + 4 I .. + 3,
 // columns 8J + 8 + 4 Jt .. + 3, minus the product of the panel's rows.
-template <typename T, int R> __device__ __forceinline__ void solve_tile(T* Lm, int J, int I, int Jt)
+template <int R> __device__ __forceinline__ void solve_tile(float* Lm, int J, int I, int Jt)
 {
-    typedef Rec<T, R> RC;
-    typedef KPair<T> K;
-    typedef typename K::P P;
-    const T* xp = Lm + RC::row(J, 8 + 4 * I);   // four consecutive rows, 16 values apart
-    const T* lp = Lm + RC::row(J, 8 + 4 * Jt);
-    typename K::A sr[4][4], si[4][4];
+    typedef Rec<float, R> RC;
+    typedef KPair<float> K;
+    typedef K::P P;
+    const float* xp = Lm + RC::row(J, 8 + 4 * I);   // four consecutive rows, 16 values apart
+    const float* lp = Lm + RC::row(J, 8 + 4 * Jt);
+    K::A sr[4][4], si[4][4];
 #pragma unroll
     for (int u = 0; u < 4; ++u)
 #pragma unroll
@@ -323,11 +318,11 @@ template <typename T, int R> __device__ __forceinline__ void solve_tile(T* Lm, i
         }
     }
     const int c = 8 * J + 8 + 4 * Jt, Jd = c >> 3, r0 = 8 * J + 8 + 4 * I;
-    T* dp = Lm + RC::row(Jd, r0 - 8 * Jd) + (c & 7);
+    float* dp = Lm + RC::row(Jd, r0 - 8 * Jd) + (c & 7);
 #pragma unroll
     for (int u = 0; u < 4; ++u) {
         if (r0 + u <= RC::D) {
-            T a[4], b[4];
+            float a[4], b[4];
             ld4(dp + 16 * u, a);
             ld4(dp + 16 * u + 8, b);
 #pragma unroll
@@ -343,21 +338,21 @@ template <typename T, int R> __device__ __forceinline__ void solve_tile(T* Lm, i
 
 // The row of conj(y) (row D) of the trailing matrix, columns 8J + 8 + 4 Jt ..
 // + 3, where D is a multiple of 4 (otherwise it lies in the last full tiles).
-template <typename T, int R> __device__ __forceinline__ void solve_y_tile(T* Lm, int J, int Jt)
+template <int R> __device__ __forceinline__ void solve_y_tile(float* Lm, int J, int Jt)
 {
-    typedef Rec<T, R> RC;
-    typedef KPair<T> K;
-    typedef typename K::P P;
-    const T* xp = Lm + RC::row(J, RC::D - 8 * J);
-    const T* lp = Lm + RC::row(J, 8 + 4 * Jt);
+    typedef Rec<float, R> RC;
+    typedef KPair<float> K;
+    typedef K::P P;
+    const float* xp = Lm + RC::row(J, RC::D - 8 * J);
+    const float* lp = Lm + RC::row(J, 8 + 4 * Jt);
     P xr[4], xi[4], nr[4];
     load8(xp, xr);
     load8(xp + 8, xi);
 #pragma unroll
     for (int t = 0; t < 4; ++t) nr[t] = K::neg(xr[t]);
-    T a[4], b[4];
+    float a[4], b[4];
     const int c = 8 * J + 8 + 4 * Jt, Jd = c >> 3;
-    T* dp = Lm + RC::row(Jd, RC::D - 8 * Jd) + (c & 7);
+    float* dp = Lm + RC::row(Jd, RC::D - 8 * Jd) + (c & 7);
     ld4(dp, a);
     ld4(dp + 8, b);
 #pragma unroll
@@ -365,7 +360,7 @@ template <typename T, int R> __device__ __forceinline__ void solve_y_tile(T* Lm,
         P lr[4], li[4];
         load8(lp + 16 * v, lr);
         load8(lp + 16 * v + 8, li);
-        typename K::A sr = K::zero(), si = K::zero();
+        K::A sr = K::zero(), si = K::zero();
 #pragma unroll
         for (int t = 0; t < 4; ++t) {
             sr = K::fma(K::fma(sr, xr[t], lr[t]), xi[t], li[t]);
@@ -474,15 +469,14 @@ __device__ __forceinline__ bool solve_chol(T* Lm, T tol, volatile int* fail, int
                 const int I = tri(x);
                 solve_tile2<R>(Lm, J, I, x - I * (I + 1) / 2);
             }
-            __syncthreads();
-            continue;
-        }
-        const int mc = max(0, (D - 8 * J - 5) / 4), nt = mc * (mc + 1) / 2;
-        if constexpr (D % 4 == 0)
-            for (int x = nthr - 1 - tid; x < mc; x += nthr) solve_y_tile<T, R>(Lm, J, x);
-        for (int x = tid; x < nt; x += nthr) {
-            const int I = tri(x);
-            solve_tile<T, R>(Lm, J, I, x - I * (I + 1) / 2);
+        } else {
+            const int mc = max(0, (D - 8 * J - 5) / 4), nt = mc * (mc + 1) / 2;
+            if constexpr (D % 4 == 0)
+                for (int x = nthr - 1 - tid; x < mc; x += nthr) solve_y_tile<R>(Lm, J, x);
+            for (int x = tid; x < nt; x += nthr) {
+                const int I = tri(x);
+                solve_tile<R>(Lm, J, I, x - I * (I + 1) / 2);
+            }
         }
         __syncthreads();
     }
