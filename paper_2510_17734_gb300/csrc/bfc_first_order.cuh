@@ -64,6 +64,26 @@ __device__ __forceinline__ void stage_rows(const typename cvec<T>::type* __restr
             reinterpret_cast<float4*>(w_s)[x] =
                 make_float4(w.x * r.x + w.y * r.y, w.x * r.y - w.y * r.x, w.z * r.x + w.w * r.y, w.z * r.y - w.w * r.x);
         }
+    } else if constexpr (sizeof(V) == 8) {
+        // all loads of a thread's R values in flight together
+        V h[R], w[R], r[R];
+#pragma unroll
+        for (int u = 0; u < R; ++u) {
+            const int x = min(tid + 128 * u, cnt * R - 1);
+            h[u] = H[(size_t)base * R + x];
+            w[u] = Wm[(size_t)base * R + x];
+            r[u] = Rc[base + x / R];
+        }
+#pragma unroll
+        for (int u = 0; u < R; ++u) {
+            const int x = tid + 128 * u;
+            if (x < cnt * R) {
+                V rw = czero<V>();
+                cmacc(rw, w[u], r[u]);
+                h_s[x] = h[u];
+                w_s[x] = rw;
+            }
+        }
     } else {
         for (int x = tid; x < cnt * R; x += 128) {
             V rw = czero<V>();
