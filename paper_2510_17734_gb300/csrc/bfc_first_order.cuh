@@ -534,8 +534,8 @@ k_h1_rows(const int32_t* __restrict__ seg, int nfib, const typename cvec<T>::typ
 
 // ---------------------------------------------------------------- matvec
 
-// L = 0: Y[p][q] = sum over the leaf of zL(j)^T v_q(j), p = j / b (the
-// contraction of S^{L+2} with the vectors over j_L); one thread per (p, q).
+// Y[p][q] = sum over the leaf of zL(j)^T v_q(j), p = j / b (the contraction of
+// S^{L+2} with the vectors over j_L); one thread per (p, q).
 template <typename T, int R>
 __global__ void k_mv_leaf(const typename cvec<T>::type* __restrict__ zL, const double2* __restrict__ Vin, int b,
                           int nvec, int npre, typename cvec<T>::type* __restrict__ Y)
@@ -757,21 +757,79 @@ k_mv_pass(MvPass ps, const typename cvec<T>::type* __restrict__ Z, const typenam
     }
 }
 
-// u_q(i) = z1(i)^T Y[q], Y the leaf contraction, for L = 0; one thread per (i, q).
+// Level m of the contraction (m = L .. 1) by itself, one thread per (k, q) (the
+// FP64 form for few vectors, see MvRule).  Intermediates are laid out [k][q][c].
+template <typename T, int R>
+__global__ void k_mv_level(const typename cvec<T>::type* __restrict__ Zm, const typename cvec<T>::type* __restrict__ Yin,
+                           typename cvec<T>::type* __restrict__ Yout, int m, int L, int nvec, int S)
+{
+    typedef typename cvec<T>::type V;
+    const int64_t idx = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    if (idx >= (int64_t)S * nvec) return;
+    const int k = (int)(idx / nvec), q = (int)(idx - (int64_t)k * nvec);
+    V tv[R];
+    if (m == L) {
+        const int64_t g = k & ((1 << L) - 1);
+#pragma unroll
+        for (int c = 0; c < R; ++c) tv[c] = Yin[(g * nvec + q) * R + c];
+    } else {
+        const int64_t g = ((int64_t)(k >> (m + 1)) << m) | (k & ((1 << m) - 1));
+#pragma unroll
+        for (int c = 0; c < R; ++c) {
+            const V a = Yin[((2 * g) * nvec + q) * R + c], b = Yin[((2 * g + 1) * nvec + q) * R + c];
+            tv[c].x = a.x + b.x;
+            tv[c].y = a.y + b.y;
+        }
+    }
+    const V* Z = Zm + (size_t)k * R * R;
+#pragma unroll
+    for (int a = 0; a < R; ++a) {
+        V acc = czero<V>();
+#pragma unroll
+        for (int c = 0; c < R; ++c) cmac(acc, Z[a * R + c], tv[c]);
+        Yout[idx * R + a] = acc;
+    }
+}
+
+// u_q(i) = z1(i)^T T_0[p_i], T_0[p] = Y_1[2p] + Y_1[2p + 1] (the sum over j_0)
+// for L >= 1, or the leaf contraction for L = 0; one thread per (i, q).
 template <typename T, int R>
 __global__ void k_mv_root(const typename cvec<T>::type* __restrict__ z1, const typename cvec<T>::type* __restrict__ Y,
-                          int nvec, int64_t n, double2* __restrict__ U)
+                          int b, int L, int nvec, int64_t n, double2* __restrict__ U)
 {
     typedef typename cvec<T>::type V;
     const int64_t idx = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (idx >= n * nvec) return;
     const int64_t i = idx / nvec;
     const int q = (int)(idx - i * nvec);
+    const int64_t p = i / b;
     V acc = czero<V>();
 #pragma unroll
-    for (int a = 0; a < R; ++a) cmac(acc, z1[i * R + a], Y[(int64_t)q * R + a]);
+    for (int a = 0; a < R; ++a) {
+        V t;
+        if (L == 0) {
+            t = Y[(int64_t)q * R + a];
+        } else {
+            const V x = Y[((2 * p) * nvec + q) * R + a], y = Y[((2 * p + 1) * nvec + q) * R + a];
+            t.x = x.x + y.x;
+            t.y = x.y + y.y;
+        }
+        cmac(acc, z1[i * R + a], t);
+    }
     U[idx] = to_d2(acc);
 }
+
+// Whether the mat-vec takes passes over several levels (k_mv_pass; always in
+// complex64) or goes level by level.  In FP64 the pipe counts a warp's
+// instructions whatever its lanes do, so the 16 vector lanes of a pass have to
+// be filled, and only ranks 5 .. 8 then gain.  us of kernels, levels / passes: n =
+// 65536, L = 12, r = 8 1 vector 366 / 1110, 16 1109 / 1074, 17 1122 / 1706, 64
+// 3600 / 3298; n = 4096, r = 8, 64 vectors 263 / 212, r = 4 121 / 135; n = 65536, r
+// = 12, 64 vectors 7404 / 8107.
+template <typename T, int R> struct MvRule {
+    static constexpr bool ANY = sizeof(T) == 4 || (R >= 5 && R <= 8);
+    static bool passes(int nvec) { return ANY && (sizeof(T) == 4 || 8 * nvec >= 7 * ((nvec + 15) / 16 * 16)); }
+};
 
 // --------------------------------------------------------------- drivers
 
@@ -785,47 +843,62 @@ template <typename T, int R> struct FirstOrder {
     static bfc_status matvec(Ctx* c, int nvec, const double2* Vd, double2* Ud, V* Y0, V* Y1)
     {
         const int L = c->L;
-        if (L == 0) {
+        const int64_t S = c->S;
+        if (L == 0 || !MvRule<T, R>::passes(nvec)) {
+            const int64_t npre = (int64_t)1 << L;
             {
                 ProfScope ps(c, "mv_leaf");
-                k_mv_leaf<T, R><<<nblocks(nvec, 256), 256, 0, c->stream>>>((const V*)c->zLt, Vd, c->b, nvec, 1, Y0);
+                k_mv_leaf<T, R><<<nblocks(npre * nvec, 256), 256, 0, c->stream>>>((const V*)c->zLt, Vd, c->b, nvec,
+                                                                                  (int)npre, Y0);
             }
+            V* yin = Y0;
+            V* yout = Y1;
+            if constexpr (sizeof(T) == 8)
+                for (int m = L; m >= 1; --m) {
+                    ProfScope ps(c, "mv_level");
+                    k_mv_level<T, R><<<nblocks(S * nvec, 256), 256, 0, c->stream>>>(
+                        (const V*)c->Zt + (size_t)(m - 1) * S * R * R, yin, yout, m, L, nvec, (int)S);
+                    std::swap(yin, yout);
+                }
             {
                 ProfScope ps(c, "mv_root");
-                k_mv_root<T, R><<<nblocks(c->n * nvec, 256), 256, 0, c->stream>>>((const V*)c->z1t, Y0, nvec, c->n, Ud);
+                k_mv_root<T, R><<<nblocks(c->n * nvec, 256), 256, 0, c->stream>>>((const V*)c->z1t, yin, c->b, L, nvec,
+                                                                                  c->n, Ud);
             }
             BFC_LAUNCH_CHECK(c, "matvec");
             return BFC_OK;
         }
-        typedef MvCfg<T, R> MC;
-        BFC_CK(c, cudaFuncSetAttribute(k_mv_pass<T, R>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)MC::SMEM));
-        // the last pass takes up to 3 levels, the first up to 4, the others the
-        // rest in even parts of at most 4
-        const int nlast = std::min(3, L - 1), nfirst = std::min(4, L - nlast);
-        int rest = L - nlast - nfirst, mids = (rest + 3) / 4;
-        V* yin = nullptr;
-        V* yout = Y0;
-        auto pass = [&](int M, int s, int lv, int first, int last) {
-            ProfScope ps(c, "mv_pass");
-            const MvPass mp{L, M, s, lv, first, last, c->b, nvec};
-            const unsigned groups = 1u << (L + 1 - s), per = (unsigned)(MC::E >> s);
-            const dim3 grid((groups + per - 1) / per, (unsigned)((nvec + MC::VT - 1) / MC::VT));
-            k_mv_pass<T, R><<<grid, 128, MC::SMEM, c->stream>>>(mp, (const V*)c->Zt, (const V*)c->zLt,
-                                                                (const V*)c->z1t, Vd, yin, yout, Ud);
-            V* t = yin == nullptr ? Y1 : yin;
-            yin = yout;
-            yout = t;
-        };
-        int M = L;
-        pass(M, nfirst, nfirst, 1, 0);
-        M -= nfirst;
-        for (; mids > 0; --mids) {
-            const int s = (rest + mids - 1) / mids;
-            pass(M, s, s, 0, 0);
-            M -= s;
-            rest -= s;
+        if constexpr (MvRule<T, R>::ANY) {
+            typedef MvCfg<T, R> MC;
+            BFC_CK(c, cudaFuncSetAttribute(k_mv_pass<T, R>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)MC::SMEM));
+            // the last pass takes up to 3 levels, the first up to 4, the others the
+            // rest in even parts of at most 4
+            const int nlast = std::min(3, L - 1), nfirst = std::min(4, L - nlast);
+            int rest = L - nlast - nfirst, mids = (rest + 3) / 4;
+            V* yin = nullptr;
+            V* yout = Y0;
+            auto pass = [&](int M, int s, int lv, int first, int last) {
+                ProfScope ps(c, "mv_pass");
+                const MvPass mp{L, M, s, lv, first, last, c->b, nvec};
+                const unsigned groups = 1u << (L + 1 - s), per = (unsigned)(MC::E >> s);
+                const dim3 grid((groups + per - 1) / per, (unsigned)((nvec + MC::VT - 1) / MC::VT));
+                k_mv_pass<T, R><<<grid, 128, MC::SMEM, c->stream>>>(mp, (const V*)c->Zt, (const V*)c->zLt,
+                                                                    (const V*)c->z1t, Vd, yin, yout, Ud);
+                V* t = yin == nullptr ? Y1 : yin;
+                yin = yout;
+                yout = t;
+            };
+            int M = L;
+            pass(M, nfirst, nfirst, 1, 0);
+            M -= nfirst;
+            for (; mids > 0; --mids) {
+                const int s = (rest + mids - 1) / mids;
+                pass(M, s, s, 0, 0);
+                M -= s;
+                rest -= s;
+            }
+            pass(M, nlast + 1, nlast, 0, 1);
         }
-        pass(M, nlast + 1, nlast, 0, 1);
         BFC_LAUNCH_CHECK(c, "matvec");
         return BFC_OK;
     }
