@@ -931,7 +931,8 @@ bfc_status bfc_eval(bfc_ctx* ctx, int64_t m, const int32_t* i, const int32_t* j,
     const bool host_check = !c->P.values_on_device && m <= 8192 && host_address(i) && host_address(j);
     int32_t both[16384];   // [i | j] of a small call: what is checked is what is copied, in one piece
     if (host_check) {
-        if (cudaStreamQuery(c->stream) != cudaSuccess) {
+        // (the context's own stream holds no work between calls)
+        if (c->stream != c->own_stream && cudaStreamQuery(c->stream) != cudaSuccess) {
             cudaGetLastError();   // (not ready)
             BFC_TRY(sync(c));
         }
