@@ -505,8 +505,10 @@ __device__ __forceinline__ void warp_sums_tiles(const float2* __restrict__ A, co
 // Items (FP64 always: the FP64 pipe counts instructions of a warp): lanes own
 // the R(R+1)/2 + R items.  TILES (complex64): lanes own 2 x 2 tiles of the lower
 // triangle and 2 x 1 tiles of y, EG rows at a time side by side; the EG shares
-// are added by error-free sums.  In complex64 per-chunk partials are folded into
-// Kahan-compensated sums.
+// are added by error-free sums.  In complex64 partial sums of FOLD rows (items)
+// or of a lane's share of a chunk (tiles, 32 / EG rows) are folded into
+// Kahan-compensated sums: with 32 rows for r = 4, items left the factors of a
+// sweep at n = 256 5.3e-7 from 64 bits, tiles 3.5e-7.
 template <typename T, int R, bool TILES, typename F>
 __device__ __forceinline__ void warp_sums(const typename cvec<T>::type* __restrict__ A,
                                           const typename cvec<T>::type* __restrict__ tv, int s0, int s1,
@@ -519,6 +521,8 @@ __device__ __forceinline__ void warp_sums(const typename cvec<T>::type* __restri
         return;
     }
     constexpr bool COMP = sizeof(T) == 4;
+    // rows per partial sum: no more than tiles add before theirs are folded
+    constexpr int FOLD = !COMP ? 32 : R <= 2 ? 2 : R <= 4 ? 4 : R <= 6 ? 8 : R <= 8 ? 16 : 32;
     constexpr int NP = R * (R + 1) / 2;
     constexpr int NI = NP + R;
     constexpr int IPL = (NI + 31) / 32;
@@ -558,22 +562,25 @@ __device__ __forceinline__ void warp_sums(const typename cvec<T>::type* __restri
             if (lane < cnt) t_s[lane] = tv[base + lane];
         }
         __syncwarp();
-        for (int e = 0; e < cnt; ++e) {
-            const V* ae = &a_s[e * R];
+        for (int e0 = 0; e0 < cnt; e0 += FOLD) {
+            const int e1 = min(e0 + FOLD, cnt);
+            for (int e = e0; e < e1; ++e) {
+                const V* ae = &a_s[e * R];
 #pragma unroll
-            for (int u = 0; u < IPL; ++u) {
-                if (ip[u] >= 0) {   // Gram item (iq >= 0) or right-hand side (iq == -2): one code path
-                    const V* bp = iq[u] >= 0 ? ae + iq[u] : &t_s[e];
-                    cmacc(acc[u], ae[ip[u]], *bp);
+                for (int u = 0; u < IPL; ++u) {
+                    if (ip[u] >= 0) {   // Gram item (iq >= 0) or right-hand side (iq == -2): one code path
+                        const V* bp = iq[u] >= 0 ? ae + iq[u] : &t_s[e];
+                        cmacc(acc[u], ae[ip[u]], *bp);
+                    }
                 }
             }
-        }
-        if constexpr (COMP) {
+            if constexpr (COMP) {
 #pragma unroll
-            for (int u = 0; u < IPL; ++u) {
-                kahan(sum[u].x, cmp[u].x, acc[u].x);
-                kahan(sum[u].y, cmp[u].y, acc[u].y);
-                acc[u] = czero<V>();
+                for (int u = 0; u < IPL; ++u) {
+                    kahan(sum[u].x, cmp[u].x, acc[u].x);
+                    kahan(sum[u].y, cmp[u].y, acc[u].y);
+                    acc[u] = czero<V>();
+                }
             }
         }
     }
@@ -588,12 +595,16 @@ __device__ __forceinline__ void warp_sums(const typename cvec<T>::type* __restri
 // item per lane reads two 8-byte values for each product (the shared-memory
 // return path, 128 bytes a cycle, is its bound); tiles read less, but spend up
 // to 2 us per thousand fibers on adding their shares.  us per launch, items /
-// tiles: r = 1, n = 32768, 20 rows 19 / 62, n = 4096, 300 rows 24 / 23; r = 4, n =
-// 4096, 90 rows 17 / 21, 150 rows 24 / 25, 300 rows 39 / 31; r = 8, n = 32768, 60
-// rows 82 / 85, 90 rows 112 / 103; r = 10, 40 rows 75 / 74; r = 12, n = 4096, 40
-// rows 18.5 / 19.8, 800 rows 184 / 143.
+// tiles: r = 1, n = 32768, 20 rows 35 / 62, 53 rows 74 / 68; r = 4, n = 32768, 20
+// rows 28 / 78, 80 rows 80 / 84; r = 6, n = 4096, 125 rows 23 / 25; r = 8, n =
+// 65536, 40 rows 112 / 148, 53 rows 137 / 150; r = 10, n = 32768, 20 rows 48 / 64, 53
+// rows 91 / 87; r = 12, 20 rows 55 / 64, n = 4096, 800 rows 184 / 143.  Up to 1024
+// fibers are resident at once and the adding hides: a third as many rows (n = 512,
+// r = 4, 80 rows 13.3 / 11.7, r = 8, 40 rows 13.1 / 10.6).
 template <int R> struct OuterTiles {
-    static constexpr int ROWS = R == 1 ? 300 : R <= 7 ? 160 : R == 8 ? 90 : R <= 10 ? 70 : 40;
+    static constexpr int ROWS = R <= 2 ? 45 : R <= 4 ? 90 : R <= 6 ? 140 : R == 7 ? 85 : R == 8 ? 55 : R == 9 ? 70 :
+                                R == 10 ? 40 : 28;
+    static bool use(int64_t entries, int64_t fibers) { return entries * (fibers <= 1024 ? 3 : 1) >= ROWS * fibers; }
 };
 
 // Outer fibers, stage 1: one warp per fiber accumulates K and y (r x r) over

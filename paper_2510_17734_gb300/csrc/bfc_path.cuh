@@ -107,7 +107,7 @@ template <typename T, int R> struct Path {
             ProfScope ps(c, COLS ? "outer_cols_gram" : "outer_rows_gram");
             auto gram = k_outer_gram<T, R, false>;
             if constexpr (sizeof(T) == 4)
-                if (c->N >= OuterTiles<R>::ROWS * n) gram = k_outer_gram<T, R, true>;
+                if (OuterTiles<R>::use(c->N, n)) gram = k_outer_gram<T, R, true>;
             gram<<<nblocks(n, 4), 128, 0, c->stream>>>(A, (const V*)c->tval[level], c->seg[level], (int)n, rec);
         }
         {

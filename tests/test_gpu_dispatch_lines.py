@@ -39,9 +39,9 @@ def check(n, L, b, r, count, prec, lam=1e-1, **kw):
 @pytest.mark.parametrize("side", [-1, 0])
 @pytest.mark.parametrize("r", range(1, 13))
 def test_outer_gram_forms(r, side):
-    rows = 300 if r == 1 else 160 if r <= 7 else 90 if r == 8 else 70 if r <= 10 else 40
-    n = 2 * rows
-    check(n, 0, n, r, rows * n + side, bfc.PREC_C64, lam=1e-6)
+    rows = (45, 45, 90, 90, 140, 140, 85, 55, 70, 40, 28, 28)[r - 1]
+    n = 6 * (rows // 2)                         # up to 1024 fibers: a third of the rows
+    check(n, 0, n, r, rows * n // 3 + side, bfc.PREC_C64)
 
 
 @pytest.mark.parametrize("L", [9, 10])      # 1024 and 2048 slices; 8 per SM lie between
