@@ -59,17 +59,18 @@ TC_FLOPS_PER_ENTRY = 2 * 3 * 128 * 144   # flop, one contraction position x M 12
 # metrics, mean of three launches of the first sweep: 3,774,874 entries, 8192
 # slices per level), valid for the kernel source with this sha256 prefix
 TC_GRAM_TRAFFIC = {"source": "paper_2510_17734_gb300/csrc/bfc_gram_tc.cuh", "sha": "ca3d3494f519d50b",
-                   "read_bytes": 513.94176e6, "write_bytes": 142.995456e6, "entries": 3774874, "slices": 8192}
+                   "read_bytes": 514.061568e6, "write_bytes": 142.968235e6, "entries": 3774874, "slices": 8192}
 
 
 # DRAM counters of k_mid_solve at the n = 65536 workload itself (ncu, one-pass
 # metrics, mean of three launches of the first sweep: 3,774,874 entries, 8192
-# slices per level), valid for the kernel source with this sha256 prefix
-SOLVE_TRAFFIC = {"source": "paper_2510_17734_gb300/csrc/bfc_solve.cuh", "sha": "60826c85247253b6",
+# slices per level), taken with the kernel source of this sha256 prefix: a change
+# of the source needs a capture of its own, not a new prefix
+SOLVE_TRAFFIC = {"source": "paper_2510_17734_gb300/csrc/bfc_solve.cuh", "sha": "b4b4ab89fc8c4ba3",
                  # the kernel and the device functions it calls (KPair ... k_mid_solve)
                  "span": ("// Arithmetic on pairs of neighbouring k of two rows",
                           "// FP64 fallback of the precision form: a CTA"),
-                 "read_bytes": 431.426987e6, "write_bytes": 212.522069e6, "entries": 3774874, "slices": 8192}
+                 "read_bytes": 429.718272e6, "write_bytes": 212.781653e6, "entries": 3774874, "slices": 8192}
 
 
 def kernel_source_sha(rel_path: str, span=None) -> str:
@@ -249,7 +250,7 @@ def kernel_rooflines(prob, prof, stats, peaks, fp32_meas):
         out.append({"kernel": "k_eval", "bound": "alu", "launch_ms": ms, "flop": fl,
                     "achieved": af, "peak": fp32_meas, "unit": "TFLOP/s", "frac": af / fp32_meas,
                     "per_unit": f"{8 * (L * D + 2 * r)} flop per test entry (L r x r complex products)",
-                    "note": "thread per test entry; the slices come from L2 (factors fit in it)"})
+                    "note": "8 lanes per test entry; the slices come from L2 (factors fit in it)"})
     keymap = {"k_env_right": "env_right", "k_mid_solve": "mid_solve", "k_outer_gram (rows)": "outer_rows_gram",
               "k_outer_gram (columns)": "outer_cols_gram", "k_outer_post (rows)": "outer_rows_post",
               "k_outer_post (columns)": "outer_cols_post", "k_eval": "eval"}
