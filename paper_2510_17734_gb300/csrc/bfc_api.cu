@@ -220,7 +220,7 @@ struct Inputs {
 //    per entry, for the compensated sums: n = 32768, r = 4, Radon data, error of
 //    the factors after a sweep 7.2e-7, and 8.5e-7 without those levels.  Slices of
 //    fewer than r rows (columns) group as well: with b = 1 .. 4 < r, four sweeps
-//    of ten problems each, all levels on the tensor cores / grouped leave 165 / 0
+//    of eight problems each, all levels on the tensor cores / grouped leave 165 / 0
 //    (r = 5), 1591 / 6 (r = 6), 7821 / 27 (r = 7) and 21027 / 335 (r = 8) singular
 //    systems;
 //  * next to the per-entry CUDA-core kernel, whose work per entry is that of a

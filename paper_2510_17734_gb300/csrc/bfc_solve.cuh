@@ -17,8 +17,8 @@
 //
 // Bound by latency: shared memory and registers hold 8 slices of rank 8 per SM
 // and the diagonal blocks and triangular solves are one warp's chains (ncu,
-// n = 32768, r = 8: 37 % issue slots, a third of the stalls at barriers, L1
-// line throughput 61 %).  Measured, all middle levels of a sweep, against the
+// n = 16384, r = 8: 36 % issue slots, 29 % of the stalls at barriers, L1
+// throughput 61 %).  Measured, all middle levels of a sweep, against the
 // kernel before (one warp per slice on a packed triangle, a lane per row):
 // n = 65536, r = 8 6.48 -> 5.74 ms; n = 4096, r = 12 8.8 -> 3.1 ms; n = 4096,
 // r = 6, FP64 3.75 -> 1.67 ms; n = 3072, r = 5 0.47 -> 0.38 ms.  One warp per
