@@ -4,6 +4,8 @@
 #include <string.h>
 
 #include <algorithm>
+#include <memory>
+#include <new>
 #include <string>
 #include <vector>
 
@@ -928,16 +930,19 @@ bfc_status bfc_eval(bfc_ctx* ctx, int64_t m, const int32_t* i, const int32_t* j,
     };
     const bool idx = in_place(c, i, ib, 4) && in_place(c, j, ib, 4);
     const bool direct = idx && in_place(c, out, ob, 16) && apart(i) && apart(j);
-    const bool host_check = !c->P.values_on_device && m <= 8192 && host_address(i) && host_address(j);
-    int32_t both[16384];   // [i | j] of a small call: what is checked is what is copied, in one piece
+    // [i | j] of a small call: what is checked is what is copied, in one piece
+    std::unique_ptr<int32_t[]> both;
+    if (!c->P.values_on_device && m <= 8192 && host_address(i) && host_address(j))
+        both.reset(new (std::nothrow) int32_t[2 * (size_t)m]);
+    const bool host_check = both != nullptr;
     if (host_check) {
         // (the context's own stream holds no work between calls)
         if (c->stream != c->own_stream && cudaStreamQuery(c->stream) != cudaSuccess) {
             cudaGetLastError();   // (not ready)
             BFC_TRY(sync(c));
         }
-        memcpy(both, i, ib);
-        memcpy(both + m, j, ib);
+        memcpy(both.get(), i, ib);
+        memcpy(both.get() + m, j, ib);
         for (int64_t e = 0; e < 2 * m; ++e)
             if (both[e] < 0 || both[e] >= c->n) return fail(c, BFC_EINVAL, "an index is outside [0, n)");
     }
@@ -950,7 +955,7 @@ bfc_status bfc_eval(bfc_ctx* ctx, int64_t m, const int32_t* i, const int32_t* j,
         di = d;
         dj = d + m;
         if (host_check) {
-            BFC_CK(c, cudaMemcpyAsync(d, both, 2 * ib, cudaMemcpyHostToDevice, c->stream));
+            BFC_CK(c, cudaMemcpyAsync(d, both.get(), 2 * ib, cudaMemcpyHostToDevice, c->stream));
         } else {
             BFC_CK(c, cudaMemcpyAsync(d, i, ib, in_kind(c), c->stream));
             BFC_CK(c, cudaMemcpyAsync(d + m, j, ib, in_kind(c), c->stream));
